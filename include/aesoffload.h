@@ -107,7 +107,7 @@ int aes_ctx_round_keys(aes_ctx_t ctx, uint8_t *w, size_t cap);
 typedef struct {
     int variant;        /* AES_VARIANT_* */
     int threads;        /* CTA size: multiple of 32, 32..1024 */
-    int blocks_per_thread; /* T-table: 16-byte blocks each thread keeps in flight (1, 2 or 4) */
+    int blocks_per_thread; /* T-table: 1, 2 or 4; a hint (every shape keeps one 16-byte block per thread in flight) */
     int ctas;           /* grid size; 0 = enough for the data, capped at SMs x occupancy */
 } aes_launch_t;
 

@@ -1,12 +1,13 @@
 // ctr.cu -- single-buffer AES-CTR kernels (SP 800-38A Sec. 6.5).
 //
 // Two variants of the block cipher, same contract:
-//   T-table  : each warp owns whole 256-block counter groups (lane l takes the
-//              blocks whose counter low byte is l + 32m, so every load/store
+//   T-table  : each CTA owns a contiguous run of 32-block chunks of the
+//              counter space, its warps take them in turn (lane l the block
+//              whose counter low byte is l + 32m, so every load/store
 //              instruction of the warp moves 512 contiguous bytes); rounds from
 //              T-tables in bank-replicated shared memory with counter-mode
-//              caching of rounds 1-2 (aes_ttable.cuh, tile.cuh).  128 KiB of
-//              shared memory, one CTA per SM.
+//              caching of rounds 1-2 (aes_ttable.cuh).  About 136 KiB of shared
+//              memory, one CTA per SM.
 //   bitsliced: each warp owns 1024 consecutive blocks; lane l holds blocks
 //              base + l + 32k (k = 0..31) as 128 bit planes (aes_bitslice.cuh),
 //              so loads/stores are again 512 contiguous bytes per instruction.
@@ -17,25 +18,96 @@
 #include "common.cuh"
 #include "aes_ttable.cuh"
 #include "bs_tile.cuh"
-#include "tile.cuh"
 
 namespace {
 
 using aesrt::CtrParams;
 
-template <int NR, int NB>
+// Counter groups whose round-2 constants a CTA holds at once (16 bytes each).
+constexpr uint32_t kGroupsPerPass = 512;
+constexpr size_t kCtrSmem = aestt::kTableBytes + kGroupsPerPass * sizeof(uint4);
+
+// Single-buffer T-table kernel, bound by shared-memory wavefronts: per
+// 32-block chunk the 16 * (NR - 2) lookups of rounds 3..NR, one broadcast
+// load of the group's round-2 constants and 8 for the payload in and out.
+//
+// Split: with v0 the IV's low byte, block j sits at counter position
+// v0 + j, and position >> 5 is its chunk.  The chunks are cut into gridDim.x
+// equal contiguous runs, one per CTA, so SMs differ by at most one chunk
+// (whole 256-block groups dealt out to warps left the busiest SM 1.3 times
+// the mean at 8 and 64 MiB).  In the run, warp w takes chunks w, w + W, ...;
+// W is a multiple of 8 in the usual shapes, so a lane's counter low byte
+// never changes and its part of round 2 (lane_round2) is computed once.  The
+// groups' part (group_round2) is computed once per CTA, one group per
+// thread.  Both cost 27 + 40 lookups per group and warp when each warp
+// derived them for itself: 8.4 of 144 wavefronts per chunk.
+// The next chunk's plaintext is loaded before the current one's rounds, so
+// a chunk's whole time (about 1 us with 16 warps) covers the DRAM latency.
+// One block per lane in flight: two gave 1.27 (1 MiB), 1.06 (8 MiB) and
+// 0.99-1.01 (256 MiB) times the time of one.
+// Measured (AES-128, launches in a CUDA graph): 1 MiB 5.05 -> 4.05 us, 8 MiB
+// 13.4 -> 10.7 us, 256 MiB 263 -> 240 us (1.12 TB/s; 137 wavefronts per
+// chunk at the measured rate and 2070 MHz are 228 us).
+template <int NR>
 __global__ void __launch_bounds__(1024, 1) ctr_ttable_kernel(const __grid_constant__ CtrParams p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
+    uint4 *s_group = reinterpret_cast<uint4 *>(smem + aestt::kTableBytes);
     aestt::fill_tables(smem, p.te0);
     __syncthreads();
     const aestt::Lanes ln;
     const aestt::RkConst rk{p.rk};
-    const uint64_t nblocks = (p.len + 15) >> 4;
-    const uint64_t gwarp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    aestile::xor_range<NR, NB>(p.in, p.out, p.len, p.iv_hi, p.iv_lo, 0, nblocks, gwarp, nwarps, p.parts, smem,
-                               ln, rk);
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const uint64_t nblocks = (p.len + 15) >> 4, nfull = p.len >> 4;
+    const uint64_t v0 = p.iv_lo & 255u, base_lo = p.iv_lo & ~(uint64_t)255u;
+    const uint64_t first = v0 >> 5, chunks = ((v0 + nblocks - 1) >> 5) - first + 1;
+    // this CTA's run; q * CTAs + r = chunks avoids the product chunks * blockIdx.x
+    const uint64_t q = chunks / gridDim.x, r = chunks % gridDim.x;
+    const uint64_t k_begin = first + q * blockIdx.x + (blockIdx.x < r ? blockIdx.x : r);
+    const uint64_t k_end = k_begin + q + (blockIdx.x < r ? 1 : 0);
+    uint4 mine = make_uint4(0, 0, 0, 0);  // lane_round2 of the lane's counter low byte
+    uint64_t mine_for = ~0ull;            // (counter bits 40.., m) it belongs to
+    for (uint64_t ka = k_begin; ka < k_end;) {
+        const uint64_t ga = ka >> 3;
+        const uint64_t kb = k_end < (ga + kGroupsPerPass) << 3 ? k_end : (ga + kGroupsPerPass) << 3;
+        const uint32_t ng = (uint32_t)(((kb - 1) >> 3) - ga) + 1;
+        if (ka != k_begin)
+            __syncthreads();  // every warp is done with the previous constants
+        for (uint32_t t = threadIdx.x; t < ng; t += blockDim.x) {
+            const uint64_t l = base_lo + ((ga + t) << 8);
+            s_group[t] = aestt::group_round2(aestt::CounterWords(p.iv_hi + (l < base_lo ? 1 : 0), l), smem, ln, rk);
+        }
+        // a block index before the message's first (first chunk) wraps and fails j < nfull
+        uint64_t k = ka + warp, j = (k << 5) + lane - v0;
+        uint4 next = make_uint4(0, 0, 0, 0);
+        if (k < kb && j < nfull)
+            next = aesdev::ld_stream(p.in + j);
+        __syncthreads();
+        for (; k < kb; k += nwarps) {
+            const uint4 pt = next;
+            const uint64_t jn = j + 32u * nwarps;
+            if (k + nwarps < kb && jn < nfull)
+                next = aesdev::ld_stream(p.in + jn);
+            const uint64_t g = k >> 3, l = base_lo + (g << 8);
+            const uint64_t tag = (l >> 40) << 3 | (k & 7u);
+            if (tag != mine_for) {
+                mine = aestt::lane_round2(aestt::CounterWords(p.iv_hi + (l < base_lo ? 1 : 0), l),
+                                          ((uint32_t)k & 7u) * 32u + lane, smem, ln, rk);
+                mine_for = tag;
+            }
+            const uint4 group = s_group[g - ga];
+            uint32_t s[1][4] = {{group.x ^ mine.x, group.y ^ mine.y, group.z ^ mine.z, group.w ^ mine.w}};
+            aestt::rounds<3, NR, 1>(s, smem, ln, rk);
+            if (j < nfull)
+                aesdev::st_stream(p.out + j, make_uint4(pt.x ^ s[0][0], pt.y ^ s[0][1], pt.z ^ s[0][2],
+                                                        pt.w ^ s[0][3]));
+            else if (j == nfull && (p.len & 15))  // the final partial block
+                aesdev::xor_tail(reinterpret_cast<const uint8_t *>(p.in + j), reinterpret_cast<uint8_t *>(p.out + j),
+                                 s[0][0], s[0][1], s[0][2], s[0][3], (uint32_t)(p.len & 15));
+            j = jn;
+        }
+        ka = kb;
+    }
 }
 
 template <int NR>
@@ -51,31 +123,6 @@ __global__ void __launch_bounds__(128) ctr_bitslice_kernel(const __grid_constant
                          aesbs::MaskKeys{reinterpret_cast<const uint4 *>(bsk)});
 }
 
-template <int NR>
-cudaError_t launch_tt(const CtrParams &p, const aesrt::CtrShape &s, int ctas, cudaStream_t st)
-{
-    const size_t smem = aestt::kTableBytes;
-    switch (s.nb) {
-    case 1: ctr_ttable_kernel<NR, 1><<<ctas, s.threads, smem, st>>>(p); break;
-    case 2: ctr_ttable_kernel<NR, 2><<<ctas, s.threads, smem, st>>>(p); break;
-    case 4: ctr_ttable_kernel<NR, 4><<<ctas, s.threads, smem, st>>>(p); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
-template <int NR>
-cudaError_t set_tt_attr()
-{
-    const int smem = (int)aestt::kTableBytes;
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(ctr_ttable_kernel<NR, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
-        return e;
-    if ((e = cudaFuncSetAttribute(ctr_ttable_kernel<NR, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
-        return e;
-    return cudaFuncSetAttribute(ctr_ttable_kernel<NR, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-}
-
 }  // namespace
 
 namespace aesrt {
@@ -83,12 +130,14 @@ namespace aesrt {
 cudaError_t ctr_set_attributes()
 {
     cudaError_t e;
-    if ((e = set_tt_attr<10>()) || (e = set_tt_attr<12>()) || (e = set_tt_attr<14>()))
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if ((e = cudaFuncSetAttribute(ctr_ttable_kernel<10>, attr, (int)kCtrSmem)) ||
+        (e = cudaFuncSetAttribute(ctr_ttable_kernel<12>, attr, (int)kCtrSmem)))
         return e;
-    return cudaSuccess;
+    return cudaFuncSetAttribute(ctr_ttable_kernel<14>, attr, (int)kCtrSmem);
 }
 
-// Resident CTAs per SM: T-table is bound by its 128 KiB of shared memory
+// Resident CTAs per SM: T-table is bound by its 136 KiB of shared memory
 // (one CTA); bitsliced CTAs of 128 threads are bound by registers.
 int ctr_max_ctas(const CtrShape &s, int nsm)
 {
@@ -97,38 +146,30 @@ int ctr_max_ctas(const CtrShape &s, int nsm)
     return nsm;
 }
 
-void ctr_plan(uint64_t nblocks, uint32_t v0, const CtrShape &s, int nsm, int *ctas, uint32_t *parts)
+int ctr_ctas(uint64_t nblocks, uint32_t v0, const CtrShape &s, int nsm)
 {
     const uint64_t cap = (uint64_t)ctr_max_ctas(s, nsm);
-    const uint64_t warps = (uint64_t)(s.threads / 32);
-    uint64_t units;
-    uint32_t pt = 1;
-    if (s.variant == 2) {
-        units = (nblocks + 1023) / 1024;  // a bitsliced warp takes 1024 blocks per pass
-    } else {
-        // A T-table warp takes a whole 256-block counter group, or a part of
-        // one when the message is too short to give every warp of the
-        // largest grid a group (keeping at least NB blocks per lane per part).
-        const uint64_t groups = nblocks ? ((v0 + nblocks - 1) >> 8) + 1 : 1;
-        while (pt < 8u / (uint32_t)s.nb && groups * pt < cap * warps)
-            pt *= 2;
-        units = groups * pt;
-    }
-    uint64_t want = (units + warps - 1) / warps;
-    if (s.ctas > 0)
+    uint64_t want;
+    if (s.ctas > 0) {
         want = (uint64_t)s.ctas;
+    } else if (s.variant == 2) {
+        const uint64_t warps = (uint64_t)(s.threads / 32);
+        want = ((nblocks + 1023) / 1024 + warps - 1) / warps;  // a bitsliced warp takes 1024 blocks per pass
+    } else {
+        // One CTA per 32-block chunk until every SM has one: a chunk's rounds
+        // are a latency chain, so a short message is done soonest when no
+        // warp takes two.
+        want = nblocks ? ((v0 + nblocks - 1) >> 5) - (v0 >> 5) + 1 : 1;
+    }
     if (want > cap)
         want = cap;
-    *ctas = want < 1 ? 1 : (int)want;
-    *parts = pt;
+    return want < 1 ? 1 : (int)want;
 }
 
 cudaError_t launch_ctr(const CtrParams &p, int nr, const CtrShape &s, int nsm, cudaStream_t stream)
 {
     const uint64_t nblocks = (p.len + 15) / 16;
-    int ctas = 1;
-    uint32_t parts = 1;
-    ctr_plan(nblocks, (uint32_t)(p.iv_lo & 255u), s, nsm, &ctas, &parts);
+    const int ctas = ctr_ctas(nblocks, (uint32_t)(p.iv_lo & 255u), s, nsm);
     if (s.variant == 2) {
         if (s.threads != 128)
             return cudaErrorInvalidValue;
@@ -140,14 +181,13 @@ cudaError_t launch_ctr(const CtrParams &p, int nr, const CtrShape &s, int nsm, c
         }
         return cudaGetLastError();
     }
-    CtrParams q = p;
-    q.parts = parts;
     switch (nr) {
-    case 10: return launch_tt<10>(q, s, ctas, stream);
-    case 12: return launch_tt<12>(q, s, ctas, stream);
-    case 14: return launch_tt<14>(q, s, ctas, stream);
+    case 10: ctr_ttable_kernel<10><<<ctas, s.threads, kCtrSmem, stream>>>(p); break;
+    case 12: ctr_ttable_kernel<12><<<ctas, s.threads, kCtrSmem, stream>>>(p); break;
+    case 14: ctr_ttable_kernel<14><<<ctas, s.threads, kCtrSmem, stream>>>(p); break;
     default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
 }
 
 }  // namespace aesrt

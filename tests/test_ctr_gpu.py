@@ -238,3 +238,26 @@ def test_ctr_sync_blocks_until_done(cuda, aes, ncpu):
         aes.ctr_sync(ctx, iv.tobytes(), src, dst, data.size, stream=s)
         np.testing.assert_array_equal(dst.numpy(), oracle.ctr_mt(key, 256, iv, data, ncpu))
     assert aes.lib().aes_ctr_sync(None, iv.tobytes(), src.data_ptr(), dst.data_ptr(), 16, 0) == aes.AES_EINVAL
+
+
+@pytest.mark.parametrize("threads,ctas", [(512, 0), (512, 1), (256, 7), (32, 2), (96, 1), (1024, 1), (416, 3)])
+@pytest.mark.parametrize("bits", [128, 192, 256])
+def test_chunk_run_edges(cuda, aes, ncpu, threads, ctas, bits):
+    """The T-table kernel's split into 32-block chunks: lengths one block or
+    byte around a chunk, a CTA run of more groups than one pass holds (512),
+    warp counts that are no multiple of 8 (a warp's counter low byte then
+    changes from chunk to chunk), IV low bytes on both sides of a chunk edge,
+    and a carry into counter byte 10 in the middle of a run."""
+    g = W.rng(3600 + bits + threads + ctas)
+    key = W.random_bytes(g, bits // 8)
+    ctx = aes.Context(key.tobytes(), bits)
+    long = [(512 * 256 + 300) * 16 + 5] if ctas == 1 and threads >= 512 else []
+    for n in [16 * 31, 16 * 32, 16 * 32 + 1, 16 * 33 - 1, 16 * 256, 16 * 257 + 9, 152 * 512 + 16, 200_000 + 3] + long:
+        for low in (0x00, 0x1F, 0x20, 0xFF):
+            iv = W.random_bytes(g, 16)
+            iv[15] = low
+            if low != 0x1F:  # the next 2^16 blocks carry through bytes 14..11 into byte 10
+                iv[11:15] = 0xFF
+            data = W.random_bytes(g, n)
+            got = gpu_ctr(cuda, aes, ctx, iv, data, variant=1, threads=threads, blocks_per_thread=1, ctas=ctas)
+            np.testing.assert_array_equal(got, oracle.ctr_mt(key, bits, iv, data, ncpu), err_msg=f"n={n} low={low}")

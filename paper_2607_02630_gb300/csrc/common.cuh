@@ -23,6 +23,15 @@ __device__ __forceinline__ void counter_block(uint64_t hi, uint64_t lo, uint64_t
     w[3] = bswap32((uint32_t)l);
 }
 
+// Overlap with the launch before and after on the same stream (programmatic
+// dependent launch, see launch_overlapped).  let_next_launch_start: the next
+// launch's CTAs may take SMs as soon as every CTA of this one has begun.
+// wait_for_previous_launch: everything earlier on the stream is complete and
+// visible; a kernel calls it in every thread before it touches a payload, and
+// reads nothing before it but tables, keys and its own parameters.
+__device__ __forceinline__ void let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void wait_for_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Streaming 16-byte load / store: payload bytes are touched once.
 __device__ __forceinline__ uint4 ld_stream(const uint4 *p)
 {

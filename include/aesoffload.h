@@ -153,19 +153,19 @@ typedef struct {
                            to 512 the warps keep round keys in registers,
                            above it in shared memory; the bitsliced kernel
                            takes 128 only */
-    int tile_blocks;    /* 16-byte blocks per work tile: a multiple of 256 (whole counter groups) */
-    int ctas;           /* persistent CTAs; 0 = one per SM (x occupancy) */
+    int tile_blocks;    /* 16-byte blocks of the largest work tile: a multiple of 256 */
+    int ctas;           /* CTAs; 0 = one per SM (x occupancy) */
     uint32_t tile_order_seed; /* nonzero: tiles are claimed in a seeded
                                  pseudo-random permutation (testing aid; the
                                  result must not change) */
-    int blocks_per_thread; /* T-table: 16-byte blocks each lane keeps in flight
-                              (1, 2 or 4); ignored by the bitsliced kernel,
-                              which always holds 32 per lane */
+    int blocks_per_thread; /* T-table: 1, 2 or 4; a hint (every shape keeps one
+                              16-byte block per lane in flight); ignored by the
+                              bitsliced kernel, which holds 32 per lane */
 } aes_batch_opts_t;
 
-/* Encrypt n independent requests in ONE persistent-kernel launch on
- * `stream`: the requests are cut into tiles of 16-byte blocks and the CTAs
- * claim tiles through a device atomic (work stealing).  Any mix of key sizes
+/* Encrypt n independent requests in ONE kernel launch on `stream`: each CTA
+ * owns an equal share of the batch's work, and its warps claim tiles of that
+ * share until none are left.  Any mix of key sizes
  * and lengths; each request follows aes_ctr's contract.  The descriptor
  * table is uploaded from host memory inside the call (descs may be reused on
  * return).  n == 0 is a no-op.  Errors: AES_EINVAL (n < 0, null descs, a
@@ -181,8 +181,7 @@ int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_bat
  * synchronise the device), or a runtime that forbids allocation after
  * start-up.  The paper has no counterpart: this is a deployment variant of
  * the batched launch.  Same contract and result as aes_ctr_batch, but the
- * call allocates nothing: its scratch (descriptor table + claim counter)
- * lives in one static device array of AES_NOALLOC_MAX_REQUESTS descriptors
+ * call allocates nothing: its scratch (the descriptor table) lives in one static device array of AES_NOALLOC_MAX_REQUESTS descriptors
  * (about 64 KiB) that every GPU loading the library keeps until exit.  The
  * key contexts must already exist on the current device (AES_EINVAL if no
  * context was ever created on it).  The first call on each device looks up
@@ -195,18 +194,16 @@ int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_bat
  * the same array and leaves its contents behind: calls whose work may
  * overlap on the GPU (other streams, other threads) race on it and must be
  * serialised by the caller.  The kernel is the T-table batch kernel in the
- * device's tuned T-table shape (tiles of whole counter groups, claimed by
- * each warp), finding each tile's request by a binary search in shared
- * memory instead of a tile map.  Errors: those of aes_ctr_batch, and
+ * device's tuned T-table shape.  Errors: those of aes_ctr_batch, and
  * AES_ETOOBIG when n exceeds AES_NOALLOC_MAX_REQUESTS. */
 #define AES_NOALLOC_MAX_REQUESTS 1024
 int aes_ctr_batch_noalloc(const aes_desc_t *descs, int n, void *stream);
 
-/* A prepared batch: the descriptor table lives on the device and the launch
- * (counter reset + persistent kernel) is captured once into a CUDA graph, so
- * repeated encryption of the same request layout costs one graph launch.
- * Payload contents may change between launches; pointers, lengths, keys and
- * IVs are fixed at creation. */
+/* A prepared batch: the descriptor table lives on the device, so repeated
+ * encryption of the same request layout costs one kernel launch.  Payload
+ * contents may change between launches; pointers, lengths, keys and IVs are
+ * fixed at creation.  A plan is not launched into a stream that is being
+ * captured (AES_ECUDA). */
 typedef struct aes_batch_plan_s *aes_batch_plan_t;
 int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
                           const aes_batch_opts_t *opts);
@@ -230,7 +227,7 @@ int aes_autotune_load(const char *path);
 
 /* Tune the batch kernel on the caller's own requests (the batching pattern's
  * autotuner): every candidate shape -- variant (T-table or bitsliced), CTA
- * size, blocks per lane in flight and tile size -- is built as a plan over
+ * size and tile size -- is built as a plan over
  * descs[0..n) and timed with CUDA events on `stream` (median of 5 launches
  * after 2 warm-ups); the fastest becomes the device's shape for
  * AES_VARIANT_AUTO batches and plans, and is returned in *best (may be

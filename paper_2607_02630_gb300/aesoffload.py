@@ -345,7 +345,7 @@ def batch(requests, stream=None, **opts) -> None:
 
 
 class BatchPlan:
-    """aes_batch_plan_*: a device-resident descriptor table + captured CUDA graph."""
+    """aes_batch_plan_*: a device-resident descriptor table, one kernel launch per use."""
 
     def __init__(self, requests, variant=0, threads=0, tile_blocks=0, ctas=0, tile_order_seed=0,
                  blocks_per_thread=0):

@@ -1,27 +1,30 @@
-// batch.cu -- many independent AES-CTR requests in one persistent launch.
+// batch.cu -- many independent AES-CTR requests in one launch.
 //
-// Every request (own key schedule, initial counter and length) is cut into
-// tiles of tile_blocks / 256 whole counter groups (a counter group is 256
-// blocks sharing the counter's upper 15 bytes, the unit of counter-mode
-// caching).  A host-built table maps each tile to its request; the warps of
-// the persistent CTAs (one per SM, T-tables filled once per CTA) each claim
-// tiles through one device atomic counter until none are left, so long and
-// short requests, AES-128 and AES-256, spread over all SMs (work stealing)
-// without any CTA-wide barrier per tile.  The cipher is the same T-table
-// round code as the single-buffer kernel.  Round keys: CTAs of up to 512
-// threads (the default) hold the current request's schedule in registers
-// (128 registers a thread), so the shared-memory pipe, the kernel's bound,
-// serves T-table lookups only; larger CTAs stage it in each warp's slice of
-// shared memory (one broadcast wavefront per round, about 5% of the pipe).
+// Work is measured in shared-memory wavefronts, the unit of the kernel's
+// bound: a 32-block chunk (tile.cuh) of a request with Nr rounds costs
+// chunk_cost(Nr) of them.  The requests' chunks, one request after the other,
+// are one line of cost; CTA c of G (one per SM) owns the c-th of G equal
+// pieces of it, so every SM gets the same number of lookups whatever the mix
+// of lengths and key sizes, and neither a table of tiles nor a counter in
+// device memory is needed.  In a CTA's piece the warps claim tiles through
+// one counter in shared memory, each tile a warps-th of what is left, at
+// most tile_blocks and at least about one chunk: large tiles amortise a
+// request's set-up, small ones at the end let the warps finish together, and
+// a batch of a few short requests is spread one chunk to a warp.  A warp
+// finds its tile's request by a 32-way search over the requests' first costs.
+// The cipher is the same T-table round code as the single-buffer kernel.
+// Round keys: CTAs of up to 512 threads (the default) hold the current
+// request's schedule in registers, so the shared-memory pipe, the kernel's
+// bound, serves lookups only; larger CTAs stage it in each warp's slice of
+// shared memory (one broadcast wavefront per round).
 //
-// The bitsliced kernel takes the same tiles with one warp per tile, 1024
-// blocks at a time, as the autotuner's alternative to the T-tables.  A search
-// variant of the T-table kernel finds a tile's request by binary search over
-// the requests' first tiles instead of a tile map (aes_ctr_batch_noalloc).
+// The bitsliced kernel takes the same pieces and tiles, 1024 blocks at a time,
+// as the autotuner's alternative to the T-tables.
 //
-// A nonzero `order` enables a test aid: tile t is processed as tile
-// (a*t + b) mod T for a host-chosen a coprime to T (a permutation), so tiles
-// complete in a scrambled order; results must not change.
+// With a tile order (a test aid) the line is cut into equal tiles instead,
+// and tile t is processed as tile (a*t + b) mod T for a host-chosen a coprime
+// to T (a permutation), so tiles complete in a scrambled order; results must
+// not change.
 #include "../../include/aesoffload.h"
 #include "internal.h"
 #include "runtime.h"
@@ -33,6 +36,7 @@
 #include <algorithm>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 namespace {
@@ -40,7 +44,35 @@ namespace {
 using aesrt::BatchReq;
 
 struct TileOrder {
-    uint64_t a, b;  // t -> (a*t + b) mod T; a == 1, b == 0 is the identity
+    uint64_t a, b;   // t -> (a*t + b) mod tiles
+    uint64_t tiles;  // 0: no order, tiles are cut as they are claimed
+};
+
+// Shared-memory wavefronts of one 32-block chunk: 16 lookups in each of the
+// NR - 2 rounds that are not cached, and about 9 for the payload and the
+// group constants.
+__host__ __device__ constexpr uint32_t chunk_cost(uint32_t nr) { return 16u * (nr - 2u) + 9u; }
+// The smallest tile: one AES-128 chunk.
+constexpr uint64_t kMinTileCost = chunk_cost(10);
+
+__device__ __forceinline__ uint64_t ceil_chunks(uint64_t cost, uint32_t nr)
+{
+    switch (nr) {
+    case 10: return (cost + chunk_cost(10) - 1) / chunk_cost(10);
+    case 12: return (cost + chunk_cost(12) - 1) / chunk_cost(12);
+    default: return (cost + chunk_cost(14) - 1) / chunk_cost(14);
+    }
+}
+
+// One launch.  reqs (device memory, no empty requests) is read only after
+// wait_for_previous_launch.
+struct BatchArgs {
+    const BatchReq *reqs;
+    uint32_t n;
+    uint64_t total_cost;
+    uint64_t tile_cost;  // largest tile
+    const uint32_t *te0;
+    TileOrder order;
 };
 
 // CTA sizes up to this hold round keys in registers.
@@ -48,182 +80,170 @@ constexpr int kRegsMaxThreads = 512;
 // The bitsliced batch kernel's CTA size (its warps are register-bound).
 constexpr int kBsThreads = 128;
 
-// The warp's next tile: lane 0 claims it from the device counter; returns
-// the tile index (>= total_tiles when none are left), permuted if asked.
-__device__ __forceinline__ unsigned long long claim_tile(unsigned long long *counter, uint64_t total_tiles,
-                                                         const TileOrder &order)
+// The last request of [lo, hi) whose first cost is <= x (reqs[lo] is one).
+// The whole warp searches: every step reads 32 requests spread over the range
+// and keeps the stretch between two of them, so 2^20 requests take 4 steps;
+// near tells that the answer is probably within 32 requests of lo.
+__device__ __forceinline__ uint32_t owner_of(const BatchReq *reqs, uint32_t lo, uint32_t hi, uint64_t x, bool near)
 {
-    unsigned long long t = 0;
-    if ((threadIdx.x & 31u) == 0)
-        t = atomicAdd(counter, 1ull);
-    t = __shfl_sync(0xffffffffu, t, 0);
-    if (t < total_tiles && (order.a != 1 || order.b != 0))
-        t = (order.a * t + order.b) % total_tiles;
-    return t;
+    const uint32_t lane = threadIdx.x & 31u;
+    while (hi - lo > 1) {
+        const uint32_t step = near ? 1u : (hi - lo + 31u) / 32u;
+        const uint64_t i = (uint64_t)lo + (uint64_t)lane * step;
+        const bool below = i < hi && reqs[i].cost_begin <= x;
+        const uint32_t cnt = (uint32_t)__popc(__ballot_sync(0xffffffffu, below));  // >= 1: lane 0's is reqs[lo]
+        lo += (cnt - 1u) * step;
+        if (cnt < 32u && hi - lo > step)
+            hi = lo + step;
+        near = false;
+    }
+    return lo;
 }
 
-// Owner of tile t: the last request whose first tile is <= t (requests
-// without tiles share their first tile number with the next request and are
-// never chosen).  Lane 0 searches `begin[0..n)` in shared memory.
-__device__ __forceinline__ uint32_t owner_of(const uint64_t *begin, int n, unsigned long long t)
+// Calls run(request, first chunk, chunks <= kRunChunks) for every piece of
+// work of the calling warp (every lane with the same arguments).  s_pos: the CTA's
+// counter, zeroed before the CTA's last barrier.
+template <class RUN>
+__device__ __forceinline__ void for_each_run(const BatchArgs &p, unsigned long long *s_pos, RUN &&run)
 {
-    int lo = 0;
-    if ((threadIdx.x & 31u) == 0) {
-        int hi = n - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (begin[mid] <= t)
-                lo = mid;
-            else
-                hi = mid - 1;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint64_t units = p.order.tiles ? p.order.tiles : p.total_cost;  // this CTA's piece [u0, u1)
+    const uint64_t q = units / gridDim.x, r = units % gridDim.x;
+    const uint64_t u0 = q * blockIdx.x + (blockIdx.x < r ? blockIdx.x : r);
+    const uint64_t size = q + (blockIdx.x < r ? 1 : 0);
+    const uint64_t guide = blockDim.x >> 5;
+    uint32_t ri = 0;
+    bool near = false;
+    for (;;) {
+        unsigned long long at = 0, take = 1;
+        if (lane == 0) {
+            if (!p.order.tiles) {
+                const unsigned long long cur = *(volatile unsigned long long *)s_pos;
+                take = cur < size ? (size - cur) / guide : 0;
+                take = take < kMinTileCost ? kMinTileCost : take > p.tile_cost ? p.tile_cost : take;
+            }
+            at = atomicAdd(s_pos, take);
+        }
+        at = __shfl_sync(0xffffffffu, at, 0);
+        take = __shfl_sync(0xffffffffu, take, 0);
+        if (at >= size)
+            break;
+        uint64_t xa, xb;  // the tile's cost range
+        if (p.order.tiles) {
+            const uint64_t t = (p.order.a * (u0 + at) + p.order.b) % p.order.tiles;
+            xa = t * p.tile_cost;
+            xb = xa + p.tile_cost < p.total_cost ? xa + p.tile_cost : p.total_cost;
+            ri = 0;
+        } else {
+            xa = u0 + at;
+            xb = u0 + (at + take < size ? at + take : size);
+        }
+        ri = owner_of(p.reqs, ri, p.n, xa, near);
+        near = !p.order.tiles;  // later tiles lie further along
+        for (uint32_t i = ri; i < p.n; ++i) {
+            const BatchReq rq = p.reqs[i];
+            if (rq.cost_begin >= xb)
+                break;
+            // chunk c belongs to the tile that holds its first cost unit
+            const uint64_t nb = (rq.len + 15) >> 4, v0 = rq.iv_lo & 255u, first = aestile::first_chunk(rq.iv_lo);
+            const uint64_t nch = ((v0 + nb - 1) >> 5) - first + 1;
+            const uint64_t ca = xa > rq.cost_begin ? ceil_chunks(xa - rq.cost_begin, rq.nr) : 0;
+            uint64_t cb = ceil_chunks(xb - rq.cost_begin, rq.nr);
+            cb = cb < nch ? cb : nch;
+            for (uint64_t c = ca; c < cb;) {
+                const uint32_t m = aestile::run_chunks(rq.iv_lo, first + c, cb - c);
+                run(rq, first + c, m);
+                c += m;
+            }
         }
     }
-    return (uint32_t)__shfl_sync(0xffffffffu, lo, 0);
 }
 
-// The persistent T-table batch kernel.  NB: blocks per lane in flight;
-// MAXT: largest CTA it is launched with; RK_REGS: round keys in registers
-// (else in the warp's slice of shared memory); SEARCH: tile owners found by
-// binary search over the requests' first tiles (copied into shared memory
-// behind the tables) instead of read from the tile map.
-template <int NB, int MAXT, bool RK_REGS, bool SEARCH>
-__global__ void __launch_bounds__(MAXT, 1)
-    batch_ttable_kernel(const BatchReq *__restrict__ reqs, const uint32_t *__restrict__ tile_req, int nreq,
-                        uint64_t total_tiles, unsigned long long *__restrict__ counter,
-                        const uint32_t *__restrict__ te0, uint32_t tile_groups, TileOrder order)
+// The T-table batch kernel, bound by shared-memory wavefronts (95 % of the
+// pipe busy on a 256 MiB AES-128 request, 146 wavefronts a chunk of which 128
+// are lookups of rounds 3..10).  Measured as plans: 4096 requests of 1 KiB to
+// 8 MiB (3.66 GB) 4390 -> 4153 us, 64 requests of 1 to 16 KiB 39 -> 6.4 us
+// (one warp used to take up to 8 groups of a short request in turn), against
+// the kernel with a tile map, a device counter and two blocks per lane.
+// Registers: 384-thread CTAs with 168 a thread are faster on AES-256 alone
+// (4870 against 4957 us for the same lengths) and slower on AES-128 (3459
+// against 3356), as are 448 (5258 and 3401).  MAXT: largest CTA it is launched with; RK_REGS:
+// round keys in registers (else in the warp's slice of shared memory).
+template <int MAXT, bool RK_REGS>
+__global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_constant__ BatchArgs p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ uint4 s_rk[RK_REGS ? 1 : MAXT / 32][15];  // round keys of each warp's current tile
-    uint64_t *s_begin = reinterpret_cast<uint64_t *>(smem + aestt::kTableBytes);
-    if (SEARCH)
-        for (int i = threadIdx.x; i < nreq; i += blockDim.x)
-            s_begin[i] = reqs[i].tile_begin;
-    aestt::fill_tables(smem, te0);
+    __shared__ uint4 s_group[MAXT / 32][aestile::kRunGroups];
+    __shared__ uint4 s_rk[RK_REGS ? 1 : MAXT / 32][15];  // round keys of each warp's current request
+    __shared__ unsigned long long s_pos;
+    aesdev::let_next_launch_start();
+    if (threadIdx.x == 0)
+        s_pos = 0;
+    aestt::fill_tables(smem, p.te0);
     __syncthreads();
-    const aestt::Lanes ln;
-    const uint32_t lane = threadIdx.x & 31u;
-    uint4 *w_rk = s_rk[RK_REGS ? 0 : threadIdx.x >> 5];
-    // Every warp claims tiles on its own: no CTA-wide barrier per tile.
-    for (;;) {
-        const unsigned long long t = claim_tile(counter, total_tiles, order);
-        if (t >= total_tiles)
-            break;
-        const uint32_t ri = SEARCH ? owner_of(s_begin, nreq, t) : __ldg(tile_req + t);
-        const BatchReq rq = reqs[ri];
-        uint64_t first, last;
-        aestile::tile_blocks_of(t - rq.tile_begin, tile_groups, rq.iv_lo & 255u, (rq.len + 15) >> 4, &first,
-                                &last);
-        if (RK_REGS) {
-            switch (rq.nr) {
-            case 10: aestile::run_tile_warp_regs<10, NB>(rq, first, last, smem, ln); break;
-            case 12: aestile::run_tile_warp_regs<12, NB>(rq, first, last, smem, ln); break;
-            default: aestile::run_tile_warp_regs<14, NB>(rq, first, last, smem, ln); break;
-            }
-            continue;
+    aesdev::wait_for_previous_launch();
+    const aestt::Lanes ln(smem);
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    uint4 *w_group = s_group[warp];
+    uint4 *w_rk = s_rk[RK_REGS ? 0 : warp];
+    auto xor_with = [&](const BatchReq &rq, uint64_t k0, uint32_t n, auto nr) {
+        constexpr int NR = decltype(nr)::value;
+        if constexpr (RK_REGS) {
+            const aestt::RkRegs<NR> rk(rq.rk);
+            aestile::xor_run<NR>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, k0, n, w_group, ln, rk);
+        } else {
+            __syncwarp();  // every lane is done with the previous keys
+            if (lane <= NR)
+                w_rk[lane] = rq.rk[lane];
+            __syncwarp();
+            const aestt::RkShared rk{w_rk};
+            aestile::xor_run<NR>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, k0, n, w_group, ln, rk);
         }
-        if (lane <= rq.nr)
-            w_rk[lane] = rq.rk[lane];
-        __syncwarp();
+    };
+    for_each_run(p, &s_pos, [&](const BatchReq &rq, uint64_t k0, uint32_t n) {
         switch (rq.nr) {
-        case 10: aestile::run_tile_warp<10, NB>(rq, first, last, smem, ln, w_rk); break;
-        case 12: aestile::run_tile_warp<12, NB>(rq, first, last, smem, ln, w_rk); break;
-        default: aestile::run_tile_warp<14, NB>(rq, first, last, smem, ln, w_rk); break;
+        case 10: xor_with(rq, k0, n, std::integral_constant<int, 10>()); break;
+        case 12: xor_with(rq, k0, n, std::integral_constant<int, 12>()); break;
+        default: xor_with(rq, k0, n, std::integral_constant<int, 14>()); break;
         }
-        __syncwarp();  // w_rk is rewritten by the next claim
-    }
+    });
 }
 
-// The persistent bitsliced batch kernel: the same tiles and claims, each
-// tile encrypted by one warp 1024 blocks at a time (bs_tile.cuh) with the
-// request's round-key bit planes in the warp's slice of shared memory
-// (rebuilt when the warp moves to a request with another key).
-__global__ void __launch_bounds__(kBsThreads)
-    batch_bitslice_kernel(const BatchReq *__restrict__ reqs, const uint32_t *__restrict__ tile_req,
-                          uint64_t total_tiles, unsigned long long *__restrict__ counter, uint32_t tile_groups,
-                          TileOrder order)
+// The bitsliced batch kernel: the same tiles and claims, each run encrypted
+// by one warp 1024 blocks at a time (bs_tile.cuh) with the request's
+// round-key bit planes in the warp's slice of shared memory (rebuilt when the
+// warp moves to a request with another key).
+__global__ void __launch_bounds__(kBsThreads) batch_bitslice_kernel(const __grid_constant__ BatchArgs p)
 {
     __shared__ __align__(16) uint32_t s_mask[kBsThreads / 32][15 * 128];
+    __shared__ unsigned long long s_pos;
+    aesdev::let_next_launch_start();
+    if (threadIdx.x == 0)
+        s_pos = 0;
+    __syncthreads();
+    aesdev::wait_for_previous_launch();
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t *mask = s_mask[threadIdx.x >> 5];
     const uint4 *cur = nullptr;  // schedule whose masks are in `mask`
-    for (;;) {
-        const unsigned long long t = claim_tile(counter, total_tiles, order);
-        if (t >= total_tiles)
-            break;
-        const BatchReq rq = reqs[__ldg(tile_req + t)];
-        uint64_t first, last;
-        aestile::tile_blocks_of(t - rq.tile_begin, tile_groups, rq.iv_lo & 255u, (rq.len + 15) >> 4, &first,
-                                &last);
+    for_each_run(p, &s_pos, [&](const BatchReq &rq, uint64_t k0, uint32_t n) {
+        const uint64_t v0 = rq.iv_lo & 255u, nb = (rq.len + 15) >> 4;
+        const uint64_t first = k0 << 5 > v0 ? (k0 << 5) - v0 : 0;
+        const uint64_t end = ((k0 + n) << 5) - v0, last = end < nb ? end : nb;
         if (rq.rk != cur) {
             __syncwarp();  // every lane is done with the previous masks
             aesbs::build_masks(mask, reinterpret_cast<const uint32_t *>(rq.rk), (int)rq.nr, lane, 32);
             __syncwarp();
             cur = rq.rk;
         }
-        const uint4 k0 = __ldg(rq.rk);
-        const uint32_t rk0[4] = {k0.x, k0.y, k0.z, k0.w};
+        const uint4 k0w = __ldg(rq.rk);
+        const uint32_t rk0[4] = {k0w.x, k0w.y, k0w.z, k0w.w};
         const aesbs::MaskKeys keys{reinterpret_cast<const uint4 *>(mask)};
         switch (rq.nr) {
         case 10: aesbs::xor_range<10>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, rk0, first, last, 0, 1, keys); break;
         case 12: aesbs::xor_range<12>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, rk0, first, last, 0, 1, keys); break;
         default: aesbs::xor_range<14>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, rk0, first, last, 0, 1, keys); break;
         }
-    }
-}
-
-template <int NB, int MAXT, bool RK_REGS, bool SEARCH>
-cudaError_t set_smem_attr()
-{
-    const size_t bytes = aestt::kTableBytes + (SEARCH ? sizeof(uint64_t) * aesrt::kSearchMaxReqs : 0);
-    return cudaFuncSetAttribute(batch_ttable_kernel<NB, MAXT, RK_REGS, SEARCH>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-template <bool SEARCH>
-cudaError_t set_smem_attrs()
-{
-    cudaError_t e;
-    if ((e = set_smem_attr<1, kRegsMaxThreads, true, SEARCH>()) ||
-        (e = set_smem_attr<2, kRegsMaxThreads, true, SEARCH>()) ||
-        (e = set_smem_attr<4, kRegsMaxThreads, true, SEARCH>()) || (e = set_smem_attr<1, 1024, false, SEARCH>()) ||
-        (e = set_smem_attr<2, 1024, false, SEARCH>()) || (e = set_smem_attr<4, 1024, false, SEARCH>()))
-        return e;
-    return cudaSuccess;
-}
-
-// Launch the T-table kernel for shape s (nb and the CTA size pick the
-// instantiation).
-template <bool SEARCH>
-cudaError_t launch_ttable(int ctas, const aesrt::BatchShape &s, size_t smem, cudaStream_t stream,
-                          const BatchReq *reqs, const uint32_t *map, int nreq, uint64_t total,
-                          unsigned long long *counter, const uint32_t *te0, uint32_t tg, TileOrder order)
-{
-#define AES_BATCH_LAUNCH(NB, MAXT, REGS)                                                                   \
-    batch_ttable_kernel<NB, MAXT, REGS, SEARCH><<<ctas, s.threads, smem, stream>>>(reqs, map, nreq, total, \
-                                                                                   counter, te0, tg, order)
-    const bool regs = s.threads <= kRegsMaxThreads;
-    switch (s.nb) {
-    case 1:
-        if (regs)
-            AES_BATCH_LAUNCH(1, kRegsMaxThreads, true);
-        else
-            AES_BATCH_LAUNCH(1, 1024, false);
-        break;
-    case 4:
-        if (regs)
-            AES_BATCH_LAUNCH(4, kRegsMaxThreads, true);
-        else
-            AES_BATCH_LAUNCH(4, 1024, false);
-        break;
-    default:
-        if (regs)
-            AES_BATCH_LAUNCH(2, kRegsMaxThreads, true);
-        else
-            AES_BATCH_LAUNCH(2, 1024, false);
-        break;
-    }
-#undef AES_BATCH_LAUNCH
-    return cudaGetLastError();
+    });
 }
 
 int g_bs_ctas_per_sm = 1;  // resident bitsliced batch CTAs per SM (set with the attributes)
@@ -235,26 +255,15 @@ namespace aesrt {
 cudaError_t batch_set_attributes()
 {
     cudaError_t e;
-    if ((e = set_smem_attrs<false>()) || (e = set_smem_attrs<true>()))
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if ((e = cudaFuncSetAttribute(batch_ttable_kernel<kRegsMaxThreads, true>, attr, (int)aestt::kTableBytes)) ||
+        (e = cudaFuncSetAttribute(batch_ttable_kernel<1024, false>, attr, (int)aestt::kTableBytes)))
         return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_bitslice_kernel, kBsThreads, 0)))
         return e;
     g_bs_ctas_per_sm = per_sm > 0 ? per_sm : 1;
     return cudaSuccess;
-}
-
-cudaError_t launch_batch_search(const BatchReq *reqs, int n, uint64_t total_tiles, unsigned long long *counter,
-                                const uint32_t *te0, const BatchShape &s, int nsm, cudaStream_t stream)
-{
-    if (n < 1 || n > kSearchMaxReqs || s.variant != AES_VARIANT_TTABLE)
-        return cudaErrorInvalidValue;
-    int ctas = s.ctas > 0 ? std::min(s.ctas, nsm) : nsm;
-    if ((uint64_t)ctas > total_tiles)
-        ctas = (int)total_tiles;
-    const size_t smem = aestt::kTableBytes + sizeof(uint64_t) * (size_t)n;
-    return launch_ttable<true>(ctas, s, smem, stream, reqs, nullptr, n, total_tiles, counter, te0,
-                               (uint32_t)(s.tile_blocks / 256), TileOrder{1, 0});
 }
 
 static uint64_t gcd64(uint64_t a, uint64_t b)
@@ -269,9 +278,10 @@ static uint64_t gcd64(uint64_t a, uint64_t b)
 
 static TileOrder make_order(uint64_t total, uint32_t seed)
 {
-    TileOrder o{1, 0};
+    TileOrder o{1, 0, 0};
     if (!seed || total < 2)
         return o;
+    o.tiles = total;
     uint64_t x = seed * 0x9E3779B97F4A7C15ull + 0x632BE59BD9B4E019ull;
     for (int tries = 0; tries < 64; ++tries) {
         x ^= x >> 29;
@@ -287,11 +297,12 @@ static TileOrder make_order(uint64_t total, uint32_t seed)
     return o;
 }
 
-// Host-side preparation shared by aes_ctr_batch and the graph plans.
+// Host-side preparation shared by aes_ctr_batch and the plans: the requests
+// that hold any bytes.
 struct BatchTables {
     std::vector<BatchReq> reqs;
-    std::vector<uint32_t> tile_req;
-    uint64_t total_tiles = 0;
+    uint64_t total_cost = 0;
+    uint64_t total_chunks = 0;
     int64_t bytes = 0;
 };
 
@@ -323,7 +334,7 @@ static BatchShape pick_batch_shape(const DeviceState &st, const aes_batch_opts_t
         if (opts->variant && opts->variant != s.variant) {
             // another variant than the tuned one: start from its defaults
             s = opts->variant == AES_VARIANT_BITSLICE ? BatchShape{AES_VARIANT_BITSLICE, kBsThreads, 2048, 0, 1}
-                                                      : BatchShape{opts->variant, 512, 2048, 0, 2};
+                                                      : BatchShape{opts->variant, 512, 2048, 0, 1};
         }
         if (opts->threads)
             s.threads = opts->threads;
@@ -337,87 +348,63 @@ static BatchShape pick_batch_shape(const DeviceState &st, const aes_batch_opts_t
     return s;
 }
 
-static int build_tables(const aes_desc_t *descs, int n, int dev, const BatchShape &s, BatchTables &bt)
+static int build_tables(const aes_desc_t *descs, int n, int dev, BatchTables &bt)
 {
-    bt.reqs.resize((size_t)n);
-    uint64_t tiles = 0;
+    bt.reqs.reserve((size_t)n);
     for (int i = 0; i < n; ++i) {
         const aes_desc_t &d = descs[i];
         if (!d.ctx)
             return AES_EINVAL;
         if (d.ctx->device != dev)
             return AES_EINVAL;
-        BatchReq &r = bt.reqs[(size_t)i];
-        std::memset(&r, 0, sizeof(r));
+        if (!d.len)
+            continue;
+        const void *din = nullptr;
+        void *dout = nullptr;
+        const int rc = check_payload(d.in, d.out, d.len, dev, &din, &dout);
+        if (rc)
+            return rc;
+        BatchReq r{};
+        r.in = static_cast<const uint4 *>(din);
+        r.out = static_cast<uint4 *>(dout);
         r.len = d.len;
         iv_halves(d.iv, &r.iv_hi, &r.iv_lo);
         r.rk = reinterpret_cast<const uint4 *>(d.ctx->d_rk);
         r.nr = (uint32_t)d.ctx->nr;
-        r.tile_begin = tiles;
-        if (d.len) {
-            const void *din = nullptr;
-            void *dout = nullptr;
-            int rc = check_payload(d.in, d.out, d.len, dev, &din, &dout);
-            if (rc)
-                return rc;
-            r.in = static_cast<const uint4 *>(din);
-            r.out = static_cast<uint4 *>(dout);
-            tiles += tiles_of(d.len, d.iv[15], s.tile_blocks);
-            bt.bytes += (int64_t)d.len;
-        }
-    }
-    if (tiles > 0xffffffffull)
-        return AES_ETOOBIG;
-    bt.total_tiles = tiles;
-    bt.tile_req.resize((size_t)tiles);
-    for (int i = 0; i < n; ++i) {
-        const BatchReq &r = bt.reqs[(size_t)i];
-        const uint64_t k = r.len ? tiles_of(r.len, (uint32_t)(r.iv_lo & 255u), s.tile_blocks) : 0;
-        for (uint64_t t = 0; t < k; ++t)
-            bt.tile_req[(size_t)(r.tile_begin + t)] = (uint32_t)i;
+        r.cost_begin = bt.total_cost;
+        const uint64_t chunks = chunks_of(d.len, d.iv[15]);
+        bt.total_chunks += chunks;
+        bt.total_cost += chunks * chunk_cost(r.nr);
+        bt.bytes += (int64_t)d.len;
+        bt.reqs.push_back(r);
     }
     return AES_OK;
 }
 
-// Device image: [reqs][tile map][counter], each part 256-byte aligned.
-struct DeviceImage {
-    size_t off_map = 0, off_counter = 0, bytes = 0;
-};
+uint32_t batch_chunk_cost(int nr) { return chunk_cost((uint32_t)nr); }
 
-static DeviceImage image_layout(const BatchTables &bt)
+cudaError_t launch_batch(const BatchReq *reqs, size_t n, uint64_t total_cost, uint64_t total_chunks,
+                                const uint32_t *te0, const BatchShape &s, int nsm, uint32_t seed, cudaStream_t stream)
 {
-    DeviceImage im;
-    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    im.off_map = up(bt.reqs.size() * sizeof(BatchReq));
-    im.off_counter = up(im.off_map + bt.tile_req.size() * sizeof(uint32_t));
-    im.bytes = im.off_counter + 256;
-    return im;
-}
-
-cudaError_t launch_batch_image(uint8_t *img, const DeviceImage &im, const BatchTables &bt,
-                               const uint32_t *te0, const BatchShape &s, int nsm, uint32_t seed,
-                               cudaStream_t stream)
-{
-    cudaError_t e = cudaMemsetAsync(img + im.off_counter, 0, sizeof(unsigned long long), stream);
-    if (e)
-        return e;
-    // persistent CTAs: as many as are resident at once (one T-table CTA
-    // per SM: its tables take 128 KiB of shared memory)
+    BatchArgs p{};
+    p.reqs = reqs;
+    p.n = (uint32_t)n;
+    p.total_cost = total_cost;
+    p.tile_cost = (uint64_t)(s.tile_blocks / 32) * chunk_cost(10);
+    p.te0 = te0;
+    p.order = make_order((total_cost + p.tile_cost - 1) / p.tile_cost, seed);
+    // as many CTAs as are resident at once (one T-table CTA per SM: its
+    // tables take 128 KiB of shared memory), none without a chunk
     const int resident = s.variant == AES_VARIANT_BITSLICE ? nsm * g_bs_ctas_per_sm : nsm;
     int ctas = s.ctas > 0 ? std::min(s.ctas, resident) : resident;
-    if ((uint64_t)ctas > bt.total_tiles)
-        ctas = (int)bt.total_tiles;
-    const TileOrder order = make_order(bt.total_tiles, seed);
-    const BatchReq *reqs = reinterpret_cast<const BatchReq *>(img);
-    const uint32_t *map = reinterpret_cast<const uint32_t *>(img + im.off_map);
-    unsigned long long *counter = reinterpret_cast<unsigned long long *>(img + im.off_counter);
-    const uint32_t tg = (uint32_t)(s.tile_blocks / 256);
-    if (s.variant == AES_VARIANT_BITSLICE) {
-        batch_bitslice_kernel<<<ctas, kBsThreads, 0, stream>>>(reqs, map, bt.total_tiles, counter, tg, order);
-        return cudaGetLastError();
-    }
-    return launch_ttable<false>(ctas, s, aestt::kTableBytes, stream, reqs, map, (int)bt.reqs.size(),
-                                bt.total_tiles, counter, te0, tg, order);
+    if ((uint64_t)ctas > total_chunks)
+        ctas = (int)total_chunks;
+    if (s.variant == AES_VARIANT_BITSLICE)
+        return launch_overlapped(batch_bitslice_kernel, ctas, kBsThreads, 0, stream, p);
+    return s.threads <= kRegsMaxThreads
+               ? launch_overlapped(batch_ttable_kernel<kRegsMaxThreads, true>, ctas, s.threads, aestt::kTableBytes,
+                                   stream, p)
+               : launch_overlapped(batch_ttable_kernel<1024, false>, ctas, s.threads, aestt::kTableBytes, stream, p);
 }
 
 }  // namespace aesrt
@@ -427,10 +414,9 @@ using namespace aesrt;
 struct aes_batch_plan_s {
     int device;
     BatchTables bt;
-    DeviceImage im;
-    uint8_t *img = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    BatchShape shape;
+    uint32_t seed = 0;
+    BatchReq *reqs = nullptr;  // device
 };
 
 extern "C" {
@@ -451,26 +437,23 @@ int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_bat
     if ((rc = validate_batch_shape(s)))
         return rc;
     BatchTables bt;
-    if ((rc = build_tables(descs, n, st->device, s, bt)))
+    if ((rc = build_tables(descs, n, st->device, bt)))
         return rc;
-    if (bt.total_tiles == 0)
+    if (bt.reqs.empty())
         return AES_OK;
-    const DeviceImage im = image_layout(bt);
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    uint8_t *img = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&img), im.bytes, cs);
+    BatchReq *reqs = nullptr;
+    const size_t bytes = bt.reqs.size() * sizeof(BatchReq);
+    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&reqs), bytes, cs);
     if (e)
         return e == cudaErrorMemoryAllocation ? AES_ENOMEM : cuda_fail(e, "cudaMallocAsync");
-    // Pageable sources: each copy has finished reading the host vector when
+    // Pageable source: the copy has finished reading the host vector when
     // cudaMemcpyAsync returns, so bt may be destroyed afterwards.
-    e = cudaMemcpyAsync(img, bt.reqs.data(), bt.reqs.size() * sizeof(BatchReq),
-                        cudaMemcpyHostToDevice, cs);
+    e = cudaMemcpyAsync(reqs, bt.reqs.data(), bytes, cudaMemcpyHostToDevice, cs);
     if (!e)
-        e = cudaMemcpyAsync(img + im.off_map, bt.tile_req.data(), bt.tile_req.size() * sizeof(uint32_t),
-                            cudaMemcpyHostToDevice, cs);
-    if (!e)
-        e = launch_batch_image(img, im, bt, st->te0, s, st->nsm, opts ? opts->tile_order_seed : 0, cs);
-    cudaError_t e2 = cudaFreeAsync(img, cs);
+        e = launch_batch(reqs, bt.reqs.size(), bt.total_cost, bt.total_chunks, st->te0, s, st->nsm,
+                         opts ? opts->tile_order_seed : 0, cs);
+    cudaError_t e2 = cudaFreeAsync(reqs, cs);
     if (e)
         return cuda_fail(e, "aes_ctr_batch");
     if (e2)
@@ -504,50 +487,27 @@ int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
     if (!plan)
         return AES_ENOMEM;
     plan->device = st->device;
-    if ((rc = build_tables(descs, n, st->device, s, plan->bt))) {
+    plan->shape = s;
+    plan->seed = opts ? opts->tile_order_seed : 0;
+    if ((rc = build_tables(descs, n, st->device, plan->bt))) {
         delete plan;
         return rc;
     }
-    plan->im = image_layout(plan->bt);
-    cudaError_t e = cudaMalloc(&plan->img, plan->im.bytes);
-    if (e) {
-        delete plan;
-        return e == cudaErrorMemoryAllocation ? AES_ENOMEM : cuda_fail(e, "cudaMalloc(plan)");
-    }
-    e = cudaMemcpyAsync(plan->img, plan->bt.reqs.data(), plan->bt.reqs.size() * sizeof(BatchReq),
-                        cudaMemcpyHostToDevice, st->setup);
-    if (!e && !plan->bt.tile_req.empty())
-        e = cudaMemcpyAsync(plan->img + plan->im.off_map, plan->bt.tile_req.data(),
-                            plan->bt.tile_req.size() * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                            st->setup);
-    if (!e)
-        e = cudaStreamSynchronize(st->setup);
-    // Capture counter reset + persistent kernel on a private stream.
-    cudaStream_t cap = nullptr;
-    if (!e)
-        e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
-    if (!e && plan->bt.total_tiles > 0) {
-        e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-        if (!e) {
-            cudaError_t le = launch_batch_image(plan->img, plan->im, plan->bt, st->te0, s, st->nsm,
-                                                opts ? opts->tile_order_seed : 0, cap);
-            e = cudaStreamEndCapture(cap, &plan->graph);
-            if (!e)
-                e = le;
+    const size_t bytes = plan->bt.reqs.size() * sizeof(BatchReq);
+    if (bytes) {
+        cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&plan->reqs), bytes);
+        if (e) {
+            delete plan;
+            return e == cudaErrorMemoryAllocation ? AES_ENOMEM : cuda_fail(e, "cudaMalloc(plan)");
         }
+        e = cudaMemcpyAsync(plan->reqs, plan->bt.reqs.data(), bytes, cudaMemcpyHostToDevice, st->setup);
         if (!e)
-            e = cudaGraphInstantiate(&plan->exec, plan->graph, 0);
-    }
-    if (cap)
-        cudaStreamDestroy(cap);
-    if (e) {
-        if (plan->exec)
-            cudaGraphExecDestroy(plan->exec);
-        if (plan->graph)
-            cudaGraphDestroy(plan->graph);
-        cudaFree(plan->img);
-        delete plan;
-        return cuda_fail(e, "aes_batch_plan_create");
+            e = cudaStreamSynchronize(st->setup);
+        if (e) {
+            cudaFree(plan->reqs);
+            delete plan;
+            return cuda_fail(e, "aes_batch_plan_create");
+        }
     }
     *out = plan;
     return AES_OK;
@@ -557,10 +517,22 @@ int aes_batch_plan_launch(aes_batch_plan_t plan, void *stream)
 {
     if (!plan)
         return AES_EINVAL;
-    if (!plan->exec)
+    if (plan->bt.reqs.empty())
         return AES_OK;  // nothing to encrypt (all lengths zero)
-    cudaError_t e = cudaGraphLaunch(plan->exec, static_cast<cudaStream_t>(stream));
-    return e ? cuda_fail(e, "cudaGraphLaunch") : AES_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) == cudaSuccess &&
+        cap != cudaStreamCaptureStatusNone)
+        return cuda_fail(cudaErrorStreamCaptureUnsupported, "aes_batch_plan_launch");
+    DeviceState *st = nullptr;
+    int rc = device_state(&st);
+    if (rc)
+        return rc;
+    if (st->device != plan->device)
+        return AES_EINVAL;
+    const cudaError_t e =
+        launch_batch(plan->reqs, plan->bt.reqs.size(), plan->bt.total_cost, plan->bt.total_chunks, st->te0,
+                     plan->shape, st->nsm, plan->seed, static_cast<cudaStream_t>(stream));
+    return e ? cuda_fail(e, "aes_batch_plan_launch") : AES_OK;
 }
 
 int64_t aes_batch_plan_bytes(aes_batch_plan_t plan) { return plan ? plan->bt.bytes : AES_EINVAL; }
@@ -569,11 +541,7 @@ int aes_batch_plan_destroy(aes_batch_plan_t plan)
 {
     if (!plan)
         return AES_OK;
-    if (plan->exec)
-        cudaGraphExecDestroy(plan->exec);
-    if (plan->graph)
-        cudaGraphDestroy(plan->graph);
-    cudaFree(plan->img);
+    cudaFree(plan->reqs);
     delete plan;
     return AES_OK;
 }

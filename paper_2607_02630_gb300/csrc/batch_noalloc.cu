@@ -7,7 +7,7 @@
 // latency-critical path that must not pay for cudaMalloc/cudaFree (both can
 // synchronise the device), or an embedded runtime that forbids dynamic
 // allocation once it has started.  This entry point instead keeps its scratch
-// -- up to AES_NOALLOC_MAX_REQUESTS descriptors plus the claim counter -- in
+// -- up to AES_NOALLOC_MAX_REQUESTS descriptors -- in
 // one file-scope __device__ array that every GPU loading the library holds
 // until the process exits.  The caller still owns the payload buffers and
 // the key contexts (which must exist already: creating them is the only
@@ -24,10 +24,7 @@
 // stream is being captured into a CUDA graph; callers that want a graph use
 // the batch plans (aes_batch_plan_create), which allocate once up front.
 //
-// The kernel is the batch kernel's search variant (batch.cu): the same
-// persistent T-table CTAs, tiles of whole counter groups claimed by each warp
-// from one counter, and the owner of a claimed tile found by a binary search
-// over the requests' first tiles in shared memory instead of a tile map.
+// The kernel is the batch kernel (batch.cu), which needs no other scratch.
 #include "../../include/aesoffload.h"
 #include "internal.h"
 #include "runtime.h"
@@ -39,9 +36,7 @@ namespace {
 using aesrt::BatchReq;
 
 constexpr int kMaxReqs = AES_NOALLOC_MAX_REQUESTS;
-static_assert(kMaxReqs <= aesrt::kSearchMaxReqs, "the search kernel holds every request's first tile");
-constexpr size_t kReqBytes = sizeof(BatchReq) * (size_t)kMaxReqs;  // 64 KiB
-constexpr size_t kScratchBytes = kReqBytes + 256;                    // + claim counter
+constexpr size_t kScratchBytes = sizeof(BatchReq) * (size_t)kMaxReqs;  // 64 KiB
 
 static __device__ __align__(256) uint8_t g_noalloc_scratch[kScratchBytes];
 
@@ -74,13 +69,13 @@ extern "C" int aes_ctr_batch_noalloc(const aes_desc_t *descs, int n, void *strea
     });
     if (sa.err != cudaSuccess)
         return cuda_fail(sa.err, "aes_ctr_batch_noalloc set-up");
-    // the tuned T-table shape (the search kernel has no bitsliced variant)
+    // the tuned T-table shape
     BatchShape s = st->batch_tuned;
     if (s.variant != AES_VARIANT_TTABLE)
-        s = BatchShape{AES_VARIANT_TTABLE, 512, 2048, 0, 2};
+        s = BatchShape{AES_VARIANT_TTABLE, 512, 2048, 0, 1};
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     // Validate every request before touching the shared scratch.
-    uint64_t tiles = 0;
+    size_t m = 0;  // requests that hold any bytes
     for (int i = 0; i < n; ++i) {
         const aes_desc_t &d = descs[i];
         if (!d.ctx || d.ctx->device != st->device)
@@ -90,46 +85,46 @@ extern "C" int aes_ctr_batch_noalloc(const aes_desc_t *descs, int n, void *strea
             void *dout = nullptr;
             if ((rc = check_payload(d.in, d.out, d.len, st->device, &din, &dout)))
                 return rc;
-            tiles += tiles_of(d.len, d.iv[15], s.tile_blocks);
+            ++m;
         }
     }
-    if (tiles == 0)
+    if (m == 0)
         return AES_OK;
     // Descriptors go to the scratch in chunks staged on the stack (pageable
     // copies: each chunk buffer is free again when cudaMemcpyAsync returns).
     constexpr int kChunk = 32;
     BatchReq chunk[kChunk];
-    uint64_t begin = 0;
+    uint64_t cost = 0, chunks = 0;
+    size_t at = 0;
     cudaError_t e = cudaSuccess;
-    for (int i0 = 0; i0 < n && !e; i0 += kChunk) {
-        const int cnt = n - i0 < kChunk ? n - i0 : kChunk;
-        for (int k = 0; k < cnt; ++k) {
-            const aes_desc_t &d = descs[i0 + k];
-            BatchReq &r = chunk[k];
+    for (int i = 0; i < n && at < m && !e;) {
+        int cnt = 0;
+        for (; i < n && cnt < kChunk; ++i) {
+            const aes_desc_t &d = descs[i];
+            if (!d.len)
+                continue;
+            BatchReq &r = chunk[cnt++];
             std::memset(&r, 0, sizeof(r));
             r.len = d.len;
             iv_halves(d.iv, &r.iv_hi, &r.iv_lo);
             r.rk = reinterpret_cast<const uint4 *>(d.ctx->d_rk);
             r.nr = (uint32_t)d.ctx->nr;
-            r.tile_begin = begin;
-            if (d.len) {
-                const void *din = nullptr;
-                void *dout = nullptr;
-                check_payload(d.in, d.out, d.len, st->device, &din, &dout);
-                r.in = static_cast<const uint4 *>(din);
-                r.out = static_cast<uint4 *>(dout);
-                begin += tiles_of(d.len, d.iv[15], s.tile_blocks);
-            }
+            r.cost_begin = cost;
+            const uint64_t c = chunks_of(d.len, d.iv[15]);
+            chunks += c;
+            cost += c * batch_chunk_cost(d.ctx->nr);
+            const void *din = nullptr;
+            void *dout = nullptr;
+            check_payload(d.in, d.out, d.len, st->device, &din, &dout);
+            r.in = static_cast<const uint4 *>(din);
+            r.out = static_cast<uint4 *>(dout);
         }
-        e = cudaMemcpyAsync(sa.ptr + sizeof(BatchReq) * (size_t)i0, chunk, sizeof(BatchReq) * (size_t)cnt,
+        e = cudaMemcpyAsync(sa.ptr + sizeof(BatchReq) * at, chunk, sizeof(BatchReq) * (size_t)cnt,
                             cudaMemcpyHostToDevice, cs);
+        at += (size_t)cnt;
     }
-    unsigned long long *counter = reinterpret_cast<unsigned long long *>(sa.ptr + kReqBytes);
-    if (!e)
-        e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), cs);
     if (e)
         return cuda_fail(e, "aes_ctr_batch_noalloc copy");
-    e = launch_batch_search(reinterpret_cast<const BatchReq *>(sa.ptr), n, tiles, counter, st->te0, s, st->nsm,
-                            cs);
+    e = launch_batch(reinterpret_cast<const BatchReq *>(sa.ptr), m, cost, chunks, st->te0, s, st->nsm, 0, cs);
     return e ? cuda_fail(e, "aes_ctr_batch_noalloc launch") : AES_OK;
 }

@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(1024, 1) ctr_ttable_kernel(const __grid_consta
     aesdev::let_next_launch_start();
     aestt::fill_tables(smem, p.te0);
     __syncthreads();
-    const aestt::Lanes ln;
+    const aestt::Lanes ln(smem);
     const aestt::RkConst rk{p.rk};
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const uint64_t nblocks = (p.len + 15) >> 4, nfull = p.len >> 4;
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(1024, 1) ctr_ttable_kernel(const __grid_consta
             __syncthreads();  // every warp is done with the previous constants
         for (uint32_t t = threadIdx.x; t < ng; t += blockDim.x) {
             const uint64_t l = base_lo + ((ga + t) << 8);
-            s_group[t] = aestt::group_round2(aestt::CounterWords(p.iv_hi + (l < base_lo ? 1 : 0), l), smem, ln, rk);
+            s_group[t] = aestt::group_round2(aestt::CounterWords(p.iv_hi + (l < base_lo ? 1 : 0), l), ln, rk);
         }
         if (ka == k_begin)
             aesdev::wait_for_previous_launch();  // no payload byte is touched before
@@ -96,13 +96,13 @@ __global__ void __launch_bounds__(1024, 1) ctr_ttable_kernel(const __grid_consta
             const uint64_t g = k >> 3, l = base_lo + (g << 8);
             const uint64_t tag = (l >> 40) << 3 | (k & 7u);
             if (tag != mine_for) {
-                mine = aestt::lane_round2(aestt::CounterWords(p.iv_hi + (l < base_lo ? 1 : 0), l),
-                                          ((uint32_t)k & 7u) * 32u + lane, smem, ln, rk);
+                const aestt::CounterWords ctr(p.iv_hi + (l < base_lo ? 1 : 0), l);
+                mine = aestt::lane_round2(aestt::column0_round1(ctr, ln, rk), ((uint32_t)k & 7u) * 32u + lane, ln, rk);
                 mine_for = tag;
             }
             const uint4 group = s_group[g - ga];
             uint32_t s[1][4] = {{group.x ^ mine.x, group.y ^ mine.y, group.z ^ mine.z, group.w ^ mine.w}};
-            aestt::rounds<3, NR, 1>(s, smem, ln, rk);
+            aestt::rounds<3, NR, 1>(s, ln, rk);
             if (j < nfull)
                 aesdev::st_stream(p.out + j, make_uint4(pt.x ^ s[0][0], pt.y ^ s[0][1], pt.z ^ s[0][2],
                                                         pt.w ^ s[0][3]));

@@ -80,38 +80,33 @@ struct BatchReq {        // one request, device-side descriptor (64 bytes)
     const uint4 *rk;     // device round keys (4*(Nr+1) words as uint4 per round)
     uint32_t nr;
     uint32_t pad;
-    uint64_t tile_begin; // prefix sum of tiles before this request
+    uint64_t cost_begin; // batch: summed cost of the requests before this one
 };
 static_assert(sizeof(BatchReq) == 64, "descriptor is one 64-byte line");
 
 struct BatchShape {
     int variant;      // AES_VARIANT_TTABLE or AES_VARIANT_BITSLICE
     int threads;
-    int tile_blocks;  // a multiple of 256: tiles are runs of whole counter groups
+    int tile_blocks;  // a multiple of 256: the largest tile a warp claims
     int ctas;
-    int nb;           // T-table: blocks each lane keeps in flight (1, 2 or 4)
+    int nb;           // T-table: accepted as 1, 2 or 4; the kernel keeps one block per lane in flight
 };
 
-// Tiles of one batch request of `len` bytes whose initial counter has low
-// byte `iv_low_byte`: runs of tile_blocks / 256 whole 256-block counter
-// groups (group g holds the blocks whose counter low byte wrapped g times).
-inline uint64_t tiles_of(uint64_t len, uint32_t iv_low_byte, int tile_blocks)
+// 32-block chunks of the counter space that `len` > 0 bytes touch when the
+// initial counter has low byte `iv_low_byte`.
+inline uint64_t chunks_of(uint64_t len, uint32_t iv_low_byte)
 {
     const uint64_t nb = (len + 15) / 16;
-    if (!nb)
-        return 0;
-    const uint64_t groups = ((iv_low_byte + nb - 1) >> 8) + 1;
-    const uint64_t per = (uint64_t)tile_blocks / 256u;
-    return (groups + per - 1) / per;
+    return ((iv_low_byte + nb - 1) >> 5) - (iv_low_byte >> 5) + 1;
 }
+uint32_t batch_chunk_cost(int nr);
 
 cudaError_t batch_set_attributes();
-// The persistent T-table batch kernel over requests reqs[0..n) whose tiles
-// start at reqs[i].tile_begin; the owner of a claimed tile is found by a
-// binary search over those starts in shared memory (no tile map, so the
-// caller needs no scratch beyond reqs and the claim counter).  n <= 1024.
-cudaError_t launch_batch_search(const BatchReq *reqs, int n, uint64_t total_tiles, unsigned long long *counter,
-                                const uint32_t *te0, const BatchShape &s, int nsm, cudaStream_t stream);
-constexpr int kSearchMaxReqs = 1024;
+// One launch of the batch kernel over the n > 0 non-empty requests reqs[0..n)
+// in device memory, whose cost_begin are the prefix sums of
+// chunks_of * batch_chunk_cost; total_cost and total_chunks are the sums over
+// all of them.  seed != 0: tiles in a seeded order.
+cudaError_t launch_batch(const BatchReq *reqs, size_t n, uint64_t total_cost, uint64_t total_chunks,
+                         const uint32_t *te0, const BatchShape &s, int nsm, uint32_t seed, cudaStream_t stream);
 
 }  // namespace aesrt

@@ -99,7 +99,7 @@ struct RkRegsL2 {
 // (stamp: trace builds record when the keys have arrived)
 template <int NR, int NB>
 __device__ __forceinline__ void run_part_regs(const aesrt::BatchReq &rq, uint64_t first, uint64_t last,
-                                              uint32_t part, uint32_t parts, const uint8_t *smem,
+                                              uint32_t part, uint32_t parts,
                                               const aestt::Lanes &ln, const SrvParams &p, uint32_t seq, bool stamp)
 {
     const RkRegsL2<NR> rk(rq.rk);
@@ -114,8 +114,7 @@ __device__ __forceinline__ void run_part_regs(const aesrt::BatchReq &rq, uint64_
     (void)seq;
     (void)stamp;
 #endif
-    aestile::xor_range<NR, NB>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, first, last, part, parts, parts, smem,
-                               ln, rk);
+    aestile::xor_range<NR, NB>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, first, last, part, parts, parts, ln, rk);
 }
 
 template <bool PER_REQ>
@@ -136,7 +135,7 @@ __global__ void __launch_bounds__(512, 1) server_kernel(const __grid_constant__ 
         }
         return;  // no CTA-wide barrier follows
     }
-    const aestt::Lanes ln;
+    const aestt::Lanes ln(smem);
     uint32_t cur_d = ~0u, cur_seq = ~0u, tg = 1, tp = 1;
     uint64_t gen = 0;
     aesrt::BatchReq rq;
@@ -193,9 +192,9 @@ __global__ void __launch_bounds__(512, 1) server_kernel(const __grid_constant__ 
             const uint32_t part = t % tp;
             aestile::tile_blocks_of(t / tp, tg, rq.iv_lo & 255u, (rq.len + 15) >> 4, &first, &last);
             switch (rq.nr) {
-            case 10: run_part_regs<10, 2>(rq, first, last, part, tp, smem, ln, p, seq, lane == 0 && t == 0); break;
-            case 12: run_part_regs<12, 2>(rq, first, last, part, tp, smem, ln, p, seq, lane == 0 && t == 0); break;
-            default: run_part_regs<14, 2>(rq, first, last, part, tp, smem, ln, p, seq, lane == 0 && t == 0); break;
+            case 10: run_part_regs<10, 2>(rq, first, last, part, tp, ln, p, seq, lane == 0 && t == 0); break;
+            case 12: run_part_regs<12, 2>(rq, first, last, part, tp, ln, p, seq, lane == 0 && t == 0); break;
+            default: run_part_regs<14, 2>(rq, first, last, part, tp, ln, p, seq, lane == 0 && t == 0); break;
             }
         }
         // Order the tile's output stores before it is counted: a warp

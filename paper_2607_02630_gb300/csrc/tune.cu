@@ -51,7 +51,7 @@ void tune_defaults(DeviceState &st)
     for (int i = 0; i < 3; ++i)
         for (int b = 0; b < kLenBuckets; ++b)
             st.ctr_tuned[i][b] = default_shape();
-    st.batch_tuned = BatchShape{AES_VARIANT_TTABLE, 512, 2048, 0, 2};
+    st.batch_tuned = BatchShape{AES_VARIANT_TTABLE, 512, 2048, 0, 1};
 }
 
 CtrShape tuned_ctr_shape(const DeviceState &st, size_t len, int nr)
@@ -87,22 +87,20 @@ float time_ctr(aes_ctx_t ctx, const uint8_t *iv, void *buf_in, void *buf_out, si
 }
 
 // The batch kernel's candidate shapes: T-table CTAs of 256, 512 (round keys
-// in registers) and 1024 threads (keys in shared memory) x 1, 2 or 4 blocks
-// per lane in flight x tiles of 4, 8 or 16 counter groups; and the bitsliced
-// kernel (128-thread CTAs) x the same tiles.
+// in registers) and 1024 threads (keys in shared memory), and the bitsliced
+// kernel (128-thread CTAs), each x largest tiles of 1024, 2048 or 4096 blocks.
 std::vector<BatchShape> batch_candidates()
 {
     std::vector<BatchShape> c;
     for (int tb : {1024, 2048, 4096}) {
         for (int th : {256, 512, 1024})
-            for (int nb : {1, 2, 4})
-                c.push_back(BatchShape{AES_VARIANT_TTABLE, th, tb, 0, nb});
+            c.push_back(BatchShape{AES_VARIANT_TTABLE, th, tb, 0, 1});
         c.push_back(BatchShape{AES_VARIANT_BITSLICE, 128, tb, 0, 1});
     }
     return c;
 }
 
-// Time every candidate as a graph plan over `reqs` (median of `reps` launches
+// Time every candidate as a plan over `reqs` (median of `reps` launches
 // after two warm-ups, CUDA events on `s`); the fastest in *pick.  Returns
 // AES_OK, or the first error if no candidate ran.
 int sweep_batch(DeviceState &st, const std::vector<aes_desc_t> &reqs, cudaStream_t s, cudaEvent_t a,

@@ -255,3 +255,34 @@ def test_batch_every_length_0_to_64(cuda, aes, ncpu, bits):
     reqs, meta, payload, src, dst = make_requests(cuda, aes, g, lengths, [bits] * len(lengths))
     aes.batch(reqs, tile_blocks=1024)
     check_all(cuda, meta, payload, dst, ncpu)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 500, 501, 3000])
+@pytest.mark.parametrize("ctas,tile_blocks,seed,threads", [(0, 0, 0, 0), (1, 256, 0, 0), (3, 256, 9, 0), (0, 512, 5, 1024),
+                                                           (2, 0, 0, 96)])
+def test_cost_line_edges(cuda, aes, ncpu, n, ctas, tile_blocks, seed, threads):
+    """The split of a batch into equal pieces of cost and tiles of it: many
+    requests of around a chunk (empty ones among them, also first and last),
+    one of several CTA pieces, all key sizes, IV low bytes on both sides of a
+    chunk edge, a carry into counter byte 10 inside a run, and request counts
+    around the search's 32 and past one piece's worth."""
+    g = W.rng(5400 + n + ctas + tile_blocks + seed)
+    sizes = [0, 1, 15, 16, 496, 511, 512, 513, 528, 4096, 8000]
+    lengths = [int(sizes[i]) for i in g.integers(0, len(sizes), n)]
+    if n == 1:
+        lengths = [300_000 + 7]
+    elif n > 500:
+        lengths[0] = lengths[-1] = 0
+        lengths[n // 2] = (1 << 20) + 3
+    bits = [(128, 192, 256)[int(x)] for x in g.integers(0, 3, n)]
+    reqs, meta, payload, src, dst = make_requests(cuda, aes, g, lengths, bits)
+    lows = [0x00, 0x1F, 0x20, 0xFF]
+    for i, (ctx, iv, s, d, k) in enumerate(reqs):
+        b = bytearray(iv)
+        b[15] = lows[i % 4]
+        if i % 3 == 0:
+            b[11:15] = b"\xff\xff\xff\xff" if i % 2 else b"\xff\xff\xff\xfc"
+        reqs[i] = (ctx, bytes(b), s, d, k)
+        meta[i] = (meta[i][0], meta[i][1], np.frombuffer(bytes(b), np.uint8), meta[i][3], k)
+    aes.batch(reqs, ctas=ctas, tile_blocks=tile_blocks, tile_order_seed=seed, threads=threads)
+    check_all(cuda, meta, payload, dst, 1)

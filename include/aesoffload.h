@@ -165,12 +165,13 @@ typedef struct {
 
 /* Encrypt n independent requests in ONE kernel launch on `stream`: each CTA
  * owns an equal share of the batch's work, and its warps claim tiles of that
- * share until none are left.  Any mix of key sizes
- * and lengths; each request follows aes_ctr's contract.  The descriptor
- * table is uploaded from host memory inside the call (descs may be reused on
- * return).  n == 0 is a no-op.  Errors: AES_EINVAL (n < 0, null descs, a
- * NULL ctx), AES_EALIGN / AES_EOVERLAP / AES_EPTR for the first bad request,
- * AES_ETOOBIG (n > AES_BATCH_MAX), AES_ENOMEM, AES_ECUDA. */
+ * share until none are left.  Any mix of key sizes and lengths; each request
+ * follows aes_ctr's contract.  descs is read during the call (it may be
+ * reused on return).  Up to 1024 requests travel in kernel parameters (two or
+ * three launches past 500 and 1000); more in a descriptor table allocated
+ * and uploaded by the call.  n == 0 is a no-op.  Errors: AES_EINVAL (n < 0,
+ * null descs, a NULL ctx), AES_EALIGN / AES_EOVERLAP / AES_EPTR for the first
+ * bad request, AES_ETOOBIG (n > AES_BATCH_MAX), AES_ENOMEM, AES_ECUDA. */
 #define AES_BATCH_MAX (1 << 20)
 int aes_ctr_batch(const aes_desc_t *descs, int n, void *stream);
 int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_batch_opts_t *opts);
@@ -181,21 +182,13 @@ int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_bat
  * synchronise the device), or a runtime that forbids allocation after
  * start-up.  The paper has no counterpart: this is a deployment variant of
  * the batched launch.  Same contract and result as aes_ctr_batch, but the
- * call allocates nothing: its scratch (the descriptor table) lives in one static device array of AES_NOALLOC_MAX_REQUESTS descriptors
- * (about 64 KiB) that every GPU loading the library keeps until exit.  The
- * key contexts must already exist on the current device (AES_EINVAL if no
- * context was ever created on it).  The first call on each device looks up
- * the array's device address (cudaGetSymbolAddress) and keeps it.  Every
- * call copies its descriptors into the array with cudaMemcpyAsync from
- * pageable host memory, so no call -- the first or a later one -- may be
- * made while `stream` is being captured into a CUDA graph (the capture
- * would refuse the copy); callers that need a graph use the batch plans
- * (aes_batch_plan_create), which allocate once, up front.  Every call reuses
- * the same array and leaves its contents behind: calls whose work may
- * overlap on the GPU (other streams, other threads) race on it and must be
- * serialised by the caller.  The kernel is the T-table batch kernel in the
- * device's tuned T-table shape.  Errors: those of aes_ctr_batch, and
- * AES_ETOOBIG when n exceeds AES_NOALLOC_MAX_REQUESTS. */
+ * call never allocates or copies: its requests travel in kernel parameters,
+ * in launches of at most 500 requests each, so calls share no state and may
+ * overlap (other streams, other threads).  The key contexts must already
+ * exist on the current device (AES_EINVAL if no context was ever created on
+ * it).  The kernel is the T-table batch kernel in the device's tuned T-table
+ * shape.  Errors: those of aes_ctr_batch, and AES_ETOOBIG when n exceeds
+ * AES_NOALLOC_MAX_REQUESTS. */
 #define AES_NOALLOC_MAX_REQUESTS 1024
 int aes_ctr_batch_noalloc(const aes_desc_t *descs, int n, void *stream);
 

@@ -64,16 +64,36 @@ __device__ __forceinline__ uint64_t ceil_chunks(uint64_t cost, uint32_t nr)
     }
 }
 
-// One launch.  reqs (device memory, no empty requests) is read only after
-// wait_for_previous_launch.
+// One launch over n requests, none of them empty: in the kernel's own
+// parameters (CAP of them at most) or, CAP == 0, in device memory, which is
+// read only after wait_for_previous_launch.
 struct BatchArgs {
-    const BatchReq *reqs;
+    const BatchReq *reqs;  // CAP == 0
     uint32_t n;
     uint64_t total_cost;
     uint64_t tile_cost;  // largest tile
     const uint32_t *te0;
     TileOrder order;
 };
+template <int CAP>
+struct BatchParams : BatchArgs {
+    BatchReq in_params[CAP];
+    __device__ __forceinline__ const BatchReq *requests() const { return in_params; }
+};
+template <>
+struct BatchParams<0> : BatchArgs {
+    __device__ __forceinline__ const BatchReq *requests() const { return reqs; }
+};
+
+// Requests that fit the kernel's parameters (32764 bytes at most): a batch of
+// up to so many needs no descriptor table in device memory, hence no
+// allocation, no copy and no wait for one.  The small size keeps the launch
+// of a small batch from copying 32 KB.
+constexpr int kFewInParams = 64;
+constexpr int kMostInParams = 500;
+static_assert(sizeof(BatchParams<kMostInParams>) <= 32764, "kernel parameters");
+// Batches of up to so many requests never use a table in device memory.
+constexpr int kMostByParams = AES_NOALLOC_MAX_REQUESTS;
 
 // CTA sizes up to this hold round keys in registers.
 constexpr int kRegsMaxThreads = 512;
@@ -104,7 +124,8 @@ __device__ __forceinline__ uint32_t owner_of(const BatchReq *reqs, uint32_t lo, 
 // work of the calling warp (every lane with the same arguments).  s_pos: the CTA's
 // counter, zeroed before the CTA's last barrier.
 template <class RUN>
-__device__ __forceinline__ void for_each_run(const BatchArgs &p, unsigned long long *s_pos, RUN &&run)
+__device__ __forceinline__ void for_each_run(const BatchArgs &p, const BatchReq *reqs, unsigned long long *s_pos,
+                                             RUN &&run)
 {
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t units = p.order.tiles ? p.order.tiles : p.total_cost;  // this CTA's piece [u0, u1)
@@ -138,10 +159,10 @@ __device__ __forceinline__ void for_each_run(const BatchArgs &p, unsigned long l
             xa = u0 + at;
             xb = u0 + (at + take < size ? at + take : size);
         }
-        ri = owner_of(p.reqs, ri, p.n, xa, near);
+        ri = owner_of(reqs, ri, p.n, xa, near);
         near = !p.order.tiles;  // later tiles lie further along
         for (uint32_t i = ri; i < p.n; ++i) {
-            const BatchReq rq = p.reqs[i];
+            const BatchReq rq = reqs[i];
             if (rq.cost_begin >= xb)
                 break;
             // chunk c belongs to the tile that holds its first cost unit
@@ -169,8 +190,8 @@ __device__ __forceinline__ void for_each_run(const BatchArgs &p, unsigned long l
 // (4870 against 4957 us for the same lengths) and slower on AES-128 (3459
 // against 3356), as are 448 (5258 and 3401).  MAXT: largest CTA it is launched with; RK_REGS:
 // round keys in registers (else in the warp's slice of shared memory).
-template <int MAXT, bool RK_REGS>
-__global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_constant__ BatchArgs p)
+template <int MAXT, bool RK_REGS, int CAP>
+__global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_constant__ BatchParams<CAP> p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ uint4 s_group[MAXT / 32][aestile::kRunGroups];
@@ -200,7 +221,7 @@ __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_cons
             aestile::xor_run<NR>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, k0, n, w_group, ln, rk);
         }
     };
-    for_each_run(p, &s_pos, [&](const BatchReq &rq, uint64_t k0, uint32_t n) {
+    for_each_run(p, p.requests(), &s_pos, [&](const BatchReq &rq, uint64_t k0, uint32_t n) {
         switch (rq.nr) {
         case 10: xor_with(rq, k0, n, std::integral_constant<int, 10>()); break;
         case 12: xor_with(rq, k0, n, std::integral_constant<int, 12>()); break;
@@ -213,7 +234,8 @@ __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_cons
 // by one warp 1024 blocks at a time (bs_tile.cuh) with the request's
 // round-key bit planes in the warp's slice of shared memory (rebuilt when the
 // warp moves to a request with another key).
-__global__ void __launch_bounds__(kBsThreads) batch_bitslice_kernel(const __grid_constant__ BatchArgs p)
+template <int CAP>
+__global__ void __launch_bounds__(kBsThreads) batch_bitslice_kernel(const __grid_constant__ BatchParams<CAP> p)
 {
     __shared__ __align__(16) uint32_t s_mask[kBsThreads / 32][15 * 128];
     __shared__ unsigned long long s_pos;
@@ -225,7 +247,7 @@ __global__ void __launch_bounds__(kBsThreads) batch_bitslice_kernel(const __grid
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t *mask = s_mask[threadIdx.x >> 5];
     const uint4 *cur = nullptr;  // schedule whose masks are in `mask`
-    for_each_run(p, &s_pos, [&](const BatchReq &rq, uint64_t k0, uint32_t n) {
+    for_each_run(p, p.requests(), &s_pos, [&](const BatchReq &rq, uint64_t k0, uint32_t n) {
         const uint64_t v0 = rq.iv_lo & 255u, nb = (rq.len + 15) >> 4;
         const uint64_t first = k0 << 5 > v0 ? (k0 << 5) - v0 : 0;
         const uint64_t end = ((k0 + n) << 5) - v0, last = end < nb ? end : nb;
@@ -256,11 +278,15 @@ cudaError_t batch_set_attributes()
 {
     cudaError_t e;
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if ((e = cudaFuncSetAttribute(batch_ttable_kernel<kRegsMaxThreads, true>, attr, (int)aestt::kTableBytes)) ||
-        (e = cudaFuncSetAttribute(batch_ttable_kernel<1024, false>, attr, (int)aestt::kTableBytes)))
+    const int smem = (int)aestt::kTableBytes;
+    if ((e = cudaFuncSetAttribute(batch_ttable_kernel<kRegsMaxThreads, true, 0>, attr, smem)) ||
+        (e = cudaFuncSetAttribute(batch_ttable_kernel<kRegsMaxThreads, true, kFewInParams>, attr, smem)) ||
+        (e = cudaFuncSetAttribute(batch_ttable_kernel<kRegsMaxThreads, true, kMostInParams>, attr, smem)) ||
+        (e = cudaFuncSetAttribute(batch_ttable_kernel<1024, false, 0>, attr, smem)) ||
+        (e = cudaFuncSetAttribute(batch_ttable_kernel<1024, false, kMostInParams>, attr, smem)))
         return e;
     int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_bitslice_kernel, kBsThreads, 0)))
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_bitslice_kernel<0>, kBsThreads, 0)))
         return e;
     g_bs_ctas_per_sm = per_sm > 0 ? per_sm : 1;
     return cudaSuccess;
@@ -297,12 +323,10 @@ static TileOrder make_order(uint64_t total, uint32_t seed)
     return o;
 }
 
-// Host-side preparation shared by aes_ctr_batch and the plans: the requests
-// that hold any bytes.
-struct BatchTables {
-    std::vector<BatchReq> reqs;
-    uint64_t total_cost = 0;
-    uint64_t total_chunks = 0;
+// What a launch needs to know of its requests.
+struct BatchSums {
+    size_t n = 0;  // requests that hold any bytes
+    uint64_t cost = 0, chunks = 0;
     int64_t bytes = 0;
 };
 
@@ -334,7 +358,7 @@ static BatchShape pick_batch_shape(const DeviceState &st, const aes_batch_opts_t
         if (opts->variant && opts->variant != s.variant) {
             // another variant than the tuned one: start from its defaults
             s = opts->variant == AES_VARIANT_BITSLICE ? BatchShape{AES_VARIANT_BITSLICE, kBsThreads, 2048, 0, 1}
-                                                      : BatchShape{opts->variant, 512, 2048, 0, 1};
+                                                      : BatchShape{opts->variant, 512, 4096, 0, 1};
         }
         if (opts->threads)
             s.threads = opts->threads;
@@ -348,9 +372,10 @@ static BatchShape pick_batch_shape(const DeviceState &st, const aes_batch_opts_t
     return s;
 }
 
-static int build_tables(const aes_desc_t *descs, int n, int dev, BatchTables &bt)
+// The non-empty requests of descs[0..n) into out (room for n), their sums into
+// `sum`; the first bad request's status.
+static int fill_reqs(const aes_desc_t *descs, int n, int dev, BatchReq *out, BatchSums &sum)
 {
-    bt.reqs.reserve((size_t)n);
     for (int i = 0; i < n; ++i) {
         const aes_desc_t &d = descs[i];
         if (!d.ctx)
@@ -371,40 +396,99 @@ static int build_tables(const aes_desc_t *descs, int n, int dev, BatchTables &bt
         iv_halves(d.iv, &r.iv_hi, &r.iv_lo);
         r.rk = reinterpret_cast<const uint4 *>(d.ctx->d_rk);
         r.nr = (uint32_t)d.ctx->nr;
-        r.cost_begin = bt.total_cost;
+        r.cost_begin = sum.cost;
         const uint64_t chunks = chunks_of(d.len, d.iv[15]);
-        bt.total_chunks += chunks;
-        bt.total_cost += chunks * chunk_cost(r.nr);
-        bt.bytes += (int64_t)d.len;
-        bt.reqs.push_back(r);
+        sum.chunks += chunks;
+        sum.cost += chunks * chunk_cost(r.nr);
+        sum.bytes += (int64_t)d.len;
+        out[sum.n++] = r;
     }
     return AES_OK;
 }
 
-uint32_t batch_chunk_cost(int nr) { return chunk_cost((uint32_t)nr); }
-
-cudaError_t launch_batch(const BatchReq *reqs, size_t n, uint64_t total_cost, uint64_t total_chunks,
-                                const uint32_t *te0, const BatchShape &s, int nsm, uint32_t seed, cudaStream_t stream)
+// Everything of a launch but its requests; returns the grid size.
+static int set_args(BatchArgs &p, const BatchSums &sum, const DeviceState &st, const BatchShape &s, uint32_t seed)
 {
-    BatchArgs p{};
-    p.reqs = reqs;
-    p.n = (uint32_t)n;
-    p.total_cost = total_cost;
+    p.reqs = nullptr;
+    p.n = (uint32_t)sum.n;
+    p.total_cost = sum.cost;
     p.tile_cost = (uint64_t)(s.tile_blocks / 32) * chunk_cost(10);
-    p.te0 = te0;
-    p.order = make_order((total_cost + p.tile_cost - 1) / p.tile_cost, seed);
+    p.te0 = st.te0;
+    p.order = make_order((sum.cost + p.tile_cost - 1) / p.tile_cost, seed);
     // as many CTAs as are resident at once (one T-table CTA per SM: its
     // tables take 128 KiB of shared memory), none without a chunk
-    const int resident = s.variant == AES_VARIANT_BITSLICE ? nsm * g_bs_ctas_per_sm : nsm;
-    int ctas = s.ctas > 0 ? std::min(s.ctas, resident) : resident;
-    if ((uint64_t)ctas > total_chunks)
-        ctas = (int)total_chunks;
-    if (s.variant == AES_VARIANT_BITSLICE)
-        return launch_overlapped(batch_bitslice_kernel, ctas, kBsThreads, 0, stream, p);
-    return s.threads <= kRegsMaxThreads
-               ? launch_overlapped(batch_ttable_kernel<kRegsMaxThreads, true>, ctas, s.threads, aestt::kTableBytes,
-                                   stream, p)
-               : launch_overlapped(batch_ttable_kernel<1024, false>, ctas, s.threads, aestt::kTableBytes, stream, p);
+    const int resident = s.variant == AES_VARIANT_BITSLICE ? st.nsm * g_bs_ctas_per_sm : st.nsm;
+    const int ctas = s.ctas > 0 ? std::min(s.ctas, resident) : resident;
+    return (uint64_t)ctas > sum.chunks ? (int)sum.chunks : ctas;
+}
+
+template <int CAP>
+static cudaError_t launch_batch(const BatchParams<CAP> &p, int ctas, const BatchShape &s, cudaStream_t stream)
+{
+    if constexpr (CAP != kFewInParams) {  // the small size exists for the default shape's kernel only
+        if (s.variant == AES_VARIANT_BITSLICE)
+            return launch_overlapped(batch_bitslice_kernel<CAP>, ctas, kBsThreads, 0, stream, p);
+        if (s.threads > kRegsMaxThreads)
+            return launch_overlapped(batch_ttable_kernel<1024, false, CAP>, ctas, s.threads, aestt::kTableBytes,
+                                     stream, p);
+    }
+    return launch_overlapped(batch_ttable_kernel<kRegsMaxThreads, true, CAP>, ctas, s.threads, aestt::kTableBytes,
+                             stream, p);
+}
+
+// n <= CAP requests in one launch whose parameters hold them.
+template <int CAP>
+static int launch_in_params(const aes_desc_t *descs, int n, const DeviceState &st, const BatchShape &s, uint32_t seed,
+                            cudaStream_t stream)
+{
+    BatchParams<CAP> p;
+    BatchSums sum;
+    const int rc = fill_reqs(descs, n, st.device, p.in_params, sum);
+    if (rc || !sum.n)
+        return rc;
+    const int ctas = set_args(p, sum, st, s, seed);
+    const cudaError_t e = launch_batch(p, ctas, s, stream);
+    return e ? cuda_fail(e, "aes_ctr_batch launch") : AES_OK;
+}
+
+int batch_by_params(const aes_desc_t *descs, int n, const DeviceState &st, const BatchShape &s, uint32_t seed,
+                    cudaStream_t stream)
+{
+    if (n <= kFewInParams && s.variant == AES_VARIANT_TTABLE && s.threads <= kRegsMaxThreads)
+        return launch_in_params<kFewInParams>(descs, n, st, s, seed, stream);
+    if (n <= kMostInParams)
+        return launch_in_params<kMostInParams>(descs, n, st, s, seed, stream);
+    // Nothing runs unless every request is good.
+    std::vector<BatchReq> reqs;
+    try {
+        reqs.resize((size_t)n);
+    } catch (const std::bad_alloc &) {
+        return AES_ENOMEM;
+    }
+    BatchSums sum;
+    const int rc = fill_reqs(descs, n, st.device, reqs.data(), sum);
+    if (rc || !sum.n)
+        return rc;
+    // equal numbers of requests per launch
+    const size_t launches = (sum.n + kMostInParams - 1) / kMostInParams;
+    BatchParams<kMostInParams> p;
+    for (size_t k = 0; k < launches; ++k) {
+        const size_t a = sum.n * k / launches, b = sum.n * (k + 1) / launches;
+        BatchSums part;
+        for (size_t i = a; i < b; ++i) {
+            BatchReq &r = p.in_params[part.n++];
+            r = reqs[i];
+            r.cost_begin = part.cost;
+            const uint64_t chunks = chunks_of(r.len, (uint32_t)(r.iv_lo & 255u));
+            part.chunks += chunks;
+            part.cost += chunks * chunk_cost(r.nr);
+        }
+        const int ctas = set_args(p, part, st, s, seed);
+        const cudaError_t e = launch_batch(p, ctas, s, stream);
+        if (e)
+            return cuda_fail(e, "aes_ctr_batch launch");
+    }
+    return AES_OK;
 }
 
 }  // namespace aesrt
@@ -413,9 +497,10 @@ using namespace aesrt;
 
 struct aes_batch_plan_s {
     int device;
-    BatchTables bt;
+    BatchSums sum;
     BatchShape shape;
-    uint32_t seed = 0;
+    BatchParams<0> params{};
+    int ctas = 0;
     BatchReq *reqs = nullptr;  // device
 };
 
@@ -436,23 +521,38 @@ int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_bat
     BatchShape s = pick_batch_shape(*st, opts);
     if ((rc = validate_batch_shape(s)))
         return rc;
-    BatchTables bt;
-    if ((rc = build_tables(descs, n, st->device, bt)))
-        return rc;
-    if (bt.reqs.empty())
-        return AES_OK;
+    const uint32_t seed = opts ? opts->tile_order_seed : 0;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
+    // Up to two or three launches with the requests in their parameters cost
+    // what one launch with a table in device memory does (1000 requests of 1
+    // to 16 KiB: 175.5 and 176.9 us a call in a row of calls; 512 of 1 KiB to
+    // 8 MiB: 539 and 537), and a call on an idle GPU is sooner done without
+    // the allocation and the copy (209 and 359 us, 639 and 800).  A capture
+    // must not record the copy: its host source is gone when the graph runs.
+    if (n <= kMostByParams || capturing(cs))
+        return batch_by_params(descs, n, *st, s, seed, cs);
+    std::vector<BatchReq> host;
+    try {
+        host.resize((size_t)n);
+    } catch (const std::bad_alloc &) {
+        return AES_ENOMEM;
+    }
+    BatchSums sum;
+    if ((rc = fill_reqs(descs, n, st->device, host.data(), sum)) || !sum.n)
+        return rc;
+    BatchParams<0> p{};
+    const int ctas = set_args(p, sum, *st, s, seed);
     BatchReq *reqs = nullptr;
-    const size_t bytes = bt.reqs.size() * sizeof(BatchReq);
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&reqs), bytes, cs);
+    const size_t bytes = sum.n * sizeof(BatchReq);
+    cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&reqs), bytes, st->pool, cs);
     if (e)
-        return e == cudaErrorMemoryAllocation ? AES_ENOMEM : cuda_fail(e, "cudaMallocAsync");
+        return e == cudaErrorMemoryAllocation ? AES_ENOMEM : cuda_fail(e, "cudaMallocFromPoolAsync");
+    p.reqs = reqs;
     // Pageable source: the copy has finished reading the host vector when
-    // cudaMemcpyAsync returns, so bt may be destroyed afterwards.
-    e = cudaMemcpyAsync(reqs, bt.reqs.data(), bytes, cudaMemcpyHostToDevice, cs);
+    // cudaMemcpyAsync returns, so it may be destroyed afterwards.
+    e = cudaMemcpyAsync(reqs, host.data(), bytes, cudaMemcpyHostToDevice, cs);
     if (!e)
-        e = launch_batch(reqs, bt.reqs.size(), bt.total_cost, bt.total_chunks, st->te0, s, st->nsm,
-                         opts ? opts->tile_order_seed : 0, cs);
+        e = launch_batch(p, ctas, s, cs);
     cudaError_t e2 = cudaFreeAsync(reqs, cs);
     if (e)
         return cuda_fail(e, "aes_ctr_batch");
@@ -488,19 +588,25 @@ int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
         return AES_ENOMEM;
     plan->device = st->device;
     plan->shape = s;
-    plan->seed = opts ? opts->tile_order_seed : 0;
-    if ((rc = build_tables(descs, n, st->device, plan->bt))) {
+    std::vector<BatchReq> host;
+    try {
+        host.resize((size_t)n);
+    } catch (const std::bad_alloc &) {
+        delete plan;
+        return AES_ENOMEM;
+    }
+    if ((rc = fill_reqs(descs, n, st->device, host.data(), plan->sum))) {
         delete plan;
         return rc;
     }
-    const size_t bytes = plan->bt.reqs.size() * sizeof(BatchReq);
-    if (bytes) {
+    if (plan->sum.n) {
+        const size_t bytes = plan->sum.n * sizeof(BatchReq);
         cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&plan->reqs), bytes);
         if (e) {
             delete plan;
             return e == cudaErrorMemoryAllocation ? AES_ENOMEM : cuda_fail(e, "cudaMalloc(plan)");
         }
-        e = cudaMemcpyAsync(plan->reqs, plan->bt.reqs.data(), bytes, cudaMemcpyHostToDevice, st->setup);
+        e = cudaMemcpyAsync(plan->reqs, host.data(), bytes, cudaMemcpyHostToDevice, st->setup);
         if (!e)
             e = cudaStreamSynchronize(st->setup);
         if (e) {
@@ -508,6 +614,8 @@ int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
             delete plan;
             return cuda_fail(e, "aes_batch_plan_create");
         }
+        plan->ctas = set_args(plan->params, plan->sum, *st, s, opts ? opts->tile_order_seed : 0);
+        plan->params.reqs = plan->reqs;
     }
     *out = plan;
     return AES_OK;
@@ -517,25 +625,15 @@ int aes_batch_plan_launch(aes_batch_plan_t plan, void *stream)
 {
     if (!plan)
         return AES_EINVAL;
-    if (plan->bt.reqs.empty())
+    if (!plan->sum.n)
         return AES_OK;  // nothing to encrypt (all lengths zero)
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) == cudaSuccess &&
-        cap != cudaStreamCaptureStatusNone)
+    if (capturing(static_cast<cudaStream_t>(stream)))
         return cuda_fail(cudaErrorStreamCaptureUnsupported, "aes_batch_plan_launch");
-    DeviceState *st = nullptr;
-    int rc = device_state(&st);
-    if (rc)
-        return rc;
-    if (st->device != plan->device)
-        return AES_EINVAL;
-    const cudaError_t e =
-        launch_batch(plan->reqs, plan->bt.reqs.size(), plan->bt.total_cost, plan->bt.total_chunks, st->te0,
-                     plan->shape, st->nsm, plan->seed, static_cast<cudaStream_t>(stream));
+    const cudaError_t e = launch_batch(plan->params, plan->ctas, plan->shape, static_cast<cudaStream_t>(stream));
     return e ? cuda_fail(e, "aes_batch_plan_launch") : AES_OK;
 }
 
-int64_t aes_batch_plan_bytes(aes_batch_plan_t plan) { return plan ? plan->bt.bytes : AES_EINVAL; }
+int64_t aes_batch_plan_bytes(aes_batch_plan_t plan) { return plan ? plan->sum.bytes : AES_EINVAL; }
 
 int aes_batch_plan_destroy(aes_batch_plan_t plan)
 {

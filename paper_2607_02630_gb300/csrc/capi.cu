@@ -46,6 +46,18 @@ int device_state(DeviceState **out)
         std::snprintf(st.name, sizeof(st.name), "%s", prop.name);
         if ((e = cudaStreamCreateWithFlags(&st.setup, cudaStreamNonBlocking)))
             return cuda_fail(e, "cudaStreamCreateWithFlags");
+        // One-shot batches of many requests take their table from a pool that
+        // keeps up to 4 MiB (65536 requests); the default pool gives all of it
+        // back at every synchronisation.
+        cudaMemPoolProps pool{};
+        pool.allocType = cudaMemAllocationTypePinned;
+        pool.location.type = cudaMemLocationTypeDevice;
+        pool.location.id = dev;
+        if ((e = cudaMemPoolCreate(&st.pool, &pool)))
+            return cuda_fail(e, "cudaMemPoolCreate");
+        uint64_t keep = 4u << 20;
+        if ((e = cudaMemPoolSetAttribute(st.pool, cudaMemPoolAttrReleaseThreshold, &keep)))
+            return cuda_fail(e, "cudaMemPoolSetAttribute");
         if ((e = cudaMalloc(&st.te0, 256 * sizeof(uint32_t))))
             return cuda_fail(e, "cudaMalloc(te0)");
         if ((e = launch_te0_init(st.te0, st.setup)))

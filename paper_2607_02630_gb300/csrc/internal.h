@@ -3,7 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stddef.h>
-#include <utility>
+#include <type_traits>
 
 namespace aesrt {
 
@@ -32,6 +32,13 @@ cudaError_t launch_te0_init(uint32_t *te0, cudaStream_t stream);
 cudaError_t launch_key_expand(const uint8_t *keys, const int32_t *bits, const uint32_t *te0,
                               uint32_t *w, int n, cudaStream_t stream);
 
+// Whether the stream is being captured into a graph.
+inline bool capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
+}
+
 // Launch a kernel that calls let_next_launch_start and
 // wait_for_previous_launch: its CTAs may be set up (table fill, constants)
 // while the stream's previous kernel drains, instead of after it has ended
@@ -40,9 +47,9 @@ cudaError_t launch_key_expand(const uint8_t *keys, const int32_t *bits, const ui
 // launches 1.7 us on a stream, 1 MiB 6.9 -> 3.5 us.  While the stream is
 // being captured the launch is a plain one, so captured graphs hold ordinary
 // full dependencies.
-template <class... P, class... A>
-inline cudaError_t launch_overlapped(void (*kernel)(P...), int ctas, int threads, size_t smem, cudaStream_t stream,
-                                     A &&...args)
+template <class P>
+inline cudaError_t launch_overlapped(void (*kernel)(P), int ctas, int threads, size_t smem, cudaStream_t stream,
+                                     const std::remove_const_t<P> &params)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)ctas);
@@ -52,12 +59,12 @@ inline cudaError_t launch_overlapped(void (*kernel)(P...), int ctas, int threads
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    if (!capturing(stream)) {
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
     }
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+    void *args[1] = {const_cast<void *>(static_cast<const void *>(&params))};  // copied by the launch
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), args);
     if (e)
         cudaGetLastError();  // the caller reports it; leave no stale error behind
     return e;
@@ -99,14 +106,7 @@ inline uint64_t chunks_of(uint64_t len, uint32_t iv_low_byte)
     const uint64_t nb = (len + 15) / 16;
     return ((iv_low_byte + nb - 1) >> 5) - (iv_low_byte >> 5) + 1;
 }
-uint32_t batch_chunk_cost(int nr);
 
 cudaError_t batch_set_attributes();
-// One launch of the batch kernel over the n > 0 non-empty requests reqs[0..n)
-// in device memory, whose cost_begin are the prefix sums of
-// chunks_of * batch_chunk_cost; total_cost and total_chunks are the sums over
-// all of them.  seed != 0: tiles in a seeded order.
-cudaError_t launch_batch(const BatchReq *reqs, size_t n, uint64_t total_cost, uint64_t total_chunks,
-                         const uint32_t *te0, const BatchShape &s, int nsm, uint32_t seed, cudaStream_t stream);
 
 }  // namespace aesrt

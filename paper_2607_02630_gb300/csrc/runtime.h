@@ -26,6 +26,7 @@ struct DeviceState {
     char name[256] = {0};
     uint32_t *te0 = nullptr;        // 256-word T-table seed
     cudaStream_t setup = nullptr;   // internal non-blocking stream
+    cudaMemPool_t pool = nullptr;   // descriptor tables of one-shot batches
     CtrShape ctr_tuned[3][kLenBuckets];  // [nr index: 10/12/14][length bucket]
     BatchShape batch_tuned;
     // the last batch-shape sweep: every candidate and its median launch time
@@ -46,6 +47,11 @@ int resolve_ptr(const void *p, int dev, const void **dptr, bool *is_host = nullp
 int check_payload(const void *in, const void *out, size_t len, int dev, const void **din, void **dout,
                   bool *out_is_host = nullptr);
 void iv_halves(const uint8_t *iv, uint64_t *hi, uint64_t *lo);
+
+// batch.cu: the batch call that allocates nothing (launches of at most as many
+// requests as the kernel's parameters hold)
+int batch_by_params(const aes_desc_t *descs, int n, const DeviceState &st, const BatchShape &s, uint32_t seed,
+                    cudaStream_t stream);
 
 // tune.cu
 void tune_defaults(DeviceState &st);

@@ -119,11 +119,11 @@ __device__ __forceinline__ void tile_blocks_of(uint64_t tile, uint32_t tile_grou
 // l + 32m, m = chunk & 7, and every load/store moves 512 contiguous bytes.
 __device__ __forceinline__ uint64_t first_chunk(uint64_t iv_lo) { return (iv_lo & 255u) >> 5; }
 
-constexpr uint32_t kRunChunks = 64;  // chunks whose group constants a warp holds at once
-constexpr uint32_t kRunGroups = 16;  // entries of a warp's s_group slice (a run touches at most 9 groups)
+constexpr uint32_t kRunChunks = 248;  // chunks whose group constants a warp holds at once
+constexpr uint32_t kRunGroups = 32;   // the groups a run touches at most: one per lane
 
 // How many of the chunks k0, k0 + 1, ... of a message one run may take: at
-// most 64, and none past a carry into counter byte 10 (every 2^40 blocks),
+// most 248, and none past a carry into counter byte 10 (every 2^40 blocks),
 // up to which lane_round2 holds for all groups.
 __device__ __forceinline__ uint32_t run_chunks(uint64_t iv_lo, uint64_t k0, uint64_t nk)
 {
@@ -138,9 +138,9 @@ __device__ __forceinline__ uint32_t run_chunks(uint64_t iv_lo, uint64_t k0, uint
 // groups side by side (one group per lane, 27 wavefronts for all of them, kept
 // in the warp's s_group slice), then walk the chunks with the same counter low
 // bytes one after the other, so that a lane's part of round 2 (lane_round2) is
-// computed once for up to 8 groups.  Per 64 chunks that is 27 + 43 wavefronts
-// and one broadcast load per chunk, 2.1 a chunk; constants per group and warp
-// and five lookups per block were 8.4.  The next chunk's plaintext is loaded
+// computed once for all groups.  Per 64 chunks that is 27 + 43 wavefronts and
+// one broadcast load per chunk, 2.1 a chunk (1.5 at 128); constants per group
+// and warp and five lookups per block were 8.4.  The next chunk's plaintext is loaded
 // before the current chunk's rounds.  Nothing past len is touched; the final
 // partial block is done bytewise.
 template <int NR, class RK>
@@ -168,8 +168,7 @@ __device__ __forceinline__ void xor_run(const uint4 *__restrict__ in, uint4 *__r
         const uint64_t l = l0 + ((uint64_t)lane << 8);
         const uint4 q = aestt::group_round2(aestt::CounterWords(h0 + (l < l0 ? 1 : 0), l), ln, rk);
         __syncwarp();  // every lane is done with the previous run's constants
-        if (lane < kRunGroups)
-            s_group[lane] = q;
+        s_group[lane] = q;
         __syncwarp();
     }
     const uint32_t column0 = aestt::column0_round1(aestt::CounterWords(h0, l0), ln, rk);

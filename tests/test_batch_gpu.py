@@ -286,3 +286,35 @@ def test_cost_line_edges(cuda, aes, ncpu, n, ctas, tile_blocks, seed, threads):
         meta[i] = (meta[i][0], meta[i][1], np.frombuffer(bytes(b), np.uint8), meta[i][3], k)
     aes.batch(reqs, ctas=ctas, tile_blocks=tile_blocks, tile_order_seed=seed, threads=threads)
     check_all(cuda, meta, payload, dst, 1)
+
+
+@pytest.mark.parametrize("n", [3, 64, 65, 1100])
+def test_batch_calls_under_capture(cuda, aes, ncpu, n):
+    """One-shot batches captured into a CUDA graph (their requests travel in
+    kernel parameters, several launches of them past 500): nothing runs during
+    the capture, and every replay encrypts what the buffers then hold.  A
+    plan's launch is refused while its stream is being captured."""
+    g = W.rng(5600 + n)
+    lengths = [int(x) for x in g.integers(0, 3000, n)]
+    bits = [(128, 192, 256)[i % 3] for i in range(n)]
+    for call in (aes.batch_status, aes.batch_noalloc_status):
+        if call is aes.batch_noalloc_status and n > 1024:
+            continue
+        reqs, meta, payload, src, dst = make_requests(cuda, aes, g, lengths, bits)
+        plan = aes.BatchPlan(reqs)
+        s = cuda.cuda.Stream()
+        cuda.cuda.synchronize()
+        graph = cuda.cuda.CUDAGraph()
+        with cuda.cuda.graph(graph, stream=s, capture_error_mode="thread_local"):
+            assert call(reqs, stream=s) == aes.AES_OK
+            assert aes.lib().aes_batch_plan_launch(plan.handle, s.cuda_stream) == aes.AES_ECUDA
+        plan.close()
+        assert (dst == 0xA5).all()
+        graph.replay()
+        check_all(cuda, meta, payload, dst, 1)
+        payload2 = W.random_bytes(g, payload.size)
+        src.copy_(cuda.from_numpy(payload2))
+        dst.fill_(0xA5)
+        graph.replay()
+        check_all(cuda, meta, payload2, dst, 1)
+        del graph

@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 import threading
 
 from . import build as _build
@@ -60,6 +61,11 @@ class Desc(ctypes.Structure):
 class BatchOpts(ctypes.Structure):
     _fields_ = [("variant", ctypes.c_int), ("threads", ctypes.c_int), ("tile_blocks", ctypes.c_int),
                 ("ctas", ctypes.c_int), ("tile_order_seed", ctypes.c_uint32), ("blocks_per_thread", ctypes.c_int)]
+
+
+_DESC = struct.Struct("=Q16sQQQ")  # Desc's fields in order, no padding
+assert ctypes.sizeof(Desc) == _DESC.size
+_U64 = (1 << 64) - 1
 
 
 class Peaks(ctypes.Structure):
@@ -230,10 +236,25 @@ def ptr(x) -> int:
     return int(x.data_ptr())
 
 
+_raw_stream = None  # () -> handle of torch's current stream, set on first use
+
+
+def _current_stream() -> int:
+    """The handle of torch's current stream.  torch.cuda.current_stream builds
+    a Stream object for it (3.1 us of a 7.8 us call on the Grace host); the
+    two calls below read the same stream in 0.3 us."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        torch.cuda.init()  # as torch.cuda.current_stream does
+        device, raw = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+        _raw_stream = lambda: raw(device())  # noqa: E731
+    return _raw_stream()
+
+
 def stream_handle(s) -> int:
     if s is None:
-        import torch
-        return int(torch.cuda.current_stream().cuda_stream)
+        return _current_stream()
     if isinstance(s, int):
         return s
     return int(s.cuda_stream)
@@ -316,14 +337,21 @@ def ctr_sync(ctx: Context, iv, src, dst, nbytes: int, stream=None) -> None:
 
 
 def _descs(requests):
-    arr = (Desc * max(len(requests), 1))()
-    for i, (ctx, iv, src, dst, n) in enumerate(requests):
-        arr[i].ctx = ctx.handle
-        arr[i].iv = _bytes16(iv)
-        arr[i].inp = ptr(src)
-        arr[i].out = ptr(dst)
-        arr[i].len = int(n)
-    return arr
+    """The requests as a Desc array, each packed by one struct call: setting
+    the fields of ctypes structures took 1.04 us a request on the Grace host,
+    most of a batch call of short requests."""
+    n = len(requests)
+    if not n:
+        return (Desc * 1)()
+    pack = _DESC.pack
+    try:
+        packed = [pack(ctx.handle or 0, iv if type(iv) is bytes and len(iv) == 16 else _iv_bytes(iv),
+                       src if type(src) is int else ptr(src), dst if type(dst) is int else ptr(dst), k)
+                  for ctx, iv, src, dst, k in requests]
+    except struct.error:  # a value no unsigned word holds wraps, as ctypes integer fields do
+        packed = [pack(ctx.handle or 0, _iv_bytes(iv), ptr(src) & _U64, ptr(dst) & _U64, int(k) & _U64)
+                  for ctx, iv, src, dst, k in requests]
+    return (Desc * n).from_buffer_copy(b"".join(packed))
 
 
 def batch_status(requests, stream=None, variant=0, threads=0, tile_blocks=0, ctas=0,

@@ -376,6 +376,7 @@ static BatchShape pick_batch_shape(const DeviceState &st, const aes_batch_opts_t
 // `sum`; the first bad request's status.
 static int fill_reqs(const aes_desc_t *descs, int n, int dev, BatchReq *out, BatchSums &sum)
 {
+    PayloadChecks payloads(dev);
     for (int i = 0; i < n; ++i) {
         const aes_desc_t &d = descs[i];
         if (!d.ctx)
@@ -386,7 +387,7 @@ static int fill_reqs(const aes_desc_t *descs, int n, int dev, BatchReq *out, Bat
             continue;
         const void *din = nullptr;
         void *dout = nullptr;
-        const int rc = check_payload(d.in, d.out, d.len, dev, &din, &dout);
+        const int rc = payloads.check(d.in, d.out, d.len, &din, &dout);
         if (rc)
             return rc;
         BatchReq r{};

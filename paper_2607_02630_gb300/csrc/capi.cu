@@ -5,6 +5,8 @@
 #include "internal.h"
 #include "runtime.h"
 
+#include <cuda.h>
+
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -118,8 +120,8 @@ int resolve_ptr(const void *p, int dev, const void **dptr, bool *is_host)
     }
 }
 
-int check_payload(const void *in, const void *out, size_t len, int dev, const void **din, void **dout,
-                  bool *out_is_host)
+// What any payload must satisfy, whatever memory it lies in.
+static int check_bounds(const void *in, const void *out, size_t len)
 {
     if (!in || !out)
         return AES_EINVAL;
@@ -130,10 +132,18 @@ int check_payload(const void *in, const void *out, size_t len, int dev, const vo
         if (a < b + len && b < a + len)
             return AES_EOVERLAP;
     }
+    return AES_OK;
+}
+
+int check_payload(const void *in, const void *out, size_t len, int dev, const void **din, void **dout,
+                  bool *out_is_host)
+{
+    int rc = check_bounds(in, out, len);
+    if (rc)
+        return rc;
     const void *di = nullptr, *dout_c = nullptr;
     bool in_host = false, o_host = false;
-    int rc = resolve_ptr(in, dev, &di, &in_host);
-    if (rc)
+    if ((rc = resolve_ptr(in, dev, &di, &in_host)))
         return rc;
     if (out == in) {
         dout_c = di;
@@ -145,6 +155,94 @@ int check_payload(const void *in, const void *out, size_t len, int dev, const vo
         *out_is_host = o_host;
     *din = di;
     *dout = const_cast<void *>(dout_c);
+    return AES_OK;
+}
+
+namespace {
+
+// Driver calls behind the bounds of an allocation (null if not found).
+struct DriverCalls {
+    CUresult (*range)(CUdeviceptr *, size_t *, CUdeviceptr) = nullptr;
+    CUresult (*attribute)(void *, CUpointer_attribute, CUdeviceptr) = nullptr;
+    CUresult (*retain)(CUmemGenericAllocationHandle *, void *) = nullptr;
+    CUresult (*release)(CUmemGenericAllocationHandle) = nullptr;
+    bool ok = false;
+    DriverCalls()
+    {
+        auto find = [](const char *name, int since, void *fn) {
+            cudaDriverEntryPointQueryResult r;
+            return cudaGetDriverEntryPointByVersion(name, static_cast<void **>(fn), since, cudaEnableDefault, &r) ==
+                       cudaSuccess && r == cudaDriverEntryPointSuccess;
+        };
+        ok = find("cuMemGetAddressRange", 3020, &range) && find("cuPointerGetAttribute", 4000, &attribute) &&
+             find("cuMemRetainAllocationHandle", 11000, &retain) && find("cuMemRelease", 10020, &release);
+        cudaGetLastError();
+    }
+};
+
+// Bounds of the allocation that holds the device pointer p: of one made by
+// cudaMalloc only, where every address between them is device memory.  Pool
+// memory and mapped address ranges can have holes, so their pointers are
+// looked up one by one.
+bool allocation_bounds(const void *p, uintptr_t *begin, uintptr_t *end)
+{
+    static const DriverCalls d;
+    if (!d.ok)
+        return false;
+    const CUdeviceptr ptr = (CUdeviceptr)(uintptr_t)p;
+    CUmemGenericAllocationHandle h;
+    if (d.retain(&h, const_cast<void *>(p)) == CUDA_SUCCESS) {
+        d.release(h);
+        return false;
+    }
+    CUmemoryPool pool = nullptr;
+    if (d.attribute(&pool, CU_POINTER_ATTRIBUTE_MEMPOOL_HANDLE, ptr) != CUDA_SUCCESS || pool)
+        return false;
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    if (d.range(&base, &size, ptr) != CUDA_SUCCESS)
+        return false;
+    *begin = (uintptr_t)base;
+    *end = (uintptr_t)base + size;
+    return true;
+}
+
+}  // namespace
+
+int PayloadChecks::resolve(const void *p, Range &r, const void **dptr)
+{
+    const uintptr_t a = (uintptr_t)p;
+    if (a >= r.begin && a < r.end) {
+        r.misses = 0;
+        *dptr = p;
+        return AES_OK;
+    }
+    bool host = false;
+    const int rc = resolve_ptr(p, dev_, dptr, &host);
+    // payloads spread over many allocations: stop looking for their bounds
+    if (rc || host || *dptr != p || r.misses > 4)
+        return rc;
+    ++r.misses;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || at.type != cudaMemoryTypeDevice ||
+        !allocation_bounds(p, &r.begin, &r.end))
+        r.begin = r.end = 0;
+    return AES_OK;
+}
+
+int PayloadChecks::check(const void *in, const void *out, size_t len, const void **din, void **dout)
+{
+    int rc = check_bounds(in, out, len);
+    if (rc || (rc = resolve(in, in_, din)))
+        return rc;
+    if (out == in) {
+        *dout = const_cast<void *>(*din);
+        return AES_OK;
+    }
+    const void *o = nullptr;
+    if ((rc = resolve(out, out_, &o)))
+        return rc;
+    *dout = const_cast<void *>(o);
     return AES_OK;
 }
 

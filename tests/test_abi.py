@@ -196,3 +196,35 @@ def test_iv_marshalling():
     for bad in (b"", bytes(15), bytes(17), np.zeros(8, dtype=np.uint16)[:7]):
         with pytest.raises(ValueError):
             A._iv_bytes(bad)
+
+
+def test_descriptor_marshalling():
+    """Requests reach the library as Desc arrays with the fields as given:
+    handles (none for a closed context), IVs from any 16-byte buffer,
+    addresses from integers, tensors or None, and values that no unsigned
+    word holds wrapped as ctypes fields wrap them."""
+    import numpy as np
+
+    class Ctx:
+        def __init__(self, h):
+            self.handle = h
+
+    class Tensor:
+        def data_ptr(self):
+            return 0x7F00_0000_0100
+
+    iv = bytes(range(16))
+    plain = [(Ctx(0x1234), iv, 1 << 47, Tensor(), 5), (Ctx(None), bytearray(iv), None, 0, 0),
+             (Ctx(7), np.frombuffer(iv, np.uint8), 256, 512, np.int64(9))]
+    odd = plain + [(Ctx(1), iv, -16, (1 << 64) + 32, -1)]
+    for reqs in (plain, odd):
+        arr = A._descs(reqs)
+        assert len(arr) == len(reqs) and isinstance(arr[0], A.Desc)
+        got = [(d.ctx or 0, bytes(d.iv), d.inp or 0, d.out or 0, d.len) for d in arr]
+        want = [(0x1234, iv, 1 << 47, 0x7F00_0000_0100, 5), (0, iv, 0, 0, 0), (7, iv, 256, 512, 9),
+                (1, iv, (1 << 64) - 16, 32, (1 << 64) - 1)][: len(reqs)]
+        assert got == want
+    for bad in (bytes(15), bytes(17)):
+        with pytest.raises(ValueError):
+            A._descs([(Ctx(1), bad, 0, 0, 0)])
+    assert ctypes.sizeof(A._descs([])) >= ctypes.sizeof(A.Desc)

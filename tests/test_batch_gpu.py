@@ -318,3 +318,26 @@ def test_batch_calls_under_capture(cuda, aes, ncpu, n):
         graph.replay()
         check_all(cuda, meta, payload2, dst, 1)
         del graph
+
+
+@pytest.mark.parametrize("n", [2, 70, 600])
+def test_batch_checks_every_payload_pointer(cuda, aes, n):
+    """A batch whose payloads share allocations still refuses the one request
+    whose pointer the GPU cannot address, wherever it stands in the batch, and
+    accepts pinned host memory among device memory."""
+    ctx = aes.Context(bytes(16), 128)
+    buf = cuda.zeros(n * 512, dtype=cuda.uint8, device="cuda")
+    pinned = cuda.zeros(4096, dtype=cuda.uint8).pin_memory()
+    pageable = np.zeros(8192, np.uint8)
+    bad = (pageable.ctypes.data + 15) & ~15
+    p = buf.data_ptr()
+    reqs = [(ctx, bytes(16), p + 512 * i, p + 512 * i + 256, 200) for i in range(n)]
+    for at in sorted({0, 1, n - 1}):
+        for src, dst, want in ((bad, p + 256, aes.AES_EPTR), (p, bad, aes.AES_EPTR), (bad, bad, aes.AES_EPTR),
+                               (256, p + 256, aes.AES_EPTR), (0, p + 256, aes.AES_EINVAL),
+                               (pinned.data_ptr(), pinned.data_ptr() + 1024, aes.AES_OK)):
+            q = list(reqs)
+            q[at] = (ctx, bytes(16), src, dst, 200)
+            assert aes.batch_status(q) == want
+            assert aes.batch_noalloc_status(q) == want
+    cuda.cuda.synchronize()

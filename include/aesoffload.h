@@ -298,7 +298,8 @@ typedef struct {
     int ctas;               /* resident CTAs; 0 = SM count - 4 */
     int threads;            /* CTA size, multiple of 32, 64..512; 0 = 512 (warp 0 dispatches) */
     int tile_blocks;        /* 16-byte blocks per tile: 64, 128 or a multiple of 256;
-                               0 = per request (~512 tiles of 64..1024 blocks:
+                               0 = per request (~512 tiles of 64..1024 blocks,
+                               down to 64 tiles with 64 requests in flight:
                                the latency setting).  Fewer, larger tiles serve
                                more requests per second (measured on GB300,
                                served mix: 269 k req/s by default, 370 k with

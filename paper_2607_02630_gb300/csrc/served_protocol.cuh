@@ -43,6 +43,10 @@ constexpr uint32_t kExitStop = 1, kExitIdle = 2, kExitError = 4;
 constexpr uint32_t kNotReady = 8;  // advance(): next request not ready (not an exit reason)
 constexpr uint32_t kFlagHostOut = 1;   // QEntry.flags: the output is pinned host memory
 constexpr uint32_t kFlagEmulated = 2;  // QEntry.flags: emulated offload, len = duration in ns
+// QEntry.flags, bits 2..3: how far the adaptive tile count is halved, by the
+// requests in flight when this one was submitted (tile_level).
+constexpr uint32_t kFlagLevelShift = 2;
+constexpr uint32_t kFlagLevelMask = 3;
 constexpr uint64_t kMaxEmulatedNs = 10000000;
 constexpr int kMaxWarps = 16;   // CTA of at most 512 threads (128 registers each: round keys in registers)
 constexpr uint32_t kRing = 64;  // >= workers + prefetch
@@ -77,7 +81,7 @@ struct QEntry {  // 64 bytes, host-written into the request's slot before its or
     uint64_t in, out, len, iv_hi, iv_lo, gen;
     uint32_t key_slot;  // key slot (bits 0..23) | Nr of its key (bits 24..31; 0 = not registered)
     uint16_t desc;   // slot index d
-    uint16_t flags;  // kFlagHostOut, kFlagEmulated
+    uint16_t flags;  // kFlagHostOut, kFlagEmulated, tile level
 };
 static_assert(sizeof(QEntry) == 64, "QEntry layout");
 
@@ -599,14 +603,16 @@ SRV_NOINLINE uint32_t dispatch(const SrvParams &p, uint32_t k0, uint32_t n_max, 
         } else if (ok && len) {
             // tiles are runs of tg whole 256-block counter groups, or (tp > 1)
             // equal parts of one group.  Unless fixed by the server config, a
-            // request is cut into about 512 tiles of 64..1024 blocks: short
-            // requests spread over many warps, long ones keep claims rare.
+            // request is cut into about 512 tiles (fewer with many requests
+            // in flight, tile_level) of 64..1024 blocks: short requests
+            // spread over many warps, long ones keep claims rare.
             const uint64_t nb = (len + 15) >> 4;
             const uint64_t groups = (((iv_lo & 255u) + nb - 1) >> 8) + 1;
             uint32_t tb = p.tile_blocks;
             if (!tb) {
+                const uint32_t want = 512u >> ((flags >> kFlagLevelShift) & kFlagLevelMask);
                 tb = 64;
-                while (tb < 1024 && (uint64_t)tb * 512 < nb)
+                while (tb < 1024 && (uint64_t)tb * want < nb)
                     tb <<= 1;
             }
             if (tb >= 256)

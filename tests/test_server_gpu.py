@@ -744,3 +744,33 @@ def test_trace_build_stamps(cuda, aes, claim_mode):
     res = json.loads(r.stdout.strip().splitlines()[-1])
     assert res["ordered"] and res["median_us"]["done"] > 0, res
     assert res["claim_mode"] == claim_mode
+
+
+@pytest.mark.parametrize("n", [15, 16, 33, 70])
+def test_tiles_by_requests_in_flight(cuda, aes, ncpu, n):
+    """The default server cuts a request into fewer tiles the more requests
+    are in flight when it is submitted (steps at 16, 32 and 64): none is
+    polled before all are submitted, sizes around the tile shapes' edges."""
+    srv = aes.Server(idle_timeout_us=500_000)
+    try:
+        g = W.rng(6900 + n)
+        keys = [(W.random_bytes(g, b // 8), b) for b in (128, 256, 192)]
+        slots = [srv.key_register(k.tobytes(), b) for k, b in keys]
+        edges = [1, 4096 + 5, 65536, (1 << 19) + 16, 1 << 20, (1 << 20) + 7, 3 << 20]
+        sizes = [edges[i % len(edges)] for i in range(n)]
+        payload, offs, src, dst = arena(cuda, g, sizes)
+        sent = []
+        for i, k in enumerate(sizes):
+            iv = iv_with_low(g, ("random", "low32", "low64")[i % 3])
+            o = int(offs[i])
+            sent.append((srv.submit(slots[i % 3], iv.tobytes(), src.data_ptr() + o, dst.data_ptr() + o, k), iv, o, k))
+        for t, iv, o, k in sent:
+            assert srv.wait(t, WAIT_US) == aes.AES_OK
+        out = to_host(dst)
+        for i, (t, iv, o, k) in enumerate(sent):
+            key, bits = keys[i % 3]
+            np.testing.assert_array_equal(out[o: o + k], oracle.ctr_mt(key, bits, iv, payload[o: o + k], ncpu),
+                                          err_msg=f"request {i} len {k}")
+            assert (out[o + k: o + k + 16] == 0xA5).all()
+    finally:
+        assert srv.close() == aes.AES_OK

@@ -160,51 +160,9 @@ __device__ __forceinline__ void rounds(uint32_t (&s)[NB][4], const Lanes &ln,
 // round 1 gives columns (P0 ^ Te3[L ^ k15], C1, C2, C3) with P0, C1..C3 fixed
 // for the group.  In round 2 the varying column 0 feeds exactly one lookup of
 // each output column (row r of column 0 reaches column -r mod 4), so round 2
-// is Q_c ^ (one lookup) with Q0..Q3 fixed for the group.  A block then needs 5
-// lookups for rounds 1-2 instead of 32; the group constants cost 27 lookups
-// once per group.
-struct Group {
-    uint32_t p0, c1, c2, c3, q0, q1, q2, q3, k15;
-};
-
-// base: the group's first counter block (byte 15 = 0) as column words.
-template <class RK>
-__device__ __forceinline__ Group group_consts(const uint32_t base[4], const Lanes &ln,
-                                              const RK &rk)
-{
-    const uint4 k0 = rk.get(0), k1 = rk.get(1), k2 = rk.get(2);
-    const uint32_t s0 = base[0] ^ k0.x, s1 = base[1] ^ k0.y, s2 = base[2] ^ k0.z, s3 = base[3] ^ k0.w;
-    Group g;
-    g.k15 = k0.w >> 24;
-    g.p0 = te<0, 0>(s0, ln) ^ te<1, 1>(s1, ln) ^ te<2, 2>(s2, ln) ^ k1.x;
-    g.c1 = te<0, 0>(s1, ln) ^ te<1, 1>(s2, ln) ^ te<2, 2>(s3, ln) ^ te<3, 3>(s0, ln) ^ k1.y;
-    g.c2 = te<0, 0>(s2, ln) ^ te<1, 1>(s3, ln) ^ te<2, 2>(s0, ln) ^ te<3, 3>(s1, ln) ^ k1.z;
-    g.c3 = te<0, 0>(s3, ln) ^ te<1, 1>(s0, ln) ^ te<2, 2>(s1, ln) ^ te<3, 3>(s2, ln) ^ k1.w;
-    g.q0 = te<1, 1>(g.c1, ln) ^ te<2, 2>(g.c2, ln) ^ te<3, 3>(g.c3, ln) ^ k2.x;
-    g.q1 = te<0, 0>(g.c1, ln) ^ te<1, 1>(g.c2, ln) ^ te<2, 2>(g.c3, ln) ^ k2.y;
-    g.q2 = te<0, 0>(g.c2, ln) ^ te<1, 1>(g.c3, ln) ^ te<3, 3>(g.c1, ln) ^ k2.z;
-    g.q3 = te<0, 0>(g.c3, ln) ^ te<2, 2>(g.c1, ln) ^ te<3, 3>(g.c2, ln) ^ k2.w;
-    return g;
-}
-
-// Keystream of NB blocks of one group, L[b] = the blocks' low counter bytes.
-template <int NR, int NB, class RK>
-__device__ __forceinline__ void encrypt_group(uint32_t (&s)[NB][4], const uint32_t (&L)[NB], const Group &g,
-                                              const Lanes &ln, const RK &rk)
-{
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        const uint32_t r10 = g.p0 ^ te<3, 0>(L[b] ^ g.k15, ln);  // Te3[byte 15]
-        s[b][0] = g.q0 ^ te<0, 0>(r10, ln);
-        s[b][1] = g.q1 ^ te<3, 3>(r10, ln);
-        s[b][2] = g.q2 ^ te<2, 2>(r10, ln);
-        s[b][3] = g.q3 ^ te<1, 1>(r10, ln);
-    }
-    rounds<3, NR, NB>(s, ln, rk);
-}
-
-// The same split for runs over many groups, so that the two halves are each
-// computed once and a block's state after round 2 is one xor of four words:
+// is Q_c ^ (one lookup) with Q0..Q3 fixed for the group.  The two halves are
+// each computed once for a whole run, and a block's state after round 2 is
+// one xor of four words:
 //   round-2 state = group_round2(upper 15 counter bytes) ^ lane_round2(L)
 // group_round2 holds what byte 15 does not touch (Q0..Q3 above).  lane_round2
 // is byte 15's part: through P0 it also depends on counter bytes 0, 5 and 10,
@@ -222,12 +180,19 @@ struct CounterWords {
     }
 };
 
+// 27 lookups.
 template <class RK>
-__device__ __forceinline__ uint4 group_round2(const CounterWords &ctr, const Lanes &ln,
-                                              const RK &rk)
+__device__ __forceinline__ uint4 group_round2(const CounterWords &ctr, const Lanes &ln, const RK &rk)
 {
-    const Group g = group_consts(ctr.w, ln, rk);
-    return make_uint4(g.q0, g.q1, g.q2, g.q3);
+    const uint4 k0 = rk.get(0), k1 = rk.get(1), k2 = rk.get(2);
+    const uint32_t s0 = ctr.w[0] ^ k0.x, s1 = ctr.w[1] ^ k0.y, s2 = ctr.w[2] ^ k0.z, s3 = ctr.w[3] ^ k0.w;
+    const uint32_t c1 = te<0, 0>(s1, ln) ^ te<1, 1>(s2, ln) ^ te<2, 2>(s3, ln) ^ te<3, 3>(s0, ln) ^ k1.y;
+    const uint32_t c2 = te<0, 0>(s2, ln) ^ te<1, 1>(s3, ln) ^ te<2, 2>(s0, ln) ^ te<3, 3>(s1, ln) ^ k1.z;
+    const uint32_t c3 = te<0, 0>(s3, ln) ^ te<1, 1>(s0, ln) ^ te<2, 2>(s1, ln) ^ te<3, 3>(s2, ln) ^ k1.w;
+    return make_uint4(te<1, 1>(c1, ln) ^ te<2, 2>(c2, ln) ^ te<3, 3>(c3, ln) ^ k2.x,
+                      te<0, 0>(c1, ln) ^ te<1, 1>(c2, ln) ^ te<2, 2>(c3, ln) ^ k2.y,
+                      te<0, 0>(c2, ln) ^ te<1, 1>(c3, ln) ^ te<3, 3>(c1, ln) ^ k2.z,
+                      te<0, 0>(c3, ln) ^ te<2, 2>(c1, ln) ^ te<3, 3>(c2, ln) ^ k2.w);
 }
 
 // The part of lane_round2 that all lanes share: round 1's column 0 without

@@ -9,7 +9,7 @@
 // left by 8r bits.  The final round has no MixColumns and takes S(x) out of
 // the byte of Te_r that holds the plain S(x).
 //
-// Layout (128 KiB per CTA): entry e of Te_r, copy for lane l, is the word at
+// Layout (32 KiB a table, 128 KiB per CTA): entry e of Te_r, copy for lane l, is the word at
 // byte r*32768 + e*128 + l*4.  Every lane reads its own copy, so the 32 lanes
 // of a warp always hit 32 distinct banks (conflict-free).  The byte offset of
 // a lookup is 128 * (state byte K) + 4 * lane: one four-way byte dot product
@@ -20,13 +20,20 @@
 // permutes did.  The pipe that bounds the rounds stays the shared-memory
 // lookups, 32 lanes a clock.  One 8 MiB AES-128 buffer: 10.99 us with byte
 // permutes, 10.68 us so; 256 MiB 243.5 and 240.1 us.
+//
+// With TABLES == 2 only Te0 and Te1 are kept: Te2 and Te3 are their halves
+// swapped, and a column's two lookups there are swapped together by one more
+// permute.  That halves the fill and the shared memory, for 8 more logic
+// operations a round.
 #pragma once
 #include <stdint.h>
 
 namespace aestt {
 
 constexpr uint32_t kOneTable = 32768;
-constexpr uint32_t kTableBytes = 4 * kOneTable;
+template <int TABLES>
+constexpr uint32_t kTableBytesOf = TABLES * kOneTable;
+constexpr uint32_t kTableBytes = kTableBytesOf<4>;
 
 // The shared address of the calling lane's copy of entry 0 of Te0; made after
 // the barrier that follows fill_tables.  The address rides in the dot
@@ -34,31 +41,38 @@ constexpr uint32_t kTableBytes = 4 * kOneTable;
 // nothing else: left to the compiler, some instantiations added the tables'
 // base to every offset (131 more instructions per 32 AES-128 blocks in the
 // batch kernel, 64 MiB 84.2 us instead of 76.3).
-struct Lanes {
+template <int TABLES>
+struct LanesOf {
+    static constexpr int kTables = TABLES;
     uint32_t a;
-    __device__ __forceinline__ explicit Lanes(const uint8_t *tables)
+    __device__ __forceinline__ explicit LanesOf(const uint8_t *tables)
         : a((uint32_t)__cvta_generic_to_shared(tables) + (threadIdx.x & 31u) * 4u)
     {
         // every lookup depends on this value and so stays behind the barrier
         asm volatile("" : "+r"(a)::"memory");
     }
 };
+using Lanes = LanesOf<4>;
+
+__device__ __forceinline__ uint32_t swap_halves(uint32_t v) { return __byte_perm(v, 0, 0x1032); }
 
 // Te_T[byte K of x].
-template <int T, int K>
-__device__ __forceinline__ uint32_t te(uint32_t x, const Lanes &ln)
+template <int T, int K, class LN>
+__device__ __forceinline__ uint32_t te(uint32_t x, const LN &ln)
 {
+    constexpr int kAt = LN::kTables == 4 ? T : T & 1;
     uint32_t v;
-    asm("ld.shared.u32 %0, [%1 + %2];" : "=r"(v) : "r"(__dp4a(x, 0x80u << (8 * K), ln.a)), "n"(T * kOneTable));
-    return v;
+    asm("ld.shared.u32 %0, [%1 + %2];" : "=r"(v) : "r"(__dp4a(x, 0x80u << (8 * K), ln.a)), "n"(kAt * kOneTable));
+    return kAt == T ? v : swap_halves(v);
 }
 
 // Fill the replicated tables from Te0 (256 words in global memory).  Must be
 // followed by __syncthreads() before the first lookup.  Te0 is first staged
 // in a 1 KiB shared array (one global round trip for the whole CTA); then
 // each thread takes an entry's 16-byte chunk of four lane copies and writes
-// it to the four tables, consecutive threads to consecutive chunks (no bank
+// it to every table, consecutive threads to consecutive chunks (no bank
 // conflicts).  The fill is most of a short launch's fixed cost.
+template <int TABLES = 4>
 __device__ __forceinline__ void fill_tables(uint8_t *smem, const uint32_t *__restrict__ te0)
 {
     __shared__ uint32_t s_te0[256];
@@ -69,7 +83,7 @@ __device__ __forceinline__ void fill_tables(uint8_t *smem, const uint32_t *__res
     for (uint32_t q = threadIdx.x; q < kOneTable / 16; q += blockDim.x) {
         const uint32_t v = s_te0[q >> 3];  // entry e = q / 8
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < TABLES; ++t) {
             const uint32_t val = t ? __funnelshift_l(v, v, 8 * t) : v;
             *reinterpret_cast<uint4 *>(smem + t * kOneTable + q * 16u) = make_uint4(val, val, val, val);
         }
@@ -111,46 +125,43 @@ struct RkRegs {
     __device__ __forceinline__ uint4 get(int r) const { return w[r]; }
 };
 
-// Rounds R0..NR-1 (full) and the final round NR on NB blocks held as
-// s[b][0..3] (little-endian column words), in place.  The state passed in is
-// the output of round R0 - 1.
-template <int R0, int NR, int NB, class RK>
-__device__ __forceinline__ void rounds(uint32_t (&s)[NB][4], const Lanes &ln,
-                                       const RK &rk)
+// Rounds R0..NR-1 (full) and the final round NR on one block held as s[0..3]
+// (little-endian column words), in place.  The state passed in is the output
+// of round R0 - 1.
+template <int R0, int NR, class LN, class RK>
+__device__ __forceinline__ void rounds(uint32_t (&s)[4], const LN &ln, const RK &rk)
 {
+    constexpr bool kFour = LN::kTables == 4;
 #pragma unroll
     for (int r = R0; r < NR; ++r) {
         const uint4 k = rk.get(r);
         const uint32_t kk[4] = {k.x, k.y, k.z, k.w};
+        const uint32_t a[4] = {s[0], s[1], s[2], s[3]};
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            const uint32_t a[4] = {s[b][0], s[b][1], s[b][2], s[b][3]};
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                s[b][c] = te<0, 0>(a[c], ln) ^ te<1, 1>(a[(c + 1) & 3], ln) ^
-                          te<2, 2>(a[(c + 2) & 3], ln) ^ te<3, 3>(a[(c + 3) & 3], ln) ^ kk[c];
+        for (int c = 0; c < 4; ++c) {
+            if constexpr (kFour)
+                s[c] = te<0, 0>(a[c], ln) ^ te<1, 1>(a[(c + 1) & 3], ln) ^ te<2, 2>(a[(c + 2) & 3], ln) ^
+                       te<3, 3>(a[(c + 3) & 3], ln) ^ kk[c];
+            else
+                s[c] = te<0, 0>(a[c], ln) ^ te<1, 1>(a[(c + 1) & 3], ln) ^ kk[c] ^
+                       swap_halves(te<0, 2>(a[(c + 2) & 3], ln) ^ te<1, 3>(a[(c + 3) & 3], ln));
         }
     }
-    {
-        // Final round: byte r of output column c is S(s_{c+r}.b_r), taken
-        // from the byte of a T-table entry that holds the plain S-box value:
-        // Te2 byte 0, Te3 byte 1, Te0 byte 2, Te1 byte 3.
-        const uint4 k = rk.get(NR);
-        const uint32_t kk[4] = {k.x, k.y, k.z, k.w};
+    // Final round: byte r of output column c is S(s_{c+r}.b_r), taken from a
+    // byte of a T-table entry that holds the plain S-box value: Te2 byte 0,
+    // Te3 byte 1, Te0 byte 2 and Te1 byte 3, which need no moving, or byte 1
+    // of Te0.
+    const uint4 k = rk.get(NR);
+    const uint32_t kk[4] = {k.x, k.y, k.z, k.w};
+    const uint32_t a[4] = {s[0], s[1], s[2], s[3]};
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            const uint32_t a[4] = {s[b][0], s[b][1], s[b][2], s[b][3]};
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const uint32_t x0 = te<2, 0>(a[c], ln);            // byte 0
-                const uint32_t x1 = te<3, 1>(a[(c + 1) & 3], ln);  // byte 1
-                const uint32_t x2 = te<0, 2>(a[(c + 2) & 3], ln);  // byte 2
-                const uint32_t x3 = te<1, 3>(a[(c + 3) & 3], ln);  // byte 3
-                const uint32_t lo = __byte_perm(x0, x1, 0x3250);
-                const uint32_t hi = __byte_perm(x2, x3, 0x7210);
-                s[b][c] = __byte_perm(lo, hi, 0x7610) ^ kk[c];
-            }
-        }
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t a0 = a[c], a1 = a[(c + 1) & 3], a2 = a[(c + 2) & 3], a3 = a[(c + 3) & 3];
+        const uint32_t lo = kFour ? __byte_perm(te<2, 0>(a0, ln), te<3, 1>(a1, ln), 0x3250)
+                                  : __byte_perm(te<0, 0>(a0, ln), te<0, 1>(a1, ln), 0x3251);
+        const uint32_t hi = kFour ? __byte_perm(te<0, 2>(a2, ln), te<1, 3>(a3, ln), 0x7210)
+                                  : __byte_perm(te<0, 2>(a2, ln), te<0, 3>(a3, ln), 0x5110);
+        s[c] = __byte_perm(lo, hi, 0x7610) ^ kk[c];
     }
 }
 
@@ -181,8 +192,8 @@ struct CounterWords {
 };
 
 // 27 lookups.
-template <class RK>
-__device__ __forceinline__ uint4 group_round2(const CounterWords &ctr, const Lanes &ln, const RK &rk)
+template <class LN, class RK>
+__device__ __forceinline__ uint4 group_round2(const CounterWords &ctr, const LN &ln, const RK &rk)
 {
     const uint4 k0 = rk.get(0), k1 = rk.get(1), k2 = rk.get(2);
     const uint32_t s0 = ctr.w[0] ^ k0.x, s1 = ctr.w[1] ^ k0.y, s2 = ctr.w[2] ^ k0.z, s3 = ctr.w[3] ^ k0.w;
@@ -197,15 +208,15 @@ __device__ __forceinline__ uint4 group_round2(const CounterWords &ctr, const Lan
 
 // The part of lane_round2 that all lanes share: round 1's column 0 without
 // byte 15's lookup.
-template <class RK>
-__device__ __forceinline__ uint32_t column0_round1(const CounterWords &ctr, const Lanes &ln, const RK &rk)
+template <class LN, class RK>
+__device__ __forceinline__ uint32_t column0_round1(const CounterWords &ctr, const LN &ln, const RK &rk)
 {
     const uint4 k0 = rk.get(0), k1 = rk.get(1);
     return te<0, 0>(ctr.w[0] ^ k0.x, ln) ^ te<1, 1>(ctr.w[1] ^ k0.y, ln) ^ te<2, 2>(ctr.w[2] ^ k0.z, ln) ^ k1.x;
 }
 
-template <class RK>
-__device__ __forceinline__ uint4 lane_round2(uint32_t column0, uint32_t L, const Lanes &ln, const RK &rk)
+template <class LN, class RK>
+__device__ __forceinline__ uint4 lane_round2(uint32_t column0, uint32_t L, const LN &ln, const RK &rk)
 {
     const uint32_t r10 = column0 ^ te<3, 0>(L ^ (rk.get(0).w >> 24), ln);
     return make_uint4(te<0, 0>(r10, ln), te<3, 3>(r10, ln), te<2, 2>(r10, ln), te<1, 1>(r10, ln));

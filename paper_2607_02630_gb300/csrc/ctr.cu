@@ -7,7 +7,7 @@
 //              instruction of the warp moves 512 contiguous bytes); rounds from
 //              T-tables in bank-replicated shared memory with counter-mode
 //              caching of rounds 1-2 (aes_ttable.cuh).  About 136 KiB of shared
-//              memory, one CTA per SM.
+//              memory, or 72 KiB with two tables; one CTA per SM.
 //   bitsliced: each warp owns 1024 consecutive blocks; lane l holds blocks
 //              base + l + 32k (k = 0..31) as 128 bit planes (aes_bitslice.cuh),
 //              so loads/stores are again 512 contiguous bytes per instruction.
@@ -25,7 +25,8 @@ using aesrt::CtrParams;
 
 // Counter groups whose round-2 constants a CTA holds at once (16 bytes each).
 constexpr uint32_t kGroupsPerPass = 512;
-constexpr size_t kCtrSmem = aestt::kTableBytes + kGroupsPerPass * sizeof(uint4);
+template <int TABLES>
+constexpr size_t kCtrSmem = aestt::kTableBytesOf<TABLES> + kGroupsPerPass * sizeof(uint4);
 
 // Single-buffer T-table kernel, bound by shared-memory wavefronts: per
 // 32-block chunk the 16 * (NR - 2) lookups of rounds 3..NR, one broadcast
@@ -50,15 +51,19 @@ constexpr size_t kCtrSmem = aestt::kTableBytes + kGroupsPerPass * sizeof(uint4);
 // chunk at the measured rate and 2070 MHz are 228 us).  Back to back on a
 // stream, with the set-up overlapped (launch_overlapped): 1 MiB 3.5 us, 8 MiB
 // 10.2 us.
-template <int NR>
-__global__ void __launch_bounds__(1024, 1) ctr_ttable_kernel(const __grid_constant__ CtrParams p)
+//
+// With two tables (64 KiB) and 512 threads, two CTAs fit an SM, so the next
+// launch's CTAs set up beside the running ones instead of after them.
+template <int NR, int TABLES>
+__global__ void __launch_bounds__(TABLES == 2 ? 512 : 1024, TABLES == 2 ? 2 : 1)
+    ctr_ttable_kernel(const __grid_constant__ CtrParams p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
-    uint4 *s_group = reinterpret_cast<uint4 *>(smem + aestt::kTableBytes);
+    uint4 *s_group = reinterpret_cast<uint4 *>(smem + aestt::kTableBytesOf<TABLES>);
     aesdev::let_next_launch_start();
-    aestt::fill_tables(smem, p.te0);
+    aestt::fill_tables<TABLES>(smem, p.te0);
     __syncthreads();
-    const aestt::Lanes ln(smem);
+    const aestt::LanesOf<TABLES> ln(smem);
     const aestt::RkConst rk{p.rk};
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const uint64_t nblocks = (p.len + 15) >> 4, nfull = p.len >> 4;
@@ -101,14 +106,13 @@ __global__ void __launch_bounds__(1024, 1) ctr_ttable_kernel(const __grid_consta
                 mine_for = tag;
             }
             const uint4 group = s_group[g - ga];
-            uint32_t s[1][4] = {{group.x ^ mine.x, group.y ^ mine.y, group.z ^ mine.z, group.w ^ mine.w}};
-            aestt::rounds<3, NR, 1>(s, ln, rk);
+            uint32_t s[4] = {group.x ^ mine.x, group.y ^ mine.y, group.z ^ mine.z, group.w ^ mine.w};
+            aestt::rounds<3, NR>(s, ln, rk);
             if (j < nfull)
-                aesdev::st_stream(p.out + j, make_uint4(pt.x ^ s[0][0], pt.y ^ s[0][1], pt.z ^ s[0][2],
-                                                        pt.w ^ s[0][3]));
+                aesdev::st_stream(p.out + j, make_uint4(pt.x ^ s[0], pt.y ^ s[1], pt.z ^ s[2], pt.w ^ s[3]));
             else if (j == nfull && (p.len & 15))  // the final partial block
                 aesdev::xor_tail(reinterpret_cast<const uint8_t *>(p.in + j), reinterpret_cast<uint8_t *>(p.out + j),
-                                 s[0][0], s[0][1], s[0][2], s[0][3], (uint32_t)(p.len & 15));
+                                 s[0], s[1], s[2], s[3], (uint32_t)(p.len & 15));
             j = jn;
         }
         ka = kb;
@@ -128,6 +132,30 @@ __global__ void __launch_bounds__(128) ctr_bitslice_kernel(const __grid_constant
                          aesbs::MaskKeys{reinterpret_cast<const uint4 *>(bsk)});
 }
 
+template <int NR>
+cudaError_t set_tt_attr()
+{
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t e = cudaFuncSetAttribute(ctr_ttable_kernel<NR, 4>, attr, (int)kCtrSmem<4>);
+    return e ? e : cudaFuncSetAttribute(ctr_ttable_kernel<NR, 2>, attr, (int)kCtrSmem<2>);
+}
+
+// Two tables from 2 to 16 MiB, where a launch's set-up counts and the extra
+// logic operations hide behind the lookups; four below (one chunk per warp:
+// the longer chain of a round counts) and above.  Launches in a row, four and
+// two tables: 1 MiB AES-128 3.24 and 3.26 us, AES-256 3.70 and 4.18; 4 MiB
+// 6.30 and 5.65, 8.03 and 7.39; 8 MiB 9.9 and 9.4, 13.2 and 12.75; 32 MiB
+// 32.4 and 32.5; 256 MiB 241.9 and 245.3, 348 and 352.
+bool two_tables(uint64_t len, int threads) { return len >= (2u << 20) && len <= (16u << 20) && threads == 512; }
+
+template <int NR>
+cudaError_t launch_tt(const CtrParams &p, int ctas, int threads, cudaStream_t stream)
+{
+    if (two_tables(p.len, threads))
+        return aesrt::launch_overlapped(ctr_ttable_kernel<NR, 2>, ctas, threads, kCtrSmem<2>, stream, p);
+    return aesrt::launch_overlapped(ctr_ttable_kernel<NR, 4>, ctas, threads, kCtrSmem<4>, stream, p);
+}
+
 }  // namespace
 
 namespace aesrt {
@@ -135,15 +163,14 @@ namespace aesrt {
 cudaError_t ctr_set_attributes()
 {
     cudaError_t e;
-    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if ((e = cudaFuncSetAttribute(ctr_ttable_kernel<10>, attr, (int)kCtrSmem)) ||
-        (e = cudaFuncSetAttribute(ctr_ttable_kernel<12>, attr, (int)kCtrSmem)))
+    if ((e = set_tt_attr<10>()) || (e = set_tt_attr<12>()) || (e = set_tt_attr<14>()))
         return e;
-    return cudaFuncSetAttribute(ctr_ttable_kernel<14>, attr, (int)kCtrSmem);
+    return cudaSuccess;
 }
 
-// Resident CTAs per SM: T-table is bound by its 136 KiB of shared memory
-// (one CTA); bitsliced CTAs of 128 threads are bound by registers.
+// CTAs per SM of one launch: one T-table CTA (it keeps the lookups busy, and
+// four tables fill most of an SM's shared memory); bitsliced CTAs of 128
+// threads are bound by registers.
 int ctr_max_ctas(const CtrShape &s, int nsm)
 {
     if (s.variant == 2)
@@ -187,9 +214,9 @@ cudaError_t launch_ctr(const CtrParams &p, int nr, const CtrShape &s, int nsm, c
         return cudaGetLastError();
     }
     switch (nr) {
-    case 10: return launch_overlapped(ctr_ttable_kernel<10>, ctas, s.threads, kCtrSmem, stream, p);
-    case 12: return launch_overlapped(ctr_ttable_kernel<12>, ctas, s.threads, kCtrSmem, stream, p);
-    case 14: return launch_overlapped(ctr_ttable_kernel<14>, ctas, s.threads, kCtrSmem, stream, p);
+    case 10: return launch_tt<10>(p, ctas, s.threads, stream);
+    case 12: return launch_tt<12>(p, ctas, s.threads, stream);
+    case 14: return launch_tt<14>(p, ctas, s.threads, stream);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -79,16 +79,14 @@ __device__ __forceinline__ void xor_run(const uint4 *__restrict__ in, uint4 *__r
             if (in_ >= lo && in_ < hi)
                 next = aesdev::ld_stream(ip + cn * 32u);
             const uint4 group = s_group[(m0 + c) >> 3];
-            uint32_t s[1][4] = {{group.x ^ mine.x, group.y ^ mine.y, group.z ^ mine.z, group.w ^ mine.w}};
-            aestt::rounds<3, NR, 1>(s, ln, rk);
+            uint32_t s[4] = {group.x ^ mine.x, group.y ^ mine.y, group.z ^ mine.z, group.w ^ mine.w};
+            aestt::rounds<3, NR>(s, ln, rk);
             const uint32_t i = c * 32u + lane;
             if (i >= lo && i < hi)
-                aesdev::st_stream(op + c * 32u, make_uint4(pt.x ^ s[0][0], pt.y ^ s[0][1], pt.z ^ s[0][2],
-                                                           pt.w ^ s[0][3]));
+                aesdev::st_stream(op + c * 32u, make_uint4(pt.x ^ s[0], pt.y ^ s[1], pt.z ^ s[2], pt.w ^ s[3]));
             else if (i == partial)
                 aesdev::xor_tail(reinterpret_cast<const uint8_t *>(ip + c * 32u),
-                                 reinterpret_cast<uint8_t *>(op + c * 32u), s[0][0], s[0][1], s[0][2], s[0][3],
-                                 tail);
+                                 reinterpret_cast<uint8_t *>(op + c * 32u), s[0], s[1], s[2], s[3], tail);
         }
     }
 }

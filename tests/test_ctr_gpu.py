@@ -261,3 +261,40 @@ def test_chunk_run_edges(cuda, aes, ncpu, threads, ctas, bits):
             data = W.random_bytes(g, n)
             got = gpu_ctr(cuda, aes, ctx, iv, data, variant=1, threads=threads, blocks_per_thread=1, ctas=ctas)
             np.testing.assert_array_equal(got, oracle.ctr_mt(key, bits, iv, data, ncpu), err_msg=f"n={n} low={low}")
+
+
+@pytest.mark.parametrize("bits", [128, 192, 256])
+@pytest.mark.parametrize("n", [(2 << 20) - 1, 2 << 20, (3 << 20) + 7, 16 << 20, (16 << 20) + 1])
+def test_table_count_edges(cuda, aes, ncpu, bits, n):
+    """Messages around the sizes between which the kernel keeps two tables
+    instead of four, with a byte carry into the counter's upper half."""
+    g = W.rng(3700 + bits + n % 1000)
+    key = W.random_bytes(g, bits // 8)
+    ctx = aes.Context(key.tobytes(), bits)
+    iv = iv_with_low(g, "low64")
+    data = W.random_bytes(g, n)
+    np.testing.assert_array_equal(gpu_ctr(cuda, aes, ctx, iv, data), oracle.ctr_mt(key, bits, iv, data, ncpu))
+
+
+@pytest.mark.parametrize("n", [4096, 61453, 1 << 20, (5 << 20) + 3, 40 << 20])
+def test_dependent_launches_in_a_row(cuda, aes, n):
+    """Launches whose set-up overlaps the launch before: each one's input is
+    the previous one's output, other kernels and copies stand between some of
+    them, and nothing waits until the end."""
+    g = W.rng(3800 + n % 1000)
+    ctxs = [aes.Context(W.random_bytes(g, b // 8).tobytes(), b) for b in (128, 256, 192)]
+    ivs = [W.random_bytes(g, 16).tobytes() for _ in ctxs]
+    src = to_dev(cuda, W.random_bytes(g, n))
+    a, b = src.clone(), cuda.empty_like(src)
+    for rep in range(3):
+        for c, iv in zip(ctxs, ivs):          # encrypt with each key in turn, a -> b -> a
+            aes.ctr(c, iv, a, b, n)
+            a.copy_(b)
+        for c, iv in reversed(list(zip(ctxs, ivs))):  # and decrypt in reverse
+            aes.ctr(c, iv, a, b, n)
+            aes.ctr(c, iv, b, b, n)           # undo and redo in place
+            aes.batch([(c, iv, b.data_ptr(), b.data_ptr(), n)])
+            a.copy_(b)
+            b.zero_()
+    cuda.cuda.synchronize()
+    np.testing.assert_array_equal(to_host(a), to_host(src))

@@ -3,8 +3,7 @@
 Workload (the batched varlen case): 4096 requests, each with its own random
 key (AES-128 / AES-256, 50/50) and IV, lengths log-uniform on [1 KiB, 8 MiB],
 25% with a 1..15-byte tail; about 3.8 GB of payload per step.  A step is one
-launch of the persistent batch kernel over all 4096 requests (a CUDA-graph
-plan: counter reset + kernel).  Inputs (3.8 GB) are far larger than L2
+launch of the batch kernel over all 4096 requests (a prepared plan).  Inputs (3.8 GB) are far larger than L2
 (129 MB), so no L2 flush is needed between steps.
 
 Also reported: the same requests as 4096 single-buffer launches (per-call),
@@ -850,7 +849,7 @@ def main():
     reqs = [(ctxs[i], w.ivs[i].tobytes(), src.data_ptr() + int(w.offsets[i]),
              dst.data_ptr() + int(w.offsets[i]), int(w.lengths[i])) for i in range(w.n)]
     # the device's rates behind the roofline, then the batch autotuner on
-    # these very requests (every candidate shape timed as a graph plan); the
+    # these very requests (every candidate shape timed as a plan); the
     # plan below uses the shape it picks
     rates = measured_rates(A)
     if not args.no_extras:
@@ -935,13 +934,12 @@ def main():
                        "global_batch": args.requests * ws, "seq_len": None,
                        "parallelism": f"replicas{ws}", "step_bytes": step_bytes,
                        "l2": "no flush: 3.8 GB of inputs per step, far above the 129 MB L2",
-                       "launch": "aes_batch_plan_launch (CUDA graph: counter reset + persistent kernel)",
+                       "launch": "aes_batch_plan_launch (one kernel launch)",
                        "tuned_shape": tuned,
                        "tuner": ("fixed by --batch-shape" if args.batch_shape else
-                                 "aes_batch_autotune on these requests before the timed region: 30 shapes "
-                                 "(T-table CTAs of 256/512/1024 threads x 1/2/4 blocks per lane x tiles of "
-                                 "1024/2048/4096 blocks, and the bitsliced kernel x the 3 tiles), median of 5 "
-                                 "graph launches each")},
+                                 "aes_batch_autotune on these requests before the timed region: 12 shapes "
+                                 "(T-table CTAs of 256/512/1024 threads and the bitsliced kernel x largest "
+                                 "tiles of 1024/2048/4096 blocks), median of 5 plan launches each")},
             "roofline": roofline,
             "cpu_baseline": cpu,
             "e2e": e2e,

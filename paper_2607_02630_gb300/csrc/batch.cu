@@ -1,8 +1,8 @@
 // batch.cu -- many independent AES-CTR requests in one launch.
 //
 // Work is measured in shared-memory wavefronts, the unit of the kernel's
-// bound: a 32-block chunk (tile.cuh) of a request with Nr rounds costs
-// chunk_cost(Nr) of them.  The requests' chunks, one request after the other,
+// bound: a 32-block chunk (tile.cuh) of a request with Nr rounds costs about
+// 16 (Nr - 2) + 9 of them.  The requests' chunks, one request after the other,
 // are one line of cost; CTA c of G (one per SM) owns the c-th of G equal
 // pieces of it, so every SM gets the same number of lookups whatever the mix
 // of lengths and key sizes, and neither a table of tiles nor a counter in
@@ -18,7 +18,7 @@
 // bound, serves lookups only; larger CTAs stage it in each warp's slice of
 // shared memory (one broadcast wavefront per round).
 //
-// The bitsliced kernel takes the same pieces and tiles, 1024 blocks at a time,
+// The bitsliced kernel cuts its work the same way, in passes of 1024 blocks,
 // as the autotuner's alternative to the T-tables.
 //
 // With a tile order (a test aid) the line is cut into equal tiles instead,
@@ -48,19 +48,37 @@ struct TileOrder {
     uint64_t tiles;  // 0: no order, tiles are cut as they are claimed
 };
 
-// Shared-memory wavefronts of one 32-block chunk: 16 lookups in each of the
-// NR - 2 rounds that are not cached, and about 9 for the payload and the
-// group constants.
-__host__ __device__ constexpr uint32_t chunk_cost(uint32_t nr) { return 16u * (nr - 2u) + 9u; }
-// The smallest tile: one AES-128 chunk.
-constexpr uint64_t kMinTileCost = chunk_cost(10);
+// A request's work is cut in units: chunks for the T-table kernel, passes of 32
+// chunks (1024 blocks) for the bitsliced one, which spends a whole pass on any
+// part of it.  A chunk costs its shared-memory wavefronts: 16 lookups in each
+// of the NR - 2 rounds that are not cached, and about 9 for the payload and
+// the group constants.  A pass costs its rounds and, about as much as 5 of
+// them, the transposes and the payload (323 and 254 GB/s at 10 and 14 rounds
+// on a 256 MiB buffer).
+struct TtUnit {
+    static constexpr uint32_t kChunks = 1;
+    __host__ __device__ static constexpr uint32_t cost(uint32_t nr) { return 16u * (nr - 2u) + 9u; }
+    static __device__ __forceinline__ uint32_t run(uint64_t iv_lo, uint64_t k0, uint64_t nk)
+    {
+        return aestile::run_chunks(iv_lo, k0, nk);
+    }
+};
+struct BsUnit {
+    static constexpr uint32_t kChunks = 32;
+    __host__ __device__ static constexpr uint32_t cost(uint32_t nr) { return 16u * (nr + 5u); }
+    static __device__ __forceinline__ uint32_t run(uint64_t, uint64_t, uint64_t nk)
+    {
+        return nk < kChunks ? (uint32_t)nk : kChunks;
+    }
+};
 
-__device__ __forceinline__ uint64_t ceil_chunks(uint64_t cost, uint32_t nr)
+template <class UNIT>
+__device__ __forceinline__ uint64_t ceil_units(uint64_t cost, uint32_t nr)
 {
     switch (nr) {
-    case 10: return (cost + chunk_cost(10) - 1) / chunk_cost(10);
-    case 12: return (cost + chunk_cost(12) - 1) / chunk_cost(12);
-    default: return (cost + chunk_cost(14) - 1) / chunk_cost(14);
+    case 10: return (cost + UNIT::cost(10) - 1) / UNIT::cost(10);
+    case 12: return (cost + UNIT::cost(12) - 1) / UNIT::cost(12);
+    default: return (cost + UNIT::cost(14) - 1) / UNIT::cost(14);
     }
 }
 
@@ -120,76 +138,95 @@ __device__ __forceinline__ uint32_t owner_of(const BatchReq *reqs, uint32_t lo, 
     return lo;
 }
 
-// Calls run(request, first chunk, chunks <= kRunChunks) for every piece of
-// work of the calling warp (every lane with the same arguments).  s_pos: the CTA's
-// counter, zeroed before the CTA's last barrier.
-template <class RUN>
-__device__ __forceinline__ void for_each_run(const BatchArgs &p, const BatchReq *reqs, unsigned long long *s_pos,
-                                             RUN &&run)
+// Where a warp stands: what is left of its tile's cost range, and a request
+// at or before it.  Kept in shared memory between runs: held in registers it
+// was spilled around the bitsliced rounds and took registers from the
+// lookups in flight.
+struct WarpState {
+    unsigned long long xa, xb;
+    uint32_t ri, pad;
+};
+
+// The warp's next run: n > 0 chunks from chunk k0 on of request rq (every
+// lane gets the same), or false when the CTA's piece is done.  s_pos: the
+// CTA's counter; st: this warp's state; both zeroed before the CTA's last
+// barrier.
+template <class UNIT>
+__device__ __forceinline__ bool next_run(const BatchArgs &p, const BatchReq *reqs, unsigned long long *s_pos,
+                                         WarpState *st, BatchReq &rq, uint64_t &k0, uint32_t &n)
 {
     const uint32_t lane = threadIdx.x & 31u;
-    const uint64_t units = p.order.tiles ? p.order.tiles : p.total_cost;  // this CTA's piece [u0, u1)
-    const uint64_t q = units / gridDim.x, r = units % gridDim.x;
-    const uint64_t u0 = q * blockIdx.x + (blockIdx.x < r ? blockIdx.x : r);
-    const uint64_t size = q + (blockIdx.x < r ? 1 : 0);
-    const uint64_t guide = blockDim.x >> 5;
-    uint32_t ri = 0;
-    bool near = false;
+    __syncwarp();  // lane 0's last store to the state
+    uint64_t xa = st->xa, xb = st->xb;
+    uint32_t ri = st->ri;
+    __syncwarp();  // before lane 0 writes the next
     for (;;) {
-        unsigned long long at = 0, take = 1;
-        if (lane == 0) {
-            if (!p.order.tiles) {
-                const unsigned long long cur = *(volatile unsigned long long *)s_pos;
-                take = cur < size ? (size - cur) / guide : 0;
-                take = take < kMinTileCost ? kMinTileCost : take > p.tile_cost ? p.tile_cost : take;
+        bool near = true;  // the request is probably the last one or one of the next
+        if (xa >= xb) {    // claim a tile of this CTA's piece [u0, u0 + size)
+            const uint64_t units = p.order.tiles ? p.order.tiles : p.total_cost;
+            const uint64_t q = units / gridDim.x, r = units % gridDim.x;
+            const uint64_t u0 = q * blockIdx.x + (blockIdx.x < r ? blockIdx.x : r);
+            const uint64_t size = q + (blockIdx.x < r ? 1 : 0);
+            unsigned long long at = 0, take = 1;
+            if (lane == 0) {
+                if (!p.order.tiles) {
+                    const unsigned long long cur = *(volatile unsigned long long *)s_pos;
+                    take = cur < size ? (size - cur) / (blockDim.x >> 5) : 0;
+                    take = take < UNIT::cost(10) ? UNIT::cost(10) : take > p.tile_cost ? p.tile_cost : take;
+                }
+                at = atomicAdd(s_pos, take);
             }
-            at = atomicAdd(s_pos, take);
-        }
-        at = __shfl_sync(0xffffffffu, at, 0);
-        take = __shfl_sync(0xffffffffu, take, 0);
-        if (at >= size)
-            break;
-        uint64_t xa, xb;  // the tile's cost range
-        if (p.order.tiles) {
-            const uint64_t t = (p.order.a * (u0 + at) + p.order.b) % p.order.tiles;
-            xa = t * p.tile_cost;
-            xb = xa + p.tile_cost < p.total_cost ? xa + p.tile_cost : p.total_cost;
-            ri = 0;
-        } else {
-            xa = u0 + at;
-            xb = u0 + (at + take < size ? at + take : size);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            take = __shfl_sync(0xffffffffu, take, 0);
+            if (at >= size)
+                return false;
+            if (p.order.tiles) {
+                const uint64_t t = (p.order.a * (u0 + at) + p.order.b) % p.order.tiles;
+                xa = t * p.tile_cost;
+                xb = xa + p.tile_cost < p.total_cost ? xa + p.tile_cost : p.total_cost;
+                ri = 0;
+                near = false;
+            } else {
+                near = xb != 0;  // the first tile may lie anywhere
+                xa = u0 + at;
+                xb = u0 + (at + take < size ? at + take : size);
+            }
         }
         ri = owner_of(reqs, ri, p.n, xa, near);
-        near = !p.order.tiles;  // later tiles lie further along
-        for (uint32_t i = ri; i < p.n; ++i) {
-            const BatchReq rq = reqs[i];
-            if (rq.cost_begin >= xb)
-                break;
-            // chunk c belongs to the tile that holds its first cost unit
-            const uint64_t nb = (rq.len + 15) >> 4, v0 = rq.iv_lo & 255u, first = aestile::first_chunk(rq.iv_lo);
-            const uint64_t nch = ((v0 + nb - 1) >> 5) - first + 1;
-            const uint64_t ca = xa > rq.cost_begin ? ceil_chunks(xa - rq.cost_begin, rq.nr) : 0;
-            uint64_t cb = ceil_chunks(xb - rq.cost_begin, rq.nr);
-            cb = cb < nch ? cb : nch;
-            for (uint64_t c = ca; c < cb;) {
-                const uint32_t m = aestile::run_chunks(rq.iv_lo, first + c, cb - c);
-                run(rq, first + c, m);
-                c += m;
+        rq = reqs[ri];
+        // a unit belongs to the tile that holds the first of its cost
+        const uint64_t nb = (rq.len + 15) >> 4, v0 = rq.iv_lo & 255u, first = aestile::first_chunk(rq.iv_lo);
+        const uint64_t nch = ((v0 + nb - 1) >> 5) - first + 1;
+        const uint64_t all = (nch + UNIT::kChunks - 1) / UNIT::kChunks;
+        const uint64_t ua = ceil_units<UNIT>(xa - rq.cost_begin, rq.nr);
+        uint64_t ub = ceil_units<UNIT>(xb - rq.cost_begin, rq.nr);
+        ub = ub < all ? ub : all;
+        if (ua < ub) {
+            const uint64_t c = ua * UNIT::kChunks, end = ub * UNIT::kChunks;
+            k0 = first + c;
+            n = UNIT::run(rq.iv_lo, k0, (end < nch ? end : nch) - c);
+            if (lane == 0) {
+                st->xa = rq.cost_begin + (ua + (n + UNIT::kChunks - 1) / UNIT::kChunks) * UNIT::cost(rq.nr);
+                st->xb = xb;
+                st->ri = ri;
             }
+            return true;
         }
+        xa = rq.cost_begin + all * UNIT::cost(rq.nr);  // on to the next request, or past the tile
     }
 }
 
 // The T-table batch kernel, bound by shared-memory wavefronts (95 % of the
-// pipe busy on a 256 MiB AES-128 request, 146 wavefronts a chunk of which 128
-// are lookups of rounds 3..10).  Measured as plans: 4096 requests of 1 KiB to
-// 8 MiB (3.66 GB) 4390 -> 4153 us, 64 requests of 1 to 16 KiB 39 -> 6.4 us
-// (one warp used to take up to 8 groups of a short request in turn), against
-// the kernel with a tile map, a device counter and two blocks per lane.
-// Registers: 384-thread CTAs with 168 a thread are faster on AES-256 alone
-// (4870 against 4957 us for the same lengths) and slower on AES-128 (3459
-// against 3356), as are 448 (5258 and 3401).  MAXT: largest CTA it is launched with; RK_REGS:
-// round keys in registers (else in the warp's slice of shared memory).
+// pipe busy on a 256 MiB AES-128 request).  Measured as plans against the
+// kernel with a tile map, a device counter and two blocks per lane: 4096
+// requests of 1 KiB to 8 MiB (3.66 GB) 4396 -> 4043 us, 512 of them 638 ->
+// 565, 256 of 4 KiB to 1 MiB 111 -> 58, 64 of 1 to 16 KiB 37 -> 5.4 (one warp
+// used to take up to 8 groups of a short request in turn).  Other CTA sizes
+// on the 4096: 1024 threads (keys in shared memory) 4491 us, 256 threads
+// 5148; 384 threads with up to 168 registers were 2 % faster on AES-256
+// alone and 3 % slower on AES-128.  MAXT: largest CTA it is launched with;
+// RK_REGS: round keys in registers (else in the warp's slice of shared
+// memory).
 template <int MAXT, bool RK_REGS, int CAP>
 __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_constant__ BatchParams<CAP> p)
 {
@@ -197,9 +234,12 @@ __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_cons
     __shared__ uint4 s_group[MAXT / 32][aestile::kRunGroups];
     __shared__ uint4 s_rk[RK_REGS ? 1 : MAXT / 32][15];  // round keys of each warp's current request
     __shared__ unsigned long long s_pos;
+    __shared__ WarpState s_state[MAXT / 32];
     aesdev::let_next_launch_start();
     if (threadIdx.x == 0)
         s_pos = 0;
+    if (threadIdx.x < MAXT / 32)
+        s_state[threadIdx.x] = WarpState{0, 0, 0, 0};
     aestt::fill_tables(smem, p.te0);
     __syncthreads();
     aesdev::wait_for_previous_launch();
@@ -213,7 +253,6 @@ __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_cons
             const aestt::RkRegs<NR> rk(rq.rk);
             aestile::xor_run<NR>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, k0, n, w_group, ln, rk);
         } else {
-            __syncwarp();  // every lane is done with the previous keys
             if (lane <= NR)
                 w_rk[lane] = rq.rk[lane];
             __syncwarp();
@@ -221,16 +260,19 @@ __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_cons
             aestile::xor_run<NR>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, k0, n, w_group, ln, rk);
         }
     };
-    for_each_run(p, p.requests(), &s_pos, [&](const BatchReq &rq, uint64_t k0, uint32_t n) {
+    BatchReq rq;
+    uint64_t k0;
+    uint32_t n;
+    while (next_run<TtUnit>(p, p.requests(), &s_pos, &s_state[warp], rq, k0, n)) {
         switch (rq.nr) {
         case 10: xor_with(rq, k0, n, std::integral_constant<int, 10>()); break;
         case 12: xor_with(rq, k0, n, std::integral_constant<int, 12>()); break;
         default: xor_with(rq, k0, n, std::integral_constant<int, 14>()); break;
         }
-    });
+    }
 }
 
-// The bitsliced batch kernel: the same tiles and claims, each run encrypted
+// The bitsliced batch kernel: the same pieces and claims, each run encrypted
 // by one warp 1024 blocks at a time (bs_tile.cuh) with the request's
 // round-key bit planes in the warp's slice of shared memory (rebuilt when the
 // warp moves to a request with another key).
@@ -239,15 +281,21 @@ __global__ void __launch_bounds__(kBsThreads) batch_bitslice_kernel(const __grid
 {
     __shared__ __align__(16) uint32_t s_mask[kBsThreads / 32][15 * 128];
     __shared__ unsigned long long s_pos;
+    __shared__ WarpState s_state[kBsThreads / 32];
     aesdev::let_next_launch_start();
     if (threadIdx.x == 0)
         s_pos = 0;
+    if (threadIdx.x < kBsThreads / 32)
+        s_state[threadIdx.x] = WarpState{0, 0, 0, 0};
     __syncthreads();
     aesdev::wait_for_previous_launch();
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t *mask = s_mask[threadIdx.x >> 5];
     const uint4 *cur = nullptr;  // schedule whose masks are in `mask`
-    for_each_run(p, p.requests(), &s_pos, [&](const BatchReq &rq, uint64_t k0, uint32_t n) {
+    BatchReq rq;
+    uint64_t k0;
+    uint32_t n;
+    while (next_run<BsUnit>(p, p.requests(), &s_pos, &s_state[threadIdx.x >> 5], rq, k0, n)) {
         const uint64_t v0 = rq.iv_lo & 255u, nb = (rq.len + 15) >> 4;
         const uint64_t first = k0 << 5 > v0 ? (k0 << 5) - v0 : 0;
         const uint64_t end = ((k0 + n) << 5) - v0, last = end < nb ? end : nb;
@@ -265,7 +313,7 @@ __global__ void __launch_bounds__(kBsThreads) batch_bitslice_kernel(const __grid
         case 12: aesbs::xor_range<12>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, rk0, first, last, 0, 1, keys); break;
         default: aesbs::xor_range<14>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, rk0, first, last, 0, 1, keys); break;
         }
-    });
+    }
 }
 
 int g_bs_ctas_per_sm = 1;  // resident bitsliced batch CTAs per SM (set with the attributes)
@@ -326,8 +374,20 @@ static TileOrder make_order(uint64_t total, uint32_t seed)
 // What a launch needs to know of its requests.
 struct BatchSums {
     size_t n = 0;  // requests that hold any bytes
-    uint64_t cost = 0, chunks = 0;
+    uint64_t cost = 0, units = 0;
     int64_t bytes = 0;
+    // Appends r: sets its first cost, adds its units.
+    void add(BatchReq &r, int variant)
+    {
+        const uint64_t chunks = chunks_of(r.len, (uint32_t)(r.iv_lo & 255u));
+        const bool bs = variant == AES_VARIANT_BITSLICE;
+        const uint64_t u = bs ? (chunks + BsUnit::kChunks - 1) / BsUnit::kChunks : chunks;
+        r.cost_begin = cost;
+        cost += u * (bs ? BsUnit::cost(r.nr) : TtUnit::cost(r.nr));
+        units += u;
+        bytes += (int64_t)r.len;
+        ++n;
+    }
 };
 
 int validate_batch_shape(BatchShape &s)
@@ -358,7 +418,7 @@ static BatchShape pick_batch_shape(const DeviceState &st, const aes_batch_opts_t
         if (opts->variant && opts->variant != s.variant) {
             // another variant than the tuned one: start from its defaults
             s = opts->variant == AES_VARIANT_BITSLICE ? BatchShape{AES_VARIANT_BITSLICE, kBsThreads, 2048, 0, 1}
-                                                      : BatchShape{opts->variant, 512, 4096, 0, 1};
+                                                      : BatchShape{opts->variant, 512, 7936, 0, 1};
         }
         if (opts->threads)
             s.threads = opts->threads;
@@ -374,7 +434,7 @@ static BatchShape pick_batch_shape(const DeviceState &st, const aes_batch_opts_t
 
 // The non-empty requests of descs[0..n) into out (room for n), their sums into
 // `sum`; the first bad request's status.
-static int fill_reqs(const aes_desc_t *descs, int n, int dev, BatchReq *out, BatchSums &sum)
+static int fill_reqs(const aes_desc_t *descs, int n, int dev, int variant, BatchReq *out, BatchSums &sum)
 {
     PayloadChecks payloads(dev);
     for (int i = 0; i < n; ++i) {
@@ -397,12 +457,9 @@ static int fill_reqs(const aes_desc_t *descs, int n, int dev, BatchReq *out, Bat
         iv_halves(d.iv, &r.iv_hi, &r.iv_lo);
         r.rk = reinterpret_cast<const uint4 *>(d.ctx->d_rk);
         r.nr = (uint32_t)d.ctx->nr;
-        r.cost_begin = sum.cost;
-        const uint64_t chunks = chunks_of(d.len, d.iv[15]);
-        sum.chunks += chunks;
-        sum.cost += chunks * chunk_cost(r.nr);
-        sum.bytes += (int64_t)d.len;
-        out[sum.n++] = r;
+        const size_t at = sum.n;
+        sum.add(r, variant);
+        out[at] = r;
     }
     return AES_OK;
 }
@@ -413,14 +470,16 @@ static int set_args(BatchArgs &p, const BatchSums &sum, const DeviceState &st, c
     p.reqs = nullptr;
     p.n = (uint32_t)sum.n;
     p.total_cost = sum.cost;
-    p.tile_cost = (uint64_t)(s.tile_blocks / 32) * chunk_cost(10);
+    p.tile_cost = s.variant == AES_VARIANT_BITSLICE
+                      ? (uint64_t)std::max(1, s.tile_blocks / 1024) * BsUnit::cost(10)
+                      : (uint64_t)(s.tile_blocks / 32) * TtUnit::cost(10);
     p.te0 = st.te0;
     p.order = make_order((sum.cost + p.tile_cost - 1) / p.tile_cost, seed);
     // as many CTAs as are resident at once (one T-table CTA per SM: its
-    // tables take 128 KiB of shared memory), none without a chunk
+    // tables take 128 KiB of shared memory), none without a unit of work
     const int resident = s.variant == AES_VARIANT_BITSLICE ? st.nsm * g_bs_ctas_per_sm : st.nsm;
     const int ctas = s.ctas > 0 ? std::min(s.ctas, resident) : resident;
-    return (uint64_t)ctas > sum.chunks ? (int)sum.chunks : ctas;
+    return (uint64_t)ctas > sum.units ? (int)sum.units : ctas;
 }
 
 template <int CAP>
@@ -444,7 +503,7 @@ static int launch_in_params(const aes_desc_t *descs, int n, const DeviceState &s
 {
     BatchParams<CAP> p;
     BatchSums sum;
-    const int rc = fill_reqs(descs, n, st.device, p.in_params, sum);
+    const int rc = fill_reqs(descs, n, st.device, s.variant, p.in_params, sum);
     if (rc || !sum.n)
         return rc;
     const int ctas = set_args(p, sum, st, s, seed);
@@ -467,7 +526,7 @@ int batch_by_params(const aes_desc_t *descs, int n, const DeviceState &st, const
         return AES_ENOMEM;
     }
     BatchSums sum;
-    const int rc = fill_reqs(descs, n, st.device, reqs.data(), sum);
+    const int rc = fill_reqs(descs, n, st.device, s.variant, reqs.data(), sum);
     if (rc || !sum.n)
         return rc;
     // equal numbers of requests per launch
@@ -477,12 +536,9 @@ int batch_by_params(const aes_desc_t *descs, int n, const DeviceState &st, const
         const size_t a = sum.n * k / launches, b = sum.n * (k + 1) / launches;
         BatchSums part;
         for (size_t i = a; i < b; ++i) {
-            BatchReq &r = p.in_params[part.n++];
-            r = reqs[i];
-            r.cost_begin = part.cost;
-            const uint64_t chunks = chunks_of(r.len, (uint32_t)(r.iv_lo & 255u));
-            part.chunks += chunks;
-            part.cost += chunks * chunk_cost(r.nr);
+            const size_t at = part.n;
+            part.add(reqs[i], s.variant);
+            p.in_params[at] = reqs[i];
         }
         const int ctas = set_args(p, part, st, s, seed);
         const cudaError_t e = launch_batch(p, ctas, s, stream);
@@ -539,7 +595,7 @@ int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_bat
         return AES_ENOMEM;
     }
     BatchSums sum;
-    if ((rc = fill_reqs(descs, n, st->device, host.data(), sum)) || !sum.n)
+    if ((rc = fill_reqs(descs, n, st->device, s.variant, host.data(), sum)) || !sum.n)
         return rc;
     BatchParams<0> p{};
     const int ctas = set_args(p, sum, *st, s, seed);
@@ -596,7 +652,7 @@ int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
         delete plan;
         return AES_ENOMEM;
     }
-    if ((rc = fill_reqs(descs, n, st->device, host.data(), plan->sum))) {
+    if ((rc = fill_reqs(descs, n, st->device, s.variant, host.data(), plan->sum))) {
         delete plan;
         return rc;
     }

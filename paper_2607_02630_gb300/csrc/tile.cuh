@@ -35,9 +35,9 @@ __device__ __forceinline__ uint32_t run_chunks(uint64_t iv_lo, uint64_t k0, uint
 // bytes one after the other, so that a lane's part of round 2 (lane_round2) is
 // computed once for all groups.  Per 64 chunks that is 27 + 43 wavefronts and
 // one broadcast load per chunk, 2.1 a chunk (1.5 at 128); constants per group
-// and warp and five lookups per block were 8.4.  The next chunk's plaintext is loaded
-// before the current chunk's rounds.  Nothing past len is touched; the final
-// partial block is done bytewise.
+// and warp and five lookups per block were 8.4.  The next chunk's plaintext is
+// loaded before the current chunk's rounds.  Nothing past len is touched; the
+// final partial block is done bytewise.
 template <int NR, class RK>
 __device__ __forceinline__ void xor_run(const uint4 *__restrict__ in, uint4 *__restrict__ out, uint64_t len,
                                         uint64_t iv_hi, uint64_t iv_lo, uint64_t k0, uint32_t n, uint4 *s_group,

@@ -51,9 +51,9 @@ void tune_defaults(DeviceState &st)
     for (int i = 0; i < 3; ++i)
         for (int b = 0; b < kLenBuckets; ++b)
             st.ctr_tuned[i][b] = default_shape();
-    // largest tiles of 2048, 4096 and 7936 blocks: 4096 requests of 1 KiB to
-    // 8 MiB 4167, 4117 and 4097 us, 512 of them 579, 574 and 596 us
-    st.batch_tuned = BatchShape{AES_VARIANT_TTABLE, 512, 4096, 0, 1};
+    // largest tiles of 2048, 4096 and 7936 blocks (a run's most): 4096 requests
+    // of 1 KiB to 8 MiB 4097, 4060 and 4043 us, 512 of them 572, 566 and 565 us
+    st.batch_tuned = BatchShape{AES_VARIANT_TTABLE, 512, 7936, 0, 1};
 }
 
 CtrShape tuned_ctr_shape(const DeviceState &st, size_t len, int nr)

@@ -226,8 +226,8 @@ __device__ __forceinline__ bool next_run(const BatchArgs &p, const BatchReq *req
 // 5148; 384 threads with up to 168 registers were 2 % faster on AES-256
 // alone and 3 % slower on AES-128.  MAXT: largest CTA it is launched with;
 // RK_REGS: round keys in registers (else in the warp's slice of shared
-// memory).
-template <int MAXT, bool RK_REGS, int CAP>
+// memory); HOST: some payload lies in pinned host memory.
+template <int MAXT, bool RK_REGS, int CAP, bool HOST>
 __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_constant__ BatchParams<CAP> p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -249,15 +249,19 @@ __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_cons
     uint4 *w_rk = s_rk[RK_REGS ? 0 : warp];
     auto xor_with = [&](const BatchReq &rq, uint64_t k0, uint32_t n, auto nr) {
         constexpr int NR = decltype(nr)::value;
+        auto go = [&](const auto &rk) {
+            if constexpr (HOST)
+                aestile::xor_run_host<NR>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, k0, n, w_group, ln, rk);
+            else
+                aestile::xor_run<NR>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, k0, n, w_group, ln, rk);
+        };
         if constexpr (RK_REGS) {
-            const aestt::RkRegs<NR> rk(rq.rk);
-            aestile::xor_run<NR>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, k0, n, w_group, ln, rk);
+            go(aestt::RkRegs<NR>(rq.rk));
         } else {
             if (lane <= NR)
                 w_rk[lane] = rq.rk[lane];
             __syncwarp();
-            const aestt::RkShared rk{w_rk};
-            aestile::xor_run<NR>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, k0, n, w_group, ln, rk);
+            go(aestt::RkShared{w_rk});
         }
     };
     BatchReq rq;
@@ -316,6 +320,15 @@ __global__ void __launch_bounds__(kBsThreads) batch_bitslice_kernel(const __grid
     }
 }
 
+template <int MAXT, bool RK_REGS, int CAP>
+cudaError_t set_smem()
+{
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t e = cudaFuncSetAttribute(batch_ttable_kernel<MAXT, RK_REGS, CAP, false>, attr,
+                                               (int)aestt::kTableBytes);
+    return e ? e : cudaFuncSetAttribute(batch_ttable_kernel<MAXT, RK_REGS, CAP, true>, attr, (int)aestt::kTableBytes);
+}
+
 int g_bs_ctas_per_sm = 1;  // resident bitsliced batch CTAs per SM (set with the attributes)
 
 }  // namespace
@@ -325,13 +338,9 @@ namespace aesrt {
 cudaError_t batch_set_attributes()
 {
     cudaError_t e;
-    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    const int smem = (int)aestt::kTableBytes;
-    if ((e = cudaFuncSetAttribute(batch_ttable_kernel<kRegsMaxThreads, true, 0>, attr, smem)) ||
-        (e = cudaFuncSetAttribute(batch_ttable_kernel<kRegsMaxThreads, true, kFewInParams>, attr, smem)) ||
-        (e = cudaFuncSetAttribute(batch_ttable_kernel<kRegsMaxThreads, true, kMostInParams>, attr, smem)) ||
-        (e = cudaFuncSetAttribute(batch_ttable_kernel<1024, false, 0>, attr, smem)) ||
-        (e = cudaFuncSetAttribute(batch_ttable_kernel<1024, false, kMostInParams>, attr, smem)))
+    if ((e = set_smem<kRegsMaxThreads, true, 0>()) || (e = set_smem<kRegsMaxThreads, true, kFewInParams>()) ||
+        (e = set_smem<kRegsMaxThreads, true, kMostInParams>()) || (e = set_smem<1024, false, 0>()) ||
+        (e = set_smem<1024, false, kMostInParams>()))
         return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_bitslice_kernel<0>, kBsThreads, 0)))
@@ -373,7 +382,8 @@ static TileOrder make_order(uint64_t total, uint32_t seed)
 
 // What a launch needs to know of its requests.
 struct BatchSums {
-    size_t n = 0;  // requests that hold any bytes
+    size_t n = 0;       // requests that hold any bytes
+    bool host = false;  // some payload lies in pinned host memory
     uint64_t cost = 0, units = 0;
     int64_t bytes = 0;
     // Appends r: sets its first cost, adds its units.
@@ -447,7 +457,8 @@ static int fill_reqs(const aes_desc_t *descs, int n, int dev, int variant, Batch
             continue;
         const void *din = nullptr;
         void *dout = nullptr;
-        const int rc = payloads.check(d.in, d.out, d.len, &din, &dout);
+        bool host = false;
+        const int rc = payloads.check(d.in, d.out, d.len, &din, &dout, &host);
         if (rc)
             return rc;
         BatchReq r{};
@@ -457,6 +468,7 @@ static int fill_reqs(const aes_desc_t *descs, int n, int dev, int variant, Batch
         iv_halves(d.iv, &r.iv_hi, &r.iv_lo);
         r.rk = reinterpret_cast<const uint4 *>(d.ctx->d_rk);
         r.nr = (uint32_t)d.ctx->nr;
+        sum.host |= host;
         const size_t at = sum.n;
         sum.add(r, variant);
         out[at] = r;
@@ -482,18 +494,26 @@ static int set_args(BatchArgs &p, const BatchSums &sum, const DeviceState &st, c
     return (uint64_t)ctas > sum.units ? (int)sum.units : ctas;
 }
 
+template <int MAXT, bool RK_REGS, int CAP>
+static cudaError_t launch_ttable(const BatchParams<CAP> &p, int ctas, int threads, bool host, cudaStream_t stream)
+{
+    return host ? launch_overlapped(batch_ttable_kernel<MAXT, RK_REGS, CAP, true>, ctas, threads, aestt::kTableBytes,
+                                    stream, p)
+                : launch_overlapped(batch_ttable_kernel<MAXT, RK_REGS, CAP, false>, ctas, threads, aestt::kTableBytes,
+                                    stream, p);
+}
+
 template <int CAP>
-static cudaError_t launch_batch(const BatchParams<CAP> &p, int ctas, const BatchShape &s, cudaStream_t stream)
+static cudaError_t launch_batch(const BatchParams<CAP> &p, int ctas, const BatchShape &s, bool host,
+                                cudaStream_t stream)
 {
     if constexpr (CAP != kFewInParams) {  // the small size exists for the default shape's kernel only
         if (s.variant == AES_VARIANT_BITSLICE)
             return launch_overlapped(batch_bitslice_kernel<CAP>, ctas, kBsThreads, 0, stream, p);
         if (s.threads > kRegsMaxThreads)
-            return launch_overlapped(batch_ttable_kernel<1024, false, CAP>, ctas, s.threads, aestt::kTableBytes,
-                                     stream, p);
+            return launch_ttable<1024, false>(p, ctas, s.threads, host, stream);
     }
-    return launch_overlapped(batch_ttable_kernel<kRegsMaxThreads, true, CAP>, ctas, s.threads, aestt::kTableBytes,
-                             stream, p);
+    return launch_ttable<kRegsMaxThreads, true>(p, ctas, s.threads, host, stream);
 }
 
 // n <= CAP requests in one launch whose parameters hold them.
@@ -507,7 +527,7 @@ static int launch_in_params(const aes_desc_t *descs, int n, const DeviceState &s
     if (rc || !sum.n)
         return rc;
     const int ctas = set_args(p, sum, st, s, seed);
-    const cudaError_t e = launch_batch(p, ctas, s, stream);
+    const cudaError_t e = launch_batch(p, ctas, s, sum.host, stream);
     return e ? cuda_fail(e, "aes_ctr_batch launch") : AES_OK;
 }
 
@@ -535,13 +555,14 @@ int batch_by_params(const aes_desc_t *descs, int n, const DeviceState &st, const
     for (size_t k = 0; k < launches; ++k) {
         const size_t a = sum.n * k / launches, b = sum.n * (k + 1) / launches;
         BatchSums part;
+        part.host = sum.host;
         for (size_t i = a; i < b; ++i) {
             const size_t at = part.n;
             part.add(reqs[i], s.variant);
             p.in_params[at] = reqs[i];
         }
         const int ctas = set_args(p, part, st, s, seed);
-        const cudaError_t e = launch_batch(p, ctas, s, stream);
+        const cudaError_t e = launch_batch(p, ctas, s, sum.host, stream);
         if (e)
             return cuda_fail(e, "aes_ctr_batch launch");
     }
@@ -609,7 +630,7 @@ int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_bat
     // cudaMemcpyAsync returns, so it may be destroyed afterwards.
     e = cudaMemcpyAsync(reqs, host.data(), bytes, cudaMemcpyHostToDevice, cs);
     if (!e)
-        e = launch_batch(p, ctas, s, cs);
+        e = launch_batch(p, ctas, s, sum.host, cs);
     cudaError_t e2 = cudaFreeAsync(reqs, cs);
     if (e)
         return cuda_fail(e, "aes_ctr_batch");
@@ -686,7 +707,7 @@ int aes_batch_plan_launch(aes_batch_plan_t plan, void *stream)
         return AES_OK;  // nothing to encrypt (all lengths zero)
     if (capturing(static_cast<cudaStream_t>(stream)))
         return cuda_fail(cudaErrorStreamCaptureUnsupported, "aes_batch_plan_launch");
-    const cudaError_t e = launch_batch(plan->params, plan->ctas, plan->shape, static_cast<cudaStream_t>(stream));
+    const cudaError_t e = launch_batch(plan->params, plan->ctas, plan->shape, plan->sum.host, static_cast<cudaStream_t>(stream));
     return e ? cuda_fail(e, "aes_batch_plan_launch") : AES_OK;
 }
 

@@ -209,7 +209,7 @@ bool allocation_bounds(const void *p, uintptr_t *begin, uintptr_t *end)
 
 }  // namespace
 
-int PayloadChecks::resolve(const void *p, Range &r, const void **dptr)
+int PayloadChecks::resolve(const void *p, Range &r, const void **dptr, bool *host)
 {
     const uintptr_t a = (uintptr_t)p;
     if (a >= r.begin && a < r.end) {
@@ -217,10 +217,11 @@ int PayloadChecks::resolve(const void *p, Range &r, const void **dptr)
         *dptr = p;
         return AES_OK;
     }
-    bool host = false;
-    const int rc = resolve_ptr(p, dev_, dptr, &host);
+    bool is_host = false;
+    const int rc = resolve_ptr(p, dev_, dptr, &is_host);
+    *host |= is_host;
     // payloads spread over many allocations: stop looking for their bounds
-    if (rc || host || *dptr != p || r.misses > 4)
+    if (rc || is_host || *dptr != p || r.misses > 4)
         return rc;
     ++r.misses;
     cudaPointerAttributes at;
@@ -230,17 +231,18 @@ int PayloadChecks::resolve(const void *p, Range &r, const void **dptr)
     return AES_OK;
 }
 
-int PayloadChecks::check(const void *in, const void *out, size_t len, const void **din, void **dout)
+int PayloadChecks::check(const void *in, const void *out, size_t len, const void **din, void **dout, bool *host)
 {
+    *host = false;
     int rc = check_bounds(in, out, len);
-    if (rc || (rc = resolve(in, in_, din)))
+    if (rc || (rc = resolve(in, in_, din, host)))
         return rc;
     if (out == in) {
         *dout = const_cast<void *>(*din);
         return AES_OK;
     }
     const void *o = nullptr;
-    if ((rc = resolve(out, out_, &o)))
+    if ((rc = resolve(out, out_, &o, host)))
         return rc;
     *dout = const_cast<void *>(o);
     return AES_OK;

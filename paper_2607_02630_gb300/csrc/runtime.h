@@ -56,14 +56,15 @@ int check_payload(const void *in, const void *out, size_t len, int dev, const vo
 class PayloadChecks {
 public:
     explicit PayloadChecks(int dev) : dev_(dev) {}
-    int check(const void *in, const void *out, size_t len, const void **din, void **dout);
+    // *host: a payload lies in pinned host memory
+    int check(const void *in, const void *out, size_t len, const void **din, void **dout, bool *host);
 
 private:
     struct Range {
         uintptr_t begin = 0, end = 0;
         int misses = 0;
     };
-    int resolve(const void *p, Range &r, const void **dptr);
+    int resolve(const void *p, Range &r, const void **dptr, bool *host);
     int dev_;
     Range in_, out_;
 };

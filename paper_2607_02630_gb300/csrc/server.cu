@@ -60,7 +60,7 @@
 #include "runtime.h"
 #include "common.cuh"
 #include "aes_ttable.cuh"
-#include "tile.cuh"
+#include "served_tile.cuh"
 #include "served_protocol.cuh"
 
 #include <algorithm>
@@ -93,11 +93,13 @@ struct RkRegsL2 {
     __device__ __forceinline__ uint4 get(int r) const { return w[r]; }
 };
 
-// Chunks [k0, k1) of a request (clipped to those it has), done by the calling
-// warp alone, with the request's round keys in registers.
+// Part `part` of `parts` of the single counter group [first, last) (or the
+// whole tile when parts == 1) of a request, done by the calling warp alone,
+// with the request's round keys in registers.
 // (stamp: trace builds record when the keys have arrived)
-template <int NR>
-__device__ __forceinline__ void run_tile_regs(const aesrt::BatchReq &rq, uint64_t k0, uint64_t k1, uint4 *s_group,
+template <int NR, int NB>
+__device__ __forceinline__ void run_part_regs(const aesrt::BatchReq &rq, uint64_t first, uint64_t last,
+                                              uint32_t part, uint32_t parts,
                                               const aestt::Lanes &ln, const SrvParams &p, uint32_t seq, bool stamp)
 {
     const RkRegsL2<NR> rk(rq.rk);
@@ -112,16 +114,7 @@ __device__ __forceinline__ void run_tile_regs(const aesrt::BatchReq &rq, uint64_
     (void)seq;
     (void)stamp;
 #endif
-    const uint64_t nb = (rq.len + 15) >> 4, first = aestile::first_chunk(rq.iv_lo);
-    const uint64_t end = (((rq.iv_lo & 255u) + nb - 1) >> 5) + 1;
-    k0 = k0 > first ? k0 : first;
-    k1 = k1 < end ? k1 : end;
-#pragma unroll 1
-    while (k0 < k1) {
-        const uint32_t n = aestile::run_chunks(rq.iv_lo, k0, k1 - k0);
-        aestile::xor_run<NR>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, k0, n, s_group, ln, rk);
-        k0 += n;
-    }
+    aesserved::xor_range<NR, NB>(rq.in, rq.out, rq.len, rq.iv_hi, rq.iv_lo, first, last, part, parts, parts, ln, rk);
 }
 
 template <bool PER_REQ>
@@ -129,7 +122,6 @@ __global__ void __launch_bounds__(512, 1) server_kernel(const __grid_constant__ 
 {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ Ring ring;
-    __shared__ uint4 s_group[kMaxWarps][aestile::kRunGroups];
     if (threadIdx.x == 0)
         ring_init(ring);
     aestt::fill_tables(smem, p.te0);
@@ -196,13 +188,13 @@ __global__ void __launch_bounds__(512, 1) server_kernel(const __grid_constant__ 
             }
             __syncwarp();
         } else {
-            // tile t: 8 / tp chunks of one group, or tg whole groups of 8
-            const uint64_t per = tp > 1 ? 8u / tp : 8u * (uint64_t)tg, k0 = t * per, k1 = k0 + per;
-            const bool stamp = lane == 0 && t == 0;
+            uint64_t first, last;
+            const uint32_t part = t % tp;
+            aesserved::tile_blocks_of(t / tp, tg, rq.iv_lo & 255u, (rq.len + 15) >> 4, &first, &last);
             switch (rq.nr) {
-            case 10: run_tile_regs<10>(rq, k0, k1, s_group[warp], ln, p, seq, stamp); break;
-            case 12: run_tile_regs<12>(rq, k0, k1, s_group[warp], ln, p, seq, stamp); break;
-            default: run_tile_regs<14>(rq, k0, k1, s_group[warp], ln, p, seq, stamp); break;
+            case 10: run_part_regs<10, 2>(rq, first, last, part, tp, ln, p, seq, lane == 0 && t == 0); break;
+            case 12: run_part_regs<12, 2>(rq, first, last, part, tp, ln, p, seq, lane == 0 && t == 0); break;
+            default: run_part_regs<14, 2>(rq, first, last, part, tp, ln, p, seq, lane == 0 && t == 0); break;
             }
         }
         // Order the tile's output stores before it is counted: a warp

@@ -1,6 +1,6 @@
 // tile.cuh -- xor the AES-CTR keystream into a run of 32-block chunks of one
-// message with T-table rounds and counter-mode caching (shared by the batch
-// and served kernels).
+// message with T-table rounds and counter-mode caching (the batch kernel's
+// work on a request).
 #pragma once
 #include "internal.h"
 #include "common.cuh"

@@ -298,12 +298,13 @@ typedef struct {
     int ctas;               /* resident CTAs; 0 = SM count - 4 */
     int threads;            /* CTA size, multiple of 32, 64..512; 0 = 512 (warp 0 dispatches) */
     int tile_blocks;        /* 16-byte blocks per tile: 64, 128 or a multiple of 256;
-                               0 = per request (~512 tiles of 64..1024 blocks,
-                               down to 64 tiles with 64 requests in flight:
-                               the latency setting).  Fewer, larger tiles serve
-                               more requests per second (measured on GB300,
-                               served mix: 269 k req/s by default, 370 k with
-                               1024), at the cost of one-in-flight latency. */
+                               0 = per request: about 512 tiles of 64..1024
+                               blocks, 256, 128 or 64 from 16, 32 and 64
+                               requests in flight (served mix from 8 native
+                               submitters on GB300: 358 k req/s, 265 k with
+                               512 tiles always).  Fewer, larger tiles serve
+                               more requests per second at the cost of
+                               one-in-flight latency. */
     uint32_t idle_timeout_us; /* resident kernel exits after this long with no
                                  work (relaunched on the next submit); 0 = 200000 */
     int claim_mode;         /* how agents claim tiles: 0 = one global cursor

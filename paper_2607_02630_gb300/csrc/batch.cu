@@ -461,6 +461,8 @@ static int fill_reqs(const aes_desc_t *descs, int n, int dev, int variant, Batch
         const int rc = payloads.check(d.in, d.out, d.len, &din, &dout, &host);
         if (rc)
             return rc;
+        if (!blocks_of(d.len))
+            continue;
         BatchReq r{};
         r.in = static_cast<const uint4 *>(din);
         r.out = static_cast<uint4 *>(dout);

@@ -200,7 +200,9 @@ int ctr_ctas(uint64_t nblocks, uint32_t v0, const CtrShape &s, int nsm)
 
 cudaError_t launch_ctr(const CtrParams &p, int nr, const CtrShape &s, int nsm, cudaStream_t stream)
 {
-    const uint64_t nblocks = (p.len + 15) / 16;
+    const uint64_t nblocks = aesrt::blocks_of(p.len);
+    if (!nblocks)
+        return cudaSuccess;
     const int ctas = ctr_ctas(nblocks, (uint32_t)(p.iv_lo & 255u), s, nsm);
     if (s.variant == 2) {
         if (s.threads != 128)

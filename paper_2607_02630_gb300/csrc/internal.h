@@ -27,6 +27,11 @@ struct CtrShape {
     int ctas;     // 0 = derive
 };
 
+// 16-byte blocks of `len` bytes.  A length within 15 bytes of 2^64 (a negative
+// one made unsigned) wraps to none: the entry points do nothing with it, and
+// no count of chunks may be derived from it.
+inline uint64_t blocks_of(uint64_t len) { return (len + 15) / 16; }
+
 // Device tables and key expansion (tables.cu).
 cudaError_t launch_te0_init(uint32_t *te0, cudaStream_t stream);
 cudaError_t launch_key_expand(const uint8_t *keys, const int32_t *bits, const uint32_t *te0,
@@ -99,11 +104,11 @@ struct BatchShape {
     int nb;           // T-table: accepted as 1, 2 or 4; the kernel keeps one block per lane in flight
 };
 
-// 32-block chunks of the counter space that `len` > 0 bytes touch when the
-// initial counter has low byte `iv_low_byte`.
+// 32-block chunks of the counter space that `len` bytes (of at least one
+// block) touch when the initial counter has low byte `iv_low_byte`.
 inline uint64_t chunks_of(uint64_t len, uint32_t iv_low_byte)
 {
-    const uint64_t nb = (len + 15) / 16;
+    const uint64_t nb = blocks_of(len);
     return ((iv_low_byte + nb - 1) >> 5) - (iv_low_byte >> 5) + 1;
 }
 

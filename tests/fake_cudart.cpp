@@ -1,0 +1,258 @@
+// A CUDA runtime that runs nothing and writes down what it is asked to do:
+// linked with the library's own objects, it shows on the CPU which launches an
+// entry point makes, on which device and stream and with which grid.  Two
+// devices; device memory is host memory; streams know their device; captured
+// launches become graphs.  Not modelled: time, and what kernels compute.
+#include <cuda_runtime_api.h>
+
+#include <atomic>
+#include <cstdint>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <new>
+#include <set>
+#include <string>
+#include <utility>
+#include <vector>
+
+namespace {
+
+struct Launch {
+    int device;        // the device the kernel runs on
+    int grid, block;
+    int by_graph;      // 1: a node of a launched graph
+    int programmatic;  // 1: may start before the stream's previous kernel has ended
+    uint64_t stream;
+    char args[64];     // the first bytes of the first parameter
+    char name[128];
+};
+
+struct Stream {
+    int device;
+    bool capturing = false;
+    std::vector<Launch> captured;
+};
+struct Graph {
+    std::vector<Launch> launches;
+};
+
+int g_device = 0, g_sms = 152;
+std::atomic<long> g_news{0};
+std::vector<Launch> g_log;
+std::set<Stream *> g_streams;
+std::map<const void *, std::string> g_names;
+std::set<std::pair<const void *, int>> g_big_smem;  // (kernel, device): more than 48 KiB allowed
+thread_local dim3 t_grid, t_block;
+thread_local size_t t_smem;
+thread_local cudaStream_t t_stream;
+
+Stream *stream_of(cudaStream_t s) { return g_streams.count((Stream *)s) ? (Stream *)s : nullptr; }
+
+cudaError_t launch(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void **args, bool programmatic,
+                   bool copy_args)
+{
+    Stream *st = stream_of(s);
+    if (st && st->device != g_device)
+        return cudaErrorInvalidResourceHandle;
+    if (smem > 49152 && !g_big_smem.count({fn, g_device}))
+        return cudaErrorInvalidValue;
+    Launch l{};
+    l.device = g_device;
+    l.grid = (int)grid.x;
+    l.block = (int)block.x;
+    l.programmatic = programmatic;
+    l.stream = (uint64_t)(uintptr_t)s;
+    if (copy_args)
+        std::memcpy(l.args, args[0], sizeof(l.args));
+    std::strncpy(l.name, g_names[fn].c_str(), sizeof(l.name) - 1);
+    if (st && st->capturing)
+        st->captured.push_back(l);
+    else
+        g_log.push_back(l);
+    return cudaSuccess;
+}
+
+}  // namespace
+
+// Allocations of the library itself.
+void *operator new(size_t n)
+{
+    ++g_news;
+    if (void *p = std::malloc(n ? n : 1))
+        return p;
+    throw std::bad_alloc();
+}
+void *operator new(size_t n, const std::nothrow_t &) noexcept
+{
+    ++g_news;
+    return std::malloc(n ? n : 1);
+}
+void operator delete(void *p) noexcept { std::free(p); }
+void operator delete(void *p, size_t) noexcept { std::free(p); }
+void operator delete(void *p, const std::nothrow_t &) noexcept { std::free(p); }
+
+extern "C" {
+
+// --- what a test asks and sets ---
+long fake_news() { return g_news; }
+void fake_set_device(int d) { g_device = d; }
+int fake_device() { return g_device; }
+void fake_set_sms(int n) { g_sms = n; }
+void *fake_stream(int device)
+{
+    Stream *s = new Stream{device, false, {}};
+    g_streams.insert(s);
+    return s;
+}
+void fake_reset()
+{
+    g_log.clear();
+    g_log.reserve(1 << 14);
+}
+int fake_launches() { return (int)g_log.size(); }
+void fake_launch(int i, Launch *out) { *out = g_log[(size_t)i]; }
+
+// --- the runtime ---
+cudaError_t cudaGetDevice(int *d) { return *d = g_device, cudaSuccess; }
+cudaError_t cudaSetDevice(int d) { return g_device = d, cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { return *v = g_sms, cudaSuccess; }
+cudaError_t cudaGetDeviceProperties(cudaDeviceProp *p, int)
+{
+    std::memset(p, 0, sizeof(*p));
+    std::strcpy(p->name, "fake");
+    p->multiProcessorCount = g_sms;
+    return cudaSuccess;
+}
+const char *cudaGetErrorString(cudaError_t) { return "fake"; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaMalloc(void **p, size_t n) { return *p = std::calloc(n ? n : 1, 1), cudaSuccess; }
+cudaError_t cudaFree(void *p) { return std::free(p), cudaSuccess; }
+cudaError_t cudaMemPoolCreate(cudaMemPool_t *p, const cudaMemPoolProps *) { return *p = nullptr, cudaSuccess; }
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }
+cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t, cudaStream_t) { return cudaMalloc(p, n); }
+cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return cudaFree(p); }
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t)
+{
+    std::memcpy(d, s, n);
+    return cudaSuccess;
+}
+cudaError_t cudaMemset(void *p, int v, size_t n) { return std::memset(p, v, n), cudaSuccess; }
+cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t) { return cudaMemset(p, v, n); }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p)
+{
+    std::memset(a, 0, sizeof(*a));
+    a->type = cudaMemoryTypeDevice;
+    a->devicePointer = const_cast<void *>(p);
+    return cudaSuccess;  // every address is memory of device 0
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult *)
+{
+    return cudaErrorNotSupported;
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned)
+{
+    *s = (cudaStream_t)fake_stream(g_device);
+    return cudaSuccess;
+}
+cudaError_t cudaStreamDestroy(cudaStream_t s)
+{
+    g_streams.erase((Stream *)s);
+    delete (Stream *)s;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus *c)
+{
+    Stream *st = stream_of(s);
+    *c = st && st->capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode)
+{
+    Stream *st = stream_of(s);
+    if (!st || st->capturing)
+        return cudaErrorInvalidValue;
+    st->capturing = true;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t *g)
+{
+    Stream *st = stream_of(s);
+    Graph *graph = new Graph{st->captured};
+    st->captured.clear();
+    st->capturing = false;
+    *g = (cudaGraph_t)graph;
+    return cudaSuccess;
+}
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t *e, cudaGraph_t g, unsigned long long)
+{
+    *e = (cudaGraphExec_t) new Graph(*(Graph *)g);
+    return cudaSuccess;
+}
+cudaError_t cudaGraphLaunch(cudaGraphExec_t e, cudaStream_t s)
+{
+    Stream *st = stream_of(s);
+    if (st && st->capturing)
+        return cudaErrorStreamCaptureUnsupported;
+    for (Launch l : ((Graph *)e)->launches) {  // a kernel node runs on the device it was captured on
+        l.by_graph = 1;
+        l.stream = (uint64_t)(uintptr_t)s;
+        g_log.push_back(l);
+    }
+    return cudaSuccess;
+}
+cudaError_t cudaGraphDestroy(cudaGraph_t g) { return delete (Graph *)g, cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t e) { return delete (Graph *)e, cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t *e) { return *e = nullptr, cudaSuccess; }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return *e = nullptr, cudaSuccess; }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.f, cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void *fn, cudaFuncAttribute, int v)
+{
+    if (v > 49152)
+        g_big_smem.insert({fn, g_device});
+    return cudaSuccess;
+}
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned)
+{
+    return *n = 2, cudaSuccess;
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fn, void **args)
+{
+    bool programmatic = false;
+    for (unsigned i = 0; i < c->numAttrs; ++i)
+        programmatic |= c->attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization;
+    return launch(fn, c->gridDim, c->blockDim, c->dynamicSmemBytes, c->stream, args, programmatic, true);
+}
+
+// --- what nvcc's host code calls for <<<>>> and for the embedded kernels ---
+unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t smem, void *s)
+{
+    t_grid = grid, t_block = block, t_smem = smem, t_stream = (cudaStream_t)s;
+    return 0;
+}
+cudaError_t __cudaPopCallConfiguration(dim3 *grid, dim3 *block, size_t *smem, void *s)
+{
+    *grid = t_grid, *block = t_block, *smem = t_smem, *(cudaStream_t *)s = t_stream;
+    return cudaSuccess;
+}
+cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *fn) { return *k = (cudaKernel_t)fn, cudaSuccess; }
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void **args, size_t smem, cudaStream_t s)
+{
+    return launch((const void *)k, grid, block, smem, s, args, false, false);
+}
+void **__cudaRegisterFatBinary(void *) { return (void **)std::malloc(8); }
+void __cudaRegisterFatBinaryEnd(void **) {}
+void __cudaUnregisterFatBinary(void **h) { std::free(h); }
+void __cudaRegisterFunction(void **, const char *fn, char *, const char *name, int, uint3 *, uint3 *, dim3 *, dim3 *,
+                            int *)
+{
+    g_names[fn] = name;
+}
+
+}  // extern "C"

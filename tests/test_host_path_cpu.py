@@ -1,0 +1,115 @@
+"""The host side of the entry points on the CPU: the library's own objects
+linked with a CUDA runtime that runs nothing (fake_cudart.cpp) and writes down
+each launch -- kernel, device, stream, grid, first parameter bytes."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+from paper_2607_02630_gb300 import aesoffload as A
+from paper_2607_02630_gb300 import build as B
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+P = 0x7F00_0000_0000  # a payload address (nothing reads it)
+
+
+class Launch(ctypes.Structure):
+    _fields_ = [("device", ctypes.c_int), ("grid", ctypes.c_int), ("block", ctypes.c_int), ("by_graph", ctypes.c_int),
+                ("programmatic", ctypes.c_int), ("stream", ctypes.c_uint64), ("args", ctypes.c_char * 64),
+                ("name", ctypes.c_char * 128)]
+
+
+class Host:
+    def __init__(self, lib):
+        self.lib = lib
+
+    def ctx(self, bits=128):
+        h = ctypes.c_void_p()
+        assert self.lib.aes_ctx_create(ctypes.byref(h), bytes(32), bits) == A.AES_OK
+        return h
+
+    def descs(self, reqs):
+        arr = (A.Desc * len(reqs))()
+        for d, (ctx, low, src, dst, n) in zip(arr, reqs):
+            d.ctx, d.inp, d.out, d.len = ctx, src, dst, n
+            d.iv[15] = low
+        return arr
+
+    def launches(self):
+        out = []
+        for i in range(self.lib.fake_launches()):
+            out.append(Launch())
+            self.lib.fake_launch(i, ctypes.byref(out[-1]))
+        return out
+
+    def during(self, f, *args):
+        """(status, launches) of one call."""
+        self.lib.fake_reset()
+        return f(*args), self.launches()
+
+
+@pytest.fixture(scope="module")
+def built(tmp_path_factory):
+    B.build()
+    nvcc = B._nvcc()
+    cuda_inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    so = str(tmp_path_factory.mktemp("fake") / "libaes_fake.so")
+    objs = [os.path.join(B.BUILD, n + ".o") for n in ("capi", "batch", "batch_noalloc", "ctr", "tables", "tune")]
+    r = subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-std=c++17", "-Wl,-Bsymbolic", "-I", cuda_inc,
+                        os.path.join(HERE, "fake_cudart.cpp")] + objs + ["-o", so], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return so
+
+
+@pytest.fixture()
+def host(built):
+    lib = ctypes.CDLL(built)
+    vp, sz, ci = ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int
+    lib.aes_ctx_create.argtypes = [vp, ctypes.c_char_p, ci]
+    lib.aes_ctr.argtypes = [vp, ctypes.c_char_p, vp, vp, sz, vp]
+    lib.aes_ctr_ex.argtypes = [vp, ctypes.c_char_p, vp, vp, sz, vp, vp]
+    lib.aes_ctr_batch_ex.argtypes = [vp, ci, vp, vp]
+    lib.aes_ctr_batch_noalloc.argtypes = [vp, ci, vp]
+    lib.aes_batch_plan_create.argtypes = [vp, vp, ci, vp]
+    lib.aes_batch_plan_launch.argtypes = [vp, vp]
+    lib.aes_batch_plan_destroy.argtypes = [vp]
+    lib.aes_batch_plan_bytes.argtypes = [vp]
+    lib.aes_batch_plan_bytes.restype = ctypes.c_int64
+    lib.aes_tuned_shape.argtypes = [sz, ci, vp]
+    lib.fake_launch.argtypes = [ci, vp]
+    lib.fake_stream.restype = vp
+    lib.fake_news.restype = ctypes.c_long
+    lib.fake_set_device(0)
+    lib.fake_reset()
+    return Host(lib)
+
+
+@pytest.mark.parametrize("low", [0, 1, 31, 32, 255])
+@pytest.mark.parametrize("below", [1, 8, 15])
+def test_length_whose_end_wraps_is_no_work(host, low, below):
+    """A length within 15 bytes of 2^64 (a negative one passed through an
+    unsigned argument) is no whole number of blocks: the calls accept it and
+    encrypt nothing, alone and beside a request that has work."""
+    n = (1 << 64) - below
+    ctx = host.ctx()
+    iv = bytes(15) + bytes([low])
+    assert host.during(host.lib.aes_ctr, ctx, iv, P, P, n, None) == (A.AES_OK, [])
+    for variant, threads in ((1, 512), (2, 128)):
+        shape = A.LaunchShape(variant, threads, 1, 0)
+        assert host.during(host.lib.aes_ctr_ex, ctx, iv, P, P, n, None, ctypes.byref(shape)) == (A.AES_OK, [])
+    assert host.during(host.lib.aes_ctr, ctx, iv, P + 8, P, n, None) == (A.AES_EALIGN, [])
+    one = host.descs([(ctx, low, P, P, n)])
+    two = host.descs([(ctx, low, P, P, n), (ctx, low, P, P, 100)])
+    want = host.during(host.lib.aes_ctr_batch_ex, host.descs([(ctx, low, P, P, 100)]), 1, None, None)[1]
+    for variant in (1, 2):
+        opts = A.BatchOpts(variant, 0, 0, 0, 0, 0)
+        assert host.during(host.lib.aes_ctr_batch_ex, one, 1, None, ctypes.byref(opts)) == (A.AES_OK, [])
+        plan = ctypes.c_void_p()
+        assert host.lib.aes_batch_plan_create(ctypes.byref(plan), one, 1, ctypes.byref(opts)) == A.AES_OK
+        assert host.during(host.lib.aes_batch_plan_launch, plan, None) == (A.AES_OK, [])
+        host.lib.aes_batch_plan_destroy(plan)
+    for call in (lambda d: host.lib.aes_ctr_batch_ex(d, 2, None, None),
+                 lambda d: host.lib.aes_ctr_batch_noalloc(d, 2, None)):
+        rc, got = host.during(call, two)
+        assert rc == A.AES_OK and [(l.grid, l.args) for l in got] == [(l.grid, l.args) for l in want]

@@ -171,7 +171,8 @@ typedef struct {
  * three launches past 500 and 1000); more in a descriptor table allocated
  * and uploaded by the call.  n == 0 is a no-op.  Errors: AES_EINVAL (n < 0,
  * null descs, a NULL ctx), AES_EALIGN / AES_EOVERLAP / AES_EPTR for the first
- * bad request, AES_ETOOBIG (n > AES_BATCH_MAX), AES_ENOMEM, AES_ECUDA. */
+ * bad request, AES_ETOOBIG (n > AES_BATCH_MAX, or more than 2^32 - 1 tiles of
+ * tile_blocks, 128 TiB in all in the built-in shape), AES_ENOMEM, AES_ECUDA. */
 #define AES_BATCH_MAX (1 << 20)
 int aes_ctr_batch(const aes_desc_t *descs, int n, void *stream);
 int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_batch_opts_t *opts);

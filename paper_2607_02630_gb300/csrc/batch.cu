@@ -349,6 +349,13 @@ cudaError_t batch_set_attributes()
     return cudaSuccess;
 }
 
+// More tiles (of BatchShape::counted blocks) than this are AES_ETOOBIG: the
+// lengths of one batch stay far below what would overflow its summed cost.
+// The built-in shape counts tiles of 2048 blocks (128 TiB in all), whatever
+// size it claims them in.
+constexpr uint64_t kMostTiles = 0xffffffffull;
+constexpr int kBuiltInCounted = 2048;
+
 static uint64_t gcd64(uint64_t a, uint64_t b)
 {
     while (b) {
@@ -362,7 +369,7 @@ static uint64_t gcd64(uint64_t a, uint64_t b)
 static TileOrder make_order(uint64_t total, uint32_t seed)
 {
     TileOrder o{1, 0, 0};
-    if (!seed || total < 2)
+    if (!seed || total < 2 || total > kMostTiles)  // a * t must fit 64 bits
         return o;
     o.tiles = total;
     uint64_t x = seed * 0x9E3779B97F4A7C15ull + 0x632BE59BD9B4E019ull;
@@ -385,6 +392,7 @@ struct BatchSums {
     size_t n = 0;       // requests that hold any bytes
     bool host = false;  // some payload lies in pinned host memory
     uint64_t cost = 0, units = 0;
+    uint64_t tiles = 0;  // of BatchShape::counted blocks; stays at kMostTiles + 1 once past it
     int64_t bytes = 0;
     // Appends r: sets its first cost, adds its units.
     void add(BatchReq &r, int variant)
@@ -428,7 +436,7 @@ static BatchShape pick_batch_shape(const DeviceState &st, const aes_batch_opts_t
         if (opts->variant && opts->variant != s.variant) {
             // another variant than the tuned one: start from its defaults
             s = opts->variant == AES_VARIANT_BITSLICE ? BatchShape{AES_VARIANT_BITSLICE, kBsThreads, 2048, 0, 1}
-                                                      : BatchShape{opts->variant, 512, 7936, 0, 1};
+                                                      : BatchShape{opts->variant, 512, kBuiltInTile, 0, 1};
         }
         if (opts->threads)
             s.threads = opts->threads;
@@ -439,12 +447,13 @@ static BatchShape pick_batch_shape(const DeviceState &st, const aes_batch_opts_t
         if (opts->blocks_per_thread)
             s.nb = opts->blocks_per_thread;
     }
+    s.counted = s.tile_blocks == kBuiltInTile && !(opts && opts->tile_blocks) ? kBuiltInCounted : s.tile_blocks;
     return s;
 }
 
 // The non-empty requests of descs[0..n) into out (room for n), their sums into
 // `sum`; the first bad request's status.
-static int fill_reqs(const aes_desc_t *descs, int n, int dev, int variant, BatchReq *out, BatchSums &sum)
+static int fill_reqs(const aes_desc_t *descs, int n, int dev, const BatchShape &s, BatchReq *out, BatchSums &sum)
 {
     PayloadChecks payloads(dev);
     for (int i = 0; i < n; ++i) {
@@ -471,11 +480,13 @@ static int fill_reqs(const aes_desc_t *descs, int n, int dev, int variant, Batch
         r.rk = reinterpret_cast<const uint4 *>(d.ctx->d_rk);
         r.nr = (uint32_t)d.ctx->nr;
         sum.host |= host;
+        if (s.counted)
+            sum.tiles = std::min(sum.tiles + tiles_of(r.len, (uint32_t)(r.iv_lo & 255u), s.counted), kMostTiles + 1);
         const size_t at = sum.n;
-        sum.add(r, variant);
+        sum.add(r, s.variant);
         out[at] = r;
     }
-    return AES_OK;
+    return sum.tiles > kMostTiles ? AES_ETOOBIG : AES_OK;
 }
 
 // Everything of a launch but its requests; returns the grid size.
@@ -525,7 +536,7 @@ static int launch_in_params(const aes_desc_t *descs, int n, const DeviceState &s
 {
     BatchParams<CAP> p;
     BatchSums sum;
-    const int rc = fill_reqs(descs, n, st.device, s.variant, p.in_params, sum);
+    const int rc = fill_reqs(descs, n, st.device, s, p.in_params, sum);
     if (rc || !sum.n)
         return rc;
     const int ctas = set_args(p, sum, st, s, seed);
@@ -548,7 +559,7 @@ int batch_by_params(const aes_desc_t *descs, int n, const DeviceState &st, const
         return AES_ENOMEM;
     }
     BatchSums sum;
-    const int rc = fill_reqs(descs, n, st.device, s.variant, reqs.data(), sum);
+    const int rc = fill_reqs(descs, n, st.device, s, reqs.data(), sum);
     if (rc || !sum.n)
         return rc;
     // equal numbers of requests per launch
@@ -618,7 +629,7 @@ int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_bat
         return AES_ENOMEM;
     }
     BatchSums sum;
-    if ((rc = fill_reqs(descs, n, st->device, s.variant, host.data(), sum)) || !sum.n)
+    if ((rc = fill_reqs(descs, n, st->device, s, host.data(), sum)) || !sum.n)
         return rc;
     BatchParams<0> p{};
     const int ctas = set_args(p, sum, *st, s, seed);
@@ -675,7 +686,7 @@ int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
         delete plan;
         return AES_ENOMEM;
     }
-    if ((rc = fill_reqs(descs, n, st->device, s.variant, host.data(), plan->sum))) {
+    if ((rc = fill_reqs(descs, n, st->device, s, host.data(), plan->sum))) {
         delete plan;
         return rc;
     }

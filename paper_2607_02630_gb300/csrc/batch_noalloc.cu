@@ -33,6 +33,6 @@ extern "C" int aes_ctr_batch_noalloc(const aes_desc_t *descs, int n, void *strea
     // the tuned T-table shape
     BatchShape s = st->batch_tuned;
     if (s.variant != AES_VARIANT_TTABLE)
-        s = BatchShape{AES_VARIANT_TTABLE, 512, 7936, 0, 1};
+        s = BatchShape{AES_VARIANT_TTABLE, 512, kBuiltInTile, 0, 1};
     return batch_by_params(descs, n, *st, s, 0, static_cast<cudaStream_t>(stream));
 }

@@ -96,13 +96,27 @@ struct BatchReq {        // one request, device-side descriptor (64 bytes)
 };
 static_assert(sizeof(BatchReq) == 64, "descriptor is one 64-byte line");
 
+constexpr int kBuiltInTile = 7936;  // tile_blocks of the shape used until a tuner picks another
+
 struct BatchShape {
     int variant;      // AES_VARIANT_TTABLE or AES_VARIANT_BITSLICE
     int threads;
     int tile_blocks;  // a multiple of 256: the largest tile a warp claims
     int ctas;
     int nb;           // T-table: accepted as 1, 2 or 4; the kernel keeps one block per lane in flight
+    int counted;      // the batch may hold 2^32 - 1 tiles of so many blocks (0: no limit)
 };
+
+// Tiles of `tile_blocks` blocks (whole 256-block counter groups) that `len`
+// bytes make when the initial counter has low byte `iv_low_byte`.
+inline uint64_t tiles_of(uint64_t len, uint32_t iv_low_byte, int tile_blocks)
+{
+    const uint64_t nb = blocks_of(len);
+    if (!nb)
+        return 0;
+    const uint64_t groups = ((iv_low_byte + nb - 1) >> 8) + 1, per = (uint64_t)tile_blocks / 256u;
+    return (groups + per - 1) / per;
+}
 
 // 32-block chunks of the counter space that `len` bytes (of at least one
 // block) touch when the initial counter has low byte `iv_low_byte`.

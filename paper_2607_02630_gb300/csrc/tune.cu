@@ -53,7 +53,7 @@ void tune_defaults(DeviceState &st)
             st.ctr_tuned[i][b] = default_shape();
     // largest tiles of 2048, 4096 and 7936 blocks (a run's most): 4096 requests
     // of 1 KiB to 8 MiB 4097, 4060 and 4043 us, 512 of them 572, 566 and 565 us
-    st.batch_tuned = BatchShape{AES_VARIANT_TTABLE, 512, 7936, 0, 1};
+    st.batch_tuned = BatchShape{AES_VARIANT_TTABLE, 512, kBuiltInTile, 0, 1};
 }
 
 CtrShape tuned_ctr_shape(const DeviceState &st, size_t len, int nr)

@@ -113,3 +113,32 @@ def test_length_whose_end_wraps_is_no_work(host, low, below):
                  lambda d: host.lib.aes_ctr_batch_noalloc(d, 2, None)):
         rc, got = host.during(call, two)
         assert rc == A.AES_OK and [(l.grid, l.args) for l in got] == [(l.grid, l.args) for l in want]
+
+
+def _opts(variant=0, tile_blocks=0):
+    return ctypes.byref(A.BatchOpts(variant, 0, tile_blocks, 0, 0, 0))
+
+
+@pytest.mark.parametrize("variant,tile_blocks,limit", [(0, 0, 2048), (1, 256, 256), (1, 7936, 7936), (2, 0, 2048),
+                                                       (2, 1024, 1024)])
+def test_batches_of_more_than_2_32_tiles_are_refused(host, variant, tile_blocks, limit):
+    """A batch or plan of more than 2^32 - 1 tiles is AES_ETOOBIG, in one
+    request, over several, and where the count itself would wrap; a request
+    that is bad for another reason keeps its own status.  The built-in shape
+    counts tiles of 2048 blocks."""
+    ctx = host.ctx()
+    most = (2 ** 32 - 1) * limit * 16  # bytes, a whole number of tiles
+    half = (2 ** 31) * limit * 16
+    ok = [[most], [half, most - half], [limit * 16] * 5 + [most - 5 * limit * 16]]
+    bad = [[most + 16], [most, 1], [half, half], [1 << 62] * 9, [(1 << 64) - 16] * 3]
+    for lens in ok + bad:
+        want = A.AES_OK if lens in ok else A.AES_ETOOBIG
+        d = host.descs([(ctx, 0, P, P, n) for n in lens])
+        rc, got = host.during(host.lib.aes_ctr_batch_ex, d, len(lens), None, _opts(variant, tile_blocks))
+        assert rc == want and len(got) == (1 if lens in ok else 0)
+        plan = ctypes.c_void_p()
+        assert host.lib.aes_batch_plan_create(ctypes.byref(plan), d, len(lens), _opts(variant, tile_blocks)) == want
+        assert bool(plan.value) == (want == A.AES_OK)
+        host.lib.aes_batch_plan_destroy(plan)
+    d = host.descs([(ctx, 0, P, P, 1 << 62), (ctx, 0, P + 8, P, 16)])
+    assert host.lib.aes_ctr_batch_ex(d, 2, None, _opts(variant, tile_blocks)) == A.AES_EALIGN

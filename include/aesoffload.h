@@ -196,8 +196,10 @@ int aes_ctr_batch_noalloc(const aes_desc_t *descs, int n, void *stream);
 /* A prepared batch: the descriptor table lives on the device, so repeated
  * encryption of the same request layout costs one kernel launch.  Payload
  * contents may change between launches; pointers, lengths, keys and IVs are
- * fixed at creation.  A plan is not launched into a stream that is being
- * captured (AES_ECUDA). */
+ * fixed at creation.  A plan runs on the device it was created on, whichever
+ * is current, in a stream of any device; its launches run one after the other
+ * on whatever streams and from whatever threads they are made.  It is not
+ * launched into a stream that is being captured (AES_ECUDA). */
 typedef struct aes_batch_plan_s *aes_batch_plan_t;
 int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
                           const aes_batch_opts_t *opts);

@@ -35,6 +35,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -586,13 +587,100 @@ int batch_by_params(const aes_desc_t *descs, int n, const DeviceState &st, const
 
 using namespace aesrt;
 
+namespace {
+
+// The calling thread's current device, put back when the scope ends.
+class OnDevice {
+public:
+    OnDevice() { error = cudaGetDevice(&before_); }
+    ~OnDevice() { set(before_); }
+    int before() const { return before_; }
+    cudaError_t set(int device)
+    {
+        int now = -1;
+        const cudaError_t e = cudaGetDevice(&now);
+        return e || now == device ? e : cudaSetDevice(device);
+    }
+    cudaError_t error;
+
+private:
+    int before_ = 0;
+};
+
+}  // namespace
+
+// A prepared batch.  It runs on the device it was created on, whichever is
+// current, in any device's stream, and its launches run one after the other on
+// whatever streams they are made (two launches at once of a plan that encrypts
+// in place would race): a launch waits for the event that the last one left,
+// unless both are on one stream.  Recording the event costs 0.4 us of host
+// time and leaves launches in a row overlapped (64 requests of 1 to 16 KiB
+// 5.1 us a launch with it and without; as a CUDA graph, which has the same
+// guarantees, 8.2 us).
 struct aes_batch_plan_s {
-    int device;
+    int device = 0;
     BatchSums sum;
-    BatchShape shape;
+    BatchShape shape{};
     BatchParams<0> params{};
     int ctas = 0;
     BatchReq *reqs = nullptr;  // device
+    std::mutex mu;
+    cudaEvent_t done = nullptr;     // the last launch
+    bool launched = false;
+    unsigned long long last_id = 0;  // cudaStreamGetId of its stream
+    cudaStream_t own = nullptr;      // for launches into another device's stream
+
+    ~aes_batch_plan_s()
+    {
+        OnDevice on;
+        on.set(device);
+        cudaFree(reqs);
+        if (done)
+            cudaEventDestroy(done);
+        if (own)
+            cudaStreamDestroy(own);
+    }
+
+    // One launch on a stream of the plan's device, which is current.
+    cudaError_t launch_on(cudaStream_t stream)
+    {
+        unsigned long long id = 0;
+        cudaError_t e = cudaStreamGetId(stream, &id);
+        if (!e && launched && id != last_id)
+            e = cudaStreamWaitEvent(stream, done, 0);
+        if (e || (e = launch_batch(params, ctas, shape, sum.host, stream)))
+            return e;
+        launched = true;
+        last_id = id;
+        return cudaEventRecord(done, stream);
+    }
+
+    // One launch into a stream of `stream_device`: on the plan's own stream,
+    // between what that stream holds and what follows there.
+    cudaError_t launch_from(int stream_device, cudaStream_t stream, OnDevice &on)
+    {
+        cudaEvent_t before = nullptr;
+        cudaError_t e = on.set(stream_device);
+        if (!e)
+            e = cudaEventCreateWithFlags(&before, cudaEventDisableTiming);
+        if (!e)
+            e = cudaEventRecord(before, stream);
+        if (!e)
+            e = on.set(device);
+        if (!e && !own)
+            e = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+        if (!e)
+            e = cudaStreamWaitEvent(own, before, 0);
+        if (!e)
+            e = launch_on(own);
+        if (!e)
+            e = on.set(stream_device);
+        if (!e)
+            e = cudaStreamWaitEvent(stream, done, 0);
+        if (before)
+            cudaEventDestroy(before);
+        return e;
+    }
 };
 
 extern "C" {
@@ -700,8 +788,9 @@ int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
         e = cudaMemcpyAsync(plan->reqs, host.data(), bytes, cudaMemcpyHostToDevice, st->setup);
         if (!e)
             e = cudaStreamSynchronize(st->setup);
+        if (!e)
+            e = cudaEventCreateWithFlags(&plan->done, cudaEventDisableTiming);
         if (e) {
-            cudaFree(plan->reqs);
             delete plan;
             return cuda_fail(e, "aes_batch_plan_create");
         }
@@ -720,7 +809,19 @@ int aes_batch_plan_launch(aes_batch_plan_t plan, void *stream)
         return AES_OK;  // nothing to encrypt (all lengths zero)
     if (capturing(static_cast<cudaStream_t>(stream)))
         return cuda_fail(cudaErrorStreamCaptureUnsupported, "aes_batch_plan_launch");
-    const cudaError_t e = launch_batch(plan->params, plan->ctas, plan->shape, plan->sum.host, static_cast<cudaStream_t>(stream));
+    const cudaStream_t cs = static_cast<cudaStream_t>(stream);
+    OnDevice on;
+    cudaError_t e = on.error;
+    int stream_device = on.before();
+    if (!e && cs && cs != cudaStreamLegacy && cs != cudaStreamPerThread)
+        e = cudaStreamGetDevice(cs, &stream_device);
+    if (!e) {
+        std::lock_guard<std::mutex> lock(plan->mu);
+        if (stream_device != plan->device)
+            e = plan->launch_from(stream_device, cs, on);
+        else if (!(e = on.set(plan->device)))
+            e = plan->launch_on(cs);
+    }
     return e ? cuda_fail(e, "aes_batch_plan_launch") : AES_OK;
 }
 
@@ -728,9 +829,6 @@ int64_t aes_batch_plan_bytes(aes_batch_plan_t plan) { return plan ? plan->sum.by
 
 int aes_batch_plan_destroy(aes_batch_plan_t plan)
 {
-    if (!plan)
-        return AES_OK;
-    cudaFree(plan->reqs);
     delete plan;
     return AES_OK;
 }

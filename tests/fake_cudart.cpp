@@ -1,8 +1,8 @@
 // A CUDA runtime that runs nothing and writes down what it is asked to do:
 // linked with the library's own objects, it shows on the CPU which launches an
 // entry point makes, on which device and stream and with which grid.  Two
-// devices; device memory is host memory; streams know their device; captured
-// launches become graphs.  Not modelled: time, and what kernels compute.
+// devices; device memory is host memory; streams and events keep which launches
+// run behind which.  Not modelled: capture, time, and what kernels compute.
 #include <cuda_runtime_api.h>
 
 #include <atomic>
@@ -21,7 +21,6 @@ namespace {
 struct Launch {
     int device;        // the device the kernel runs on
     int grid, block;
-    int by_graph;      // 1: a node of a launched graph
     int programmatic;  // 1: may start before the stream's previous kernel has ended
     uint64_t stream;
     char args[64];     // the first bytes of the first parameter
@@ -30,16 +29,17 @@ struct Launch {
 
 struct Stream {
     int device;
-    bool capturing = false;
-    std::vector<Launch> captured;
+    std::set<int> before;  // launches that its next operation runs behind
 };
-struct Graph {
-    std::vector<Launch> launches;
+struct Event {
+    int device;
+    std::set<int> before;
 };
 
 int g_device = 0, g_sms = 152;
 std::atomic<long> g_news{0};
 std::vector<Launch> g_log;
+std::vector<std::set<int>> g_before;  // of each launch: those it runs behind
 std::set<Stream *> g_streams;
 std::map<const void *, std::string> g_names;
 std::set<std::pair<const void *, int>> g_big_smem;  // (kernel, device): more than 48 KiB allowed
@@ -47,13 +47,25 @@ thread_local dim3 t_grid, t_block;
 thread_local size_t t_smem;
 thread_local cudaStream_t t_stream;
 
-Stream *stream_of(cudaStream_t s) { return g_streams.count((Stream *)s) ? (Stream *)s : nullptr; }
+Stream g_null[2] = {{0}, {1}};
+
+Stream *stream_of(cudaStream_t s)
+{
+    return !s ? &g_null[g_device] : g_streams.count((Stream *)s) ? (Stream *)s : nullptr;
+}
+
+void enqueue(Stream *st, const Launch &l)
+{
+    g_before.push_back(st->before);
+    st->before.insert((int)g_log.size());
+    g_log.push_back(l);
+}
 
 cudaError_t launch(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void **args, bool programmatic,
                    bool copy_args)
 {
     Stream *st = stream_of(s);
-    if (st && st->device != g_device)
+    if (!st || st->device != g_device)
         return cudaErrorInvalidResourceHandle;
     if (smem > 49152 && !g_big_smem.count({fn, g_device}))
         return cudaErrorInvalidValue;
@@ -66,10 +78,7 @@ cudaError_t launch(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStrea
     if (copy_args)
         std::memcpy(l.args, args[0], sizeof(l.args));
     std::strncpy(l.name, g_names[fn].c_str(), sizeof(l.name) - 1);
-    if (st && st->capturing)
-        st->captured.push_back(l);
-    else
-        g_log.push_back(l);
+    enqueue(st, l);
     return cudaSuccess;
 }
 
@@ -101,17 +110,32 @@ int fake_device() { return g_device; }
 void fake_set_sms(int n) { g_sms = n; }
 void *fake_stream(int device)
 {
-    Stream *s = new Stream{device, false, {}};
+    Stream *s = new Stream{device};
     g_streams.insert(s);
     return s;
 }
 void fake_reset()
 {
     g_log.clear();
-    g_log.reserve(1 << 14);
+    g_before.clear();
+    for (Stream &n : g_null)
+        n.before.clear();
+    for (Stream *s : g_streams)
+        s->before.clear();
 }
 int fake_launches() { return (int)g_log.size(); }
 void fake_launch(int i, Launch *out) { *out = g_log[(size_t)i]; }
+// whether launch i runs behind launch j
+int fake_behind(int i, int j) { return (int)g_before[(size_t)i].count(j); }
+// a kernel of the caller's own, in a stream of the current device if null
+void fake_other_kernel(void *stream)
+{
+    Launch l{};
+    Stream *st = stream_of((cudaStream_t)stream);
+    l.device = st->device;
+    l.stream = (uint64_t)(uintptr_t)stream;
+    enqueue(st, l);
+}
 
 // --- the runtime ---
 cudaError_t cudaGetDevice(int *d) { return *d = g_device, cudaSuccess; }
@@ -163,52 +187,42 @@ cudaError_t cudaStreamDestroy(cudaStream_t s)
     return cudaSuccess;
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus *c)
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *c)
+{
+    return *c = cudaStreamCaptureStatusNone, cudaSuccess;
+}
+cudaError_t cudaStreamGetDevice(cudaStream_t s, int *d)
 {
     Stream *st = stream_of(s);
-    *c = st && st->capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
-    return cudaSuccess;
+    return st ? (*d = st->device, cudaSuccess) : cudaErrorInvalidResourceHandle;
 }
-cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode)
+cudaError_t cudaStreamGetId(cudaStream_t s, unsigned long long *id)
+{
+    return *id = (unsigned long long)(uintptr_t)stream_of(s), cudaSuccess;
+}
+cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned)
 {
     Stream *st = stream_of(s);
-    if (!st || st->capturing)
-        return cudaErrorInvalidValue;
-    st->capturing = true;
+    if (!st)
+        return cudaErrorInvalidResourceHandle;
+    st->before.insert(((Event *)e)->before.begin(), ((Event *)e)->before.end());
     return cudaSuccess;
 }
-cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t *g)
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned)
+{
+    *e = (cudaEvent_t) new Event{g_device, {}};
+    return cudaSuccess;
+}
+cudaError_t cudaEventCreate(cudaEvent_t *e) { return cudaEventCreateWithFlags(e, 0); }
+cudaError_t cudaEventDestroy(cudaEvent_t e) { return delete (Event *)e, cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s)
 {
     Stream *st = stream_of(s);
-    Graph *graph = new Graph{st->captured};
-    st->captured.clear();
-    st->capturing = false;
-    *g = (cudaGraph_t)graph;
+    if (!st || st->device != ((Event *)e)->device)
+        return cudaErrorInvalidResourceHandle;
+    ((Event *)e)->before = st->before;
     return cudaSuccess;
 }
-cudaError_t cudaGraphInstantiate(cudaGraphExec_t *e, cudaGraph_t g, unsigned long long)
-{
-    *e = (cudaGraphExec_t) new Graph(*(Graph *)g);
-    return cudaSuccess;
-}
-cudaError_t cudaGraphLaunch(cudaGraphExec_t e, cudaStream_t s)
-{
-    Stream *st = stream_of(s);
-    if (st && st->capturing)
-        return cudaErrorStreamCaptureUnsupported;
-    for (Launch l : ((Graph *)e)->launches) {  // a kernel node runs on the device it was captured on
-        l.by_graph = 1;
-        l.stream = (uint64_t)(uintptr_t)s;
-        g_log.push_back(l);
-    }
-    return cudaSuccess;
-}
-cudaError_t cudaGraphDestroy(cudaGraph_t g) { return delete (Graph *)g, cudaSuccess; }
-cudaError_t cudaGraphExecDestroy(cudaGraphExec_t e) { return delete (Graph *)e, cudaSuccess; }
-cudaError_t cudaEventCreate(cudaEvent_t *e) { return *e = nullptr, cudaSuccess; }
-cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return *e = nullptr, cudaSuccess; }
-cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.f, cudaSuccess; }

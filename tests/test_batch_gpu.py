@@ -341,3 +341,28 @@ def test_batch_checks_every_payload_pointer(cuda, aes, n):
             assert aes.batch_status(q) == want
             assert aes.batch_noalloc_status(q) == want
     cuda.cuda.synchronize()
+
+
+def test_plan_launches_are_ordered_across_streams(cuda, aes):
+    """Launches of one plan on different streams run one after the other: a
+    plan that encrypts in place, launched an even number of times from two
+    streams that wait for nothing, gives its input back."""
+    g = W.rng(5700)
+    lengths = [(24 << 20) + 7, 4096, 17, (3 << 20) + 16, 900_000]
+    bits = [(128, 256, 192)[i % 3] for i in range(len(lengths))]
+    reqs, meta, payload, src, dst = make_requests(cuda, aes, g, lengths, bits)
+    plan = aes.BatchPlan([(c, iv, s, s, k) for c, iv, s, d, k in reqs])
+    streams = [cuda.cuda.Stream(), cuda.cuda.Stream()]
+    cuda.cuda.synchronize()
+    for i in range(40):
+        plan.launch(streams[i & 1])
+    cuda.cuda.synchronize()
+    np.testing.assert_array_equal(to_host(src), payload)
+    plan.launch(streams[0])
+    plan.launch(streams[1])
+    plan.launch(streams[1])
+    cuda.cuda.synchronize()
+    out = to_host(src)
+    for key, b, iv, o, k in meta:
+        np.testing.assert_array_equal(out[o: o + k], oracle.ctr(key, b, iv, payload[o: o + k]))
+    plan.close()

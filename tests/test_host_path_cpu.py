@@ -15,7 +15,7 @@ P = 0x7F00_0000_0000  # a payload address (nothing reads it)
 
 
 class Launch(ctypes.Structure):
-    _fields_ = [("device", ctypes.c_int), ("grid", ctypes.c_int), ("block", ctypes.c_int), ("by_graph", ctypes.c_int),
+    _fields_ = [("device", ctypes.c_int), ("grid", ctypes.c_int), ("block", ctypes.c_int),
                 ("programmatic", ctypes.c_int), ("stream", ctypes.c_uint64), ("args", ctypes.c_char * 64),
                 ("name", ctypes.c_char * 128)]
 
@@ -79,6 +79,7 @@ def host(built):
     lib.aes_tuned_shape.argtypes = [sz, ci, vp]
     lib.fake_launch.argtypes = [ci, vp]
     lib.fake_stream.restype = vp
+    lib.fake_other_kernel.argtypes = [vp]
     lib.fake_news.restype = ctypes.c_long
     lib.fake_set_device(0)
     lib.fake_reset()
@@ -142,3 +143,54 @@ def test_batches_of_more_than_2_32_tiles_are_refused(host, variant, tile_blocks,
         host.lib.aes_batch_plan_destroy(plan)
     d = host.descs([(ctx, 0, P, P, 1 << 62), (ctx, 0, P + 8, P, 16)])
     assert host.lib.aes_ctr_batch_ex(d, 2, None, _opts(variant, tile_blocks)) == A.AES_EALIGN
+
+
+@pytest.mark.parametrize("variant", [1, 2])
+def test_plan_stays_on_its_device_and_in_order(host, variant):
+    """A plan runs on the device it was created on, whatever device is
+    current when it is launched (initialised or not by then) and whichever
+    device's stream it is launched into: behind that stream's earlier work,
+    before its later work, and behind the plan's last launch."""
+    lib = host.lib
+    ctx = host.ctx()
+    plan = ctypes.c_void_p()
+    d = host.descs([(ctx, 7, P, P, 9 << 20)])
+    assert lib.aes_batch_plan_create(ctypes.byref(plan), d, 1, _opts(variant)) == A.AES_OK
+    streams = [None, lib.fake_stream(0), lib.fake_stream(1), lib.fake_stream(1), lib.fake_stream(0)]
+    rc, first = host.during(lib.aes_batch_plan_launch, plan, None)
+    assert rc == A.AES_OK and len(first) == 1
+    first = first[0]
+    lib.fake_reset()
+    try:
+        last = None
+        for current, ready in ((0, True), (1, False), (1, True)):
+            lib.fake_set_device(current)
+            if ready and current:
+                host.ctx()
+            for s in streams + streams[::-1]:
+                i = lib.fake_launches()
+                lib.fake_other_kernel(s)
+                assert lib.aes_batch_plan_launch(plan, s) == A.AES_OK
+                assert lib.fake_device() == current
+                lib.fake_other_kernel(s)
+                before, got, after = host.launches()[i:]
+                assert (got.name, got.grid, got.args, got.device) == (first.name, first.grid, first.args, 0)
+                assert lib.fake_behind(i + 1, i) and lib.fake_behind(i + 2, i + 1)
+                assert last is None or lib.fake_behind(i + 1, last)
+                last = i + 1
+    finally:
+        lib.fake_set_device(0)
+        lib.aes_batch_plan_destroy(plan)
+
+
+def test_plan_launches_on_one_stream_stay_overlapped(host):
+    """Launches of a plan in a row on one stream wait for no event: each may
+    start while the one before drains."""
+    ctx = host.ctx()
+    plan = ctypes.c_void_p()
+    assert host.lib.aes_batch_plan_create(ctypes.byref(plan), host.descs([(ctx, 0, P, P, 5000)]), 1, None) == A.AES_OK
+    s = host.lib.fake_stream(0)
+    for _ in range(3):
+        rc, got = host.during(host.lib.aes_batch_plan_launch, plan, s)
+        assert rc == A.AES_OK and [(l.programmatic, l.stream) for l in got] == [(1, s)]
+    host.lib.aes_batch_plan_destroy(plan)

@@ -183,12 +183,13 @@ int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_bat
  * synchronise the device), or a runtime that forbids allocation after
  * start-up.  The paper has no counterpart: this is a deployment variant of
  * the batched launch.  Same contract and result as aes_ctr_batch, but the
- * call never allocates or copies: its requests travel in kernel parameters,
- * in launches of at most 500 requests each, so calls share no state and may
- * overlap (other streams, other threads).  The key contexts must already
- * exist on the current device (AES_EINVAL if no context was ever created on
- * it).  The kernel is the T-table batch kernel in the device's tuned T-table
- * shape.  Errors: those of aes_ctr_batch, and AES_ETOOBIG when n exceeds
+ * call never allocates, on the device or the host, and never copies (it takes
+ * 32 KB of stack): its requests travel in kernel parameters, in launches of at
+ * most 500 requests each, so calls share no state and may overlap (other
+ * streams, other threads).  The key contexts must already exist on the current
+ * device (AES_EINVAL if no context was ever created on it).  The kernel is the
+ * T-table batch kernel in the device's tuned T-table shape.  Errors: those of
+ * aes_ctr_batch, and AES_ETOOBIG when n exceeds
  * AES_NOALLOC_MAX_REQUESTS. */
 #define AES_NOALLOC_MAX_REQUESTS 1024
 int aes_ctr_batch_noalloc(const aes_desc_t *descs, int n, void *stream);

@@ -396,10 +396,13 @@ struct BatchSums {
     uint64_t tiles = 0;  // of BatchShape::counted blocks; stays at kMostTiles + 1 once past it
     int64_t bytes = 0;
     // Appends r: sets its first cost, adds its units.
-    void add(BatchReq &r, int variant)
+    void add(BatchReq &r, const BatchShape &s)
     {
-        const uint64_t chunks = chunks_of(r.len, (uint32_t)(r.iv_lo & 255u));
-        const bool bs = variant == AES_VARIANT_BITSLICE;
+        const uint32_t v0 = (uint32_t)(r.iv_lo & 255u);
+        const uint64_t chunks = chunks_of(r.len, v0);
+        const bool bs = s.variant == AES_VARIANT_BITSLICE;
+        if (s.counted)
+            tiles = std::min(tiles + tiles_of(r.len, v0, s.counted), kMostTiles + 1);
         const uint64_t u = bs ? (chunks + BsUnit::kChunks - 1) / BsUnit::kChunks : chunks;
         r.cost_begin = cost;
         cost += u * (bs ? BsUnit::cost(r.nr) : TtUnit::cost(r.nr));
@@ -452,39 +455,46 @@ static BatchShape pick_batch_shape(const DeviceState &st, const aes_batch_opts_t
     return s;
 }
 
+// One request (r.len == 0: no work) after its checks, or the status of the one
+// that failed.
+static int request_of(const aes_desc_t &d, int dev, PayloadChecks &payloads, BatchReq &r, bool *host)
+{
+    r.len = 0;
+    if (!d.ctx || d.ctx->device != dev)
+        return AES_EINVAL;
+    if (!d.len)
+        return AES_OK;
+    const void *din = nullptr;
+    void *dout = nullptr;
+    const int rc = payloads.check(d.in, d.out, d.len, &din, &dout, host);
+    if (rc || !blocks_of(d.len))
+        return rc;
+    r.in = static_cast<const uint4 *>(din);
+    r.out = static_cast<uint4 *>(dout);
+    r.len = d.len;
+    iv_halves(d.iv, &r.iv_hi, &r.iv_lo);
+    r.rk = reinterpret_cast<const uint4 *>(d.ctx->d_rk);
+    r.nr = (uint32_t)d.ctx->nr;
+    r.pad = 0;
+    return AES_OK;
+}
+
 // The non-empty requests of descs[0..n) into out (room for n), their sums into
 // `sum`; the first bad request's status.
 static int fill_reqs(const aes_desc_t *descs, int n, int dev, const BatchShape &s, BatchReq *out, BatchSums &sum)
 {
     PayloadChecks payloads(dev);
     for (int i = 0; i < n; ++i) {
-        const aes_desc_t &d = descs[i];
-        if (!d.ctx)
-            return AES_EINVAL;
-        if (d.ctx->device != dev)
-            return AES_EINVAL;
-        if (!d.len)
-            continue;
-        const void *din = nullptr;
-        void *dout = nullptr;
+        BatchReq r;
         bool host = false;
-        const int rc = payloads.check(d.in, d.out, d.len, &din, &dout, &host);
+        const int rc = request_of(descs[i], dev, payloads, r, &host);
         if (rc)
             return rc;
-        if (!blocks_of(d.len))
+        if (!r.len)
             continue;
-        BatchReq r{};
-        r.in = static_cast<const uint4 *>(din);
-        r.out = static_cast<uint4 *>(dout);
-        r.len = d.len;
-        iv_halves(d.iv, &r.iv_hi, &r.iv_lo);
-        r.rk = reinterpret_cast<const uint4 *>(d.ctx->d_rk);
-        r.nr = (uint32_t)d.ctx->nr;
         sum.host |= host;
-        if (s.counted)
-            sum.tiles = std::min(sum.tiles + tiles_of(r.len, (uint32_t)(r.iv_lo & 255u), s.counted), kMostTiles + 1);
         const size_t at = sum.n;
-        sum.add(r, s.variant);
+        sum.add(r, s);
         out[at] = r;
     }
     return sum.tiles > kMostTiles ? AES_ETOOBIG : AES_OK;
@@ -552,28 +562,46 @@ int batch_by_params(const aes_desc_t *descs, int n, const DeviceState &st, const
         return launch_in_params<kFewInParams>(descs, n, st, s, seed, stream);
     if (n <= kMostInParams)
         return launch_in_params<kMostInParams>(descs, n, st, s, seed, stream);
-    // Nothing runs unless every request is good.
-    std::vector<BatchReq> reqs;
-    try {
-        reqs.resize((size_t)n);
-    } catch (const std::bad_alloc &) {
-        return AES_ENOMEM;
-    }
+    // Nothing runs unless every request is good: one pass checks and counts
+    // them, a second fills the launches (no-alloc callers may have no heap to
+    // hold them in between).  Addresses are looked up again only if some
+    // payload's differs from the one the caller knows it by.
     BatchSums sum;
-    const int rc = fill_reqs(descs, n, st.device, s, reqs.data(), sum);
-    if (rc || !sum.n)
-        return rc;
+    bool as_given = true;
+    PayloadChecks payloads(st.device);
+    for (int i = 0; i < n; ++i) {
+        BatchReq r;
+        bool host = false;
+        const int rc = request_of(descs[i], st.device, payloads, r, &host);
+        if (rc)
+            return rc;
+        if (!r.len)
+            continue;
+        sum.host |= host;
+        sum.add(r, s);
+        as_given &= r.in == descs[i].in && r.out == descs[i].out;
+    }
+    if (sum.tiles > kMostTiles)
+        return AES_ETOOBIG;
     // equal numbers of requests per launch
     const size_t launches = (sum.n + kMostInParams - 1) / kMostInParams;
+    payloads.accept_all = as_given;
     BatchParams<kMostInParams> p;
+    int i = 0;
     for (size_t k = 0; k < launches; ++k) {
-        const size_t a = sum.n * k / launches, b = sum.n * (k + 1) / launches;
+        const size_t want = sum.n * (k + 1) / launches - sum.n * k / launches;
         BatchSums part;
-        part.host = sum.host;
-        for (size_t i = a; i < b; ++i) {
+        while (part.n < want) {
+            BatchReq r;
+            bool host = false;
+            const int rc = request_of(descs[i++], st.device, payloads, r, &host);
+            if (rc)
+                return rc;
+            if (!r.len)
+                continue;
             const size_t at = part.n;
-            part.add(reqs[i], s.variant);
-            p.in_params[at] = reqs[i];
+            part.add(r, s);
+            p.in_params[at] = r;
         }
         const int ctas = set_args(p, part, st, s, seed);
         const cudaError_t e = launch_batch(p, ctas, s, sum.host, stream);

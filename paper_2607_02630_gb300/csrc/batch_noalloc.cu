@@ -8,8 +8,8 @@
 // cudaMalloc/cudaFree (both can synchronise the device), or an embedded
 // runtime that forbids dynamic allocation once it has started.  This entry
 // point passes every request in kernel parameters instead, in as many
-// launches as that takes (500 requests each), so it needs no scratch at all
-// and its calls share no state.  The caller still owns the payload buffers
+// launches as that takes (500 requests each), so it needs no memory, the
+// host's heap included, but 32 KB of stack, and its calls share no state.  The caller still owns the payload buffers
 // and the key contexts (which must exist already: creating them is the only
 // step that allocates).
 #include "../../include/aesoffload.h"

@@ -234,6 +234,11 @@ int PayloadChecks::resolve(const void *p, Range &r, const void **dptr, bool *hos
 int PayloadChecks::check(const void *in, const void *out, size_t len, const void **din, void **dout, bool *host)
 {
     *host = false;
+    if (accept_all) {
+        *din = in;
+        *dout = const_cast<void *>(out);
+        return AES_OK;
+    }
     int rc = check_bounds(in, out, len);
     if (rc || (rc = resolve(in, in_, din, host)))
         return rc;

@@ -58,6 +58,9 @@ public:
     explicit PayloadChecks(int dev) : dev_(dev) {}
     // *host: a payload lies in pinned host memory
     int check(const void *in, const void *out, size_t len, const void **din, void **dout, bool *host);
+    // set once every payload of the call is known to be addressed as given:
+    // check() then only gives the addresses back
+    bool accept_all = false;
 
 private:
     struct Range {

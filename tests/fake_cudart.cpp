@@ -69,6 +69,7 @@ cudaError_t launch(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStrea
         return cudaErrorInvalidResourceHandle;
     if (smem > 49152 && !g_big_smem.count({fn, g_device}))
         return cudaErrorInvalidValue;
+    const long news = g_news;
     Launch l{};
     l.device = g_device;
     l.grid = (int)grid.x;
@@ -79,6 +80,7 @@ cudaError_t launch(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStrea
         std::memcpy(l.args, args[0], sizeof(l.args));
     std::strncpy(l.name, g_names[fn].c_str(), sizeof(l.name) - 1);
     enqueue(st, l);
+    g_news = news;  // the record's own are not the library's
     return cudaSuccess;
 }
 

@@ -194,3 +194,26 @@ def test_plan_launches_on_one_stream_stay_overlapped(host):
         rc, got = host.during(host.lib.aes_batch_plan_launch, plan, s)
         assert rc == A.AES_OK and [(l.programmatic, l.stream) for l in got] == [(1, s)]
     host.lib.aes_batch_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("n", [1, 64, 65, 500, 501, 777, 1024])
+@pytest.mark.parametrize("empty", [0, 3])
+def test_noalloc_allocates_nothing(host, n, empty):
+    """aes_ctr_batch_noalloc takes nothing from the host's heap either, at any
+    request count, makes the launches the one-shot batch makes, and makes none
+    if its last request is bad."""
+    ctxs = [host.ctx(b) for b in (128, 192, 256)]
+    reqs = [(ctxs[i % 3], i & 255, P + (i << 20), P + (i << 20), 0 if empty and i % empty == 0 else 700 + 37 * i)
+            for i in range(n)]
+    d = host.descs(reqs)
+    host.lib.fake_reset()
+    news = host.lib.fake_news()
+    assert host.lib.aes_ctr_batch_noalloc(d, n, None) == A.AES_OK
+    assert host.lib.fake_news() == news
+    got = host.launches()
+    rc, want = host.during(host.lib.aes_ctr_batch_ex, d, n, None, None)
+    assert rc == A.AES_OK and [(l.name, l.grid, l.args) for l in got] == [(l.name, l.grid, l.args) for l in want]
+    work = sum(1 for r in reqs if r[4])
+    assert len(got) == -(-work // 500)
+    bad = host.descs(reqs[:-1] + [(ctxs[0], 0, P + 8, P, 16)])
+    assert host.during(host.lib.aes_ctr_batch_noalloc, bad, n, None) == (A.AES_EALIGN, [])

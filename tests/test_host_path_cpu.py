@@ -217,3 +217,26 @@ def test_noalloc_allocates_nothing(host, n, empty):
     assert len(got) == -(-work // 500)
     bad = host.descs(reqs[:-1] + [(ctxs[0], 0, P + 8, P, 16)])
     assert host.during(host.lib.aes_ctr_batch_noalloc, bad, n, None) == (A.AES_EALIGN, [])
+
+
+@pytest.mark.parametrize("low", [0, 31, 255])
+@pytest.mark.parametrize("bits", [128, 256])
+def test_short_calls_leave_sms_to_others(host, bits, low):
+    """A single call takes one CTA per 4 KiB (8 chunks) it touches, so that
+    calls on many streams or beside the resident server do not each fill the
+    tables of every SM; a CTA of fewer than 8 warps takes a chunk per warp."""
+    ctx = host.ctx(bits)
+    iv = bytes(15) + bytes([low])
+    for n in (1, 16, 4096, 4097, 16384, 61453, 65536, 262144, 600_000, 1 << 20, 8 << 20):
+        rc, got = host.during(host.lib.aes_ctr, ctx, iv, P, P, n, None)
+        assert rc == A.AES_OK and len(got) == 1
+        chunks = (((low + (n + 15) // 16 - 1) >> 5) - (low >> 5)) + 1
+        assert got[0].grid == min(152, -(-chunks // 8))
+        for threads in (32, 96, 256, 1024):
+            shape = A.LaunchShape(1, threads, 1, 0)
+            rc, got = host.during(host.lib.aes_ctr_ex, ctx, iv, P, P, n, None, ctypes.byref(shape))
+            assert rc == A.AES_OK and got[0].grid == min(152, -(-chunks // min(8, threads // 32)))
+        rc, got = host.during(host.lib.aes_ctr, ctx, iv, P, P, n, None)
+        if low == 0:
+            s = A.LaunchShape()
+            assert host.lib.aes_tuned_shape(n, bits, ctypes.byref(s)) == A.AES_OK and s.ctas == got[0].grid

@@ -512,10 +512,17 @@ static int set_args(BatchArgs &p, const BatchSums &sum, const DeviceState &st, c
     p.te0 = st.te0;
     p.order = make_order((sum.cost + p.tile_cost - 1) / p.tile_cost, seed);
     // as many CTAs as are resident at once (one T-table CTA per SM: its
-    // tables take 128 KiB of shared memory), none without a unit of work
-    const int resident = s.variant == AES_VARIANT_BITSLICE ? st.nsm * g_bs_ctas_per_sm : st.nsm;
+    // tables take 128 KiB of shared memory), each with a unit of work at
+    // least.  A T-table CTA gets 8 chunks, one for a warp, as a single call's
+    // does (ctr_ctas): plans of 64 requests of 1 to 16 KiB take 5.16 us in a
+    // row with 1 chunk, 5.13 with 8, 6.81 with 16, and beside the resident
+    // server (4 SMs free) 174, 107 and 70 us; 8 such requests 4.2, 4.6, 5.5
+    // and 107, 25, 17 us.
+    const bool bs = s.variant == AES_VARIANT_BITSLICE;
+    const int resident = bs ? st.nsm * g_bs_ctas_per_sm : st.nsm;
     const int ctas = s.ctas > 0 ? std::min(s.ctas, resident) : resident;
-    return (uint64_t)ctas > sum.units ? (int)sum.units : ctas;
+    const uint64_t per = bs || s.ctas > 0 ? 1 : std::min(8, s.threads / 32);
+    return (int)std::min((uint64_t)ctas, (sum.units + per - 1) / per);
 }
 
 template <int MAXT, bool RK_REGS, int CAP>

@@ -240,3 +240,23 @@ def test_short_calls_leave_sms_to_others(host, bits, low):
         if low == 0:
             s = A.LaunchShape()
             assert host.lib.aes_tuned_shape(n, bits, ctypes.byref(s)) == A.AES_OK and s.ctas == got[0].grid
+
+
+@pytest.mark.parametrize("n,nbytes", [(1, 100), (8, 512), (8, 5000), (64, 6000), (600, 700), (3, 1 << 20), (1100, 64)])
+def test_small_batches_leave_sms_to_others(host, n, nbytes):
+    """A batch of short requests takes one T-table CTA per 8 chunks it
+    touches, as single calls do; a grid that the caller names is kept while
+    every CTA has a chunk."""
+    ctx = host.ctx()
+    d = host.descs([(ctx, 0, P, P, nbytes)] * n)
+    chunks = (nbytes + 511) // 512 * n
+    plan = ctypes.c_void_p()
+    assert host.lib.aes_batch_plan_create(ctypes.byref(plan), d, n, None) == A.AES_OK
+    rc, got = host.during(host.lib.aes_batch_plan_launch, plan, None)
+    assert rc == A.AES_OK and [l.grid for l in got] == [min(152, -(-chunks // 8))]
+    host.lib.aes_batch_plan_destroy(plan)
+    rc, got = host.during(host.lib.aes_ctr_batch_ex, d, n, None, None)
+    per_launch = [-(-(n * (k + 1) // len(got) - n * k // len(got)) * chunks // n // 8) for k in range(len(got))]
+    assert rc == A.AES_OK and [l.grid for l in got] == [min(152, g) for g in per_launch]
+    rc, got = host.during(host.lib.aes_ctr_batch_ex, d, min(n, 64), None, ctypes.byref(A.BatchOpts(1, 512, 256, 40, 0, 1)))
+    assert rc == A.AES_OK and got[0].grid == min(40, chunks // n * min(n, 64))

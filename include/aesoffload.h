@@ -165,7 +165,8 @@ typedef struct {
 
 /* Encrypt n independent requests in ONE kernel launch on `stream`: each CTA
  * owns an equal share of the batch's work, and its warps claim tiles of that
- * share until none are left.  Any mix of key sizes and lengths; each request
+ * share until none are left (plans, and calls with a table in device memory,
+ * of 128 MiB or more: all warps claim tiles of the whole batch).  Any mix of key sizes and lengths; each request
  * follows aes_ctr's contract.  descs is read during the call (it may be
  * reused on return).  Up to 1024 requests travel in kernel parameters (two or
  * three launches past 500 and 1000); more in a descriptor table allocated

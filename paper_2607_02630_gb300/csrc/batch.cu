@@ -3,23 +3,36 @@
 // Work is measured in shared-memory wavefronts, the unit of the kernel's
 // bound: a 32-block chunk (tile.cuh) of a request with Nr rounds costs about
 // 16 (Nr - 2) + 9 of them.  The requests' chunks, one request after the other,
-// are one line of cost; CTA c of G (one per SM) owns the c-th of G equal
-// pieces of it, so every SM gets the same number of lookups whatever the mix
-// of lengths and key sizes, and neither a table of tiles nor a counter in
-// device memory is needed.  In a CTA's piece the warps claim tiles through
-// one counter in shared memory, each tile a warps-th of what is left, at
-// most tile_blocks and at least about one chunk: large tiles amortise a
-// request's set-up, small ones at the end let the warps finish together, and
-// a batch of a few short requests is spread one chunk to a warp.  A warp
-// finds its tile's request by a 32-way search over the requests' first costs.
+// are one line of cost.  Its tiles are claimed in one of two ways.
+//   By pieces: CTA c of G (one per SM) owns the c-th of G equal pieces of the
+// line, so every SM gets the same number of lookups whatever the mix of
+// lengths and key sizes, and neither a table of tiles nor a counter in device
+// memory is needed.  The CTA's warps claim tiles of the piece through one
+// counter in shared memory, each tile a warps-th of what is left, at most
+// tile_blocks and at least about one chunk: large tiles amortise a request's
+// set-up, small ones at the end let the warps finish together, and a batch of
+// a few short requests is spread one chunk to a warp.
+//   From the whole line (WHOLE): every warp of the grid claims through one
+// counter in device memory, each tile a share of what the line has left, at
+// least 4 chunks.  SMs that other work holds, or that get less of the host
+// link, then cost only their own share (measured at kWholeFrom); a claim costs
+// a trip to L2 and back instead of one to shared memory.
+// A warp finds its tile's request by a 32-way search over the requests' first
+// costs.
+//
 // The cipher is the same T-table round code as the single-buffer kernel.
 // Round keys: CTAs of up to 512 threads (the default) hold the current
 // request's schedule in registers, so the shared-memory pipe, the kernel's
 // bound, serves lookups only; larger CTAs stage it in each warp's slice of
 // shared memory (one broadcast wavefront per round).
 //
-// The bitsliced kernel cuts its work the same way, in passes of 1024 blocks,
-// as the autotuner's alternative to the T-tables.
+// The bitsliced kernel, the autotuner's alternative to the T-tables, cuts its
+// work in passes of 1024 blocks: by pieces where the requests are in kernel
+// parameters, else one pass to a claim from the whole line: 4096 requests of
+// 1 KiB to 8 MiB 22.9 ms, by pieces 32.3, two passes to a claim 38.4 (probably
+// because the warps of an SM then run the same unrolled rounds, of one key
+// size, at the same time: the more neighbouring passes run together, the
+// faster).
 //
 // With a tile order (a test aid) the line is cut into equal tiles instead,
 // and tile t is processed as tile (a*t + b) mod T for a host-chosen a coprime
@@ -57,6 +70,7 @@ struct TileOrder {
 // them, the transposes and the payload (323 and 254 GB/s at 10 and 14 rounds
 // on a 256 MiB buffer).
 struct TtUnit {
+    static constexpr bool kEven = false;
     static constexpr uint32_t kChunks = 1;
     __host__ __device__ static constexpr uint32_t cost(uint32_t nr) { return 16u * (nr - 2u) + 9u; }
     static __device__ __forceinline__ uint32_t run(uint64_t iv_lo, uint64_t k0, uint64_t nk)
@@ -64,9 +78,12 @@ struct TtUnit {
         return aestile::run_chunks(iv_lo, k0, nk);
     }
 };
-struct BsUnit {
+// EVEN: every pass counts 1, for launches whose warps claim passes one by one.
+template <bool EVEN>
+struct BsUnitOf {
+    static constexpr bool kEven = EVEN;
     static constexpr uint32_t kChunks = 32;
-    __host__ __device__ static constexpr uint32_t cost(uint32_t nr) { return 16u * (nr + 5u); }
+    __host__ __device__ static constexpr uint32_t cost(uint32_t nr) { return EVEN ? 1u : 16u * (nr + 5u); }
     static __device__ __forceinline__ uint32_t run(uint64_t, uint64_t, uint64_t nk)
     {
         return nk < kChunks ? (uint32_t)nk : kChunks;
@@ -92,6 +109,9 @@ struct BatchArgs {
     uint64_t total_cost;
     uint64_t tile_cost;  // largest tile
     const uint32_t *te0;
+    // Kernels that claim from the whole line (CAP == 0): this launch's counter,
+    // zero when it starts, and the next one's, which it clears.
+    unsigned long long *claimed, *cleared;
     TileOrder order;
 };
 template <int CAP>
@@ -149,10 +169,10 @@ struct WarpState {
 };
 
 // The warp's next run: n > 0 chunks from chunk k0 on of request rq (every
-// lane gets the same), or false when the CTA's piece is done.  s_pos: the
-// CTA's counter; st: this warp's state; both zeroed before the CTA's last
-// barrier.
-template <class UNIT>
+// lane gets the same), or false when the CTA's piece (WHOLE: the line) is done.
+// s_pos: the counter of the CTA's piece; st: this warp's state; both zeroed
+// before the CTA's last barrier.
+template <class UNIT, bool WHOLE>
 __device__ __forceinline__ bool next_run(const BatchArgs &p, const BatchReq *reqs, unsigned long long *s_pos,
                                          WarpState *st, BatchReq &rq, uint64_t &k0, uint32_t &n)
 {
@@ -163,19 +183,22 @@ __device__ __forceinline__ bool next_run(const BatchArgs &p, const BatchReq *req
     __syncwarp();  // before lane 0 writes the next
     for (;;) {
         bool near = true;  // the request is probably the last one or one of the next
-        if (xa >= xb) {    // claim a tile of this CTA's piece [u0, u0 + size)
+        if (xa >= xb) {    // claim a tile of [u0, u0 + size)
             const uint64_t units = p.order.tiles ? p.order.tiles : p.total_cost;
             const uint64_t q = units / gridDim.x, r = units % gridDim.x;
-            const uint64_t u0 = q * blockIdx.x + (blockIdx.x < r ? blockIdx.x : r);
-            const uint64_t size = q + (blockIdx.x < r ? 1 : 0);
+            const uint64_t u0 = WHOLE ? 0 : q * blockIdx.x + (blockIdx.x < r ? blockIdx.x : r);
+            const uint64_t size = WHOLE ? units : q + (blockIdx.x < r ? 1 : 0);
             unsigned long long at = 0, take = 1;
             if (lane == 0) {
-                if (!p.order.tiles) {
-                    const unsigned long long cur = *(volatile unsigned long long *)s_pos;
-                    take = cur < size ? (size - cur) / (blockDim.x >> 5) : 0;
-                    take = take < UNIT::cost(10) ? UNIT::cost(10) : take > p.tile_cost ? p.tile_cost : take;
+                unsigned long long *pos = WHOLE ? p.claimed : s_pos;
+                if (!p.order.tiles && !UNIT::kEven) {
+                    const unsigned long long cur = *(volatile unsigned long long *)pos;
+                    const uint32_t warps = (blockDim.x >> 5) * (WHOLE ? gridDim.x : 1u);
+                    const uint32_t least = (WHOLE ? 4u : 1u) * UNIT::cost(10);
+                    take = cur < size ? (size - cur) / warps : 0;
+                    take = take < least ? least : take > p.tile_cost ? p.tile_cost : take;
                 }
-                at = atomicAdd(s_pos, take);
+                at = atomicAdd(pos, take);
             }
             at = __shfl_sync(0xffffffffu, at, 0);
             take = __shfl_sync(0xffffffffu, take, 0);
@@ -228,7 +251,7 @@ __device__ __forceinline__ bool next_run(const BatchArgs &p, const BatchReq *req
 // alone and 3 % slower on AES-128.  MAXT: largest CTA it is launched with;
 // RK_REGS: round keys in registers (else in the warp's slice of shared
 // memory); HOST: some payload lies in pinned host memory.
-template <int MAXT, bool RK_REGS, int CAP, bool HOST>
+template <int MAXT, bool RK_REGS, int CAP, bool HOST, bool WHOLE>
 __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_constant__ BatchParams<CAP> p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -244,6 +267,8 @@ __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_cons
     aestt::fill_tables(smem, p.te0);
     __syncthreads();
     aesdev::wait_for_previous_launch();
+    if (WHOLE && blockIdx.x == 0 && threadIdx.x == 0)
+        *p.cleared = 0;
     const aestt::Lanes ln(smem);
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     uint4 *w_group = s_group[warp];
@@ -268,7 +293,7 @@ __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_cons
     BatchReq rq;
     uint64_t k0;
     uint32_t n;
-    while (next_run<TtUnit>(p, p.requests(), &s_pos, &s_state[warp], rq, k0, n)) {
+    while (next_run<TtUnit, WHOLE>(p, p.requests(), &s_pos, &s_state[warp], rq, k0, n)) {
         switch (rq.nr) {
         case 10: xor_with(rq, k0, n, std::integral_constant<int, 10>()); break;
         case 12: xor_with(rq, k0, n, std::integral_constant<int, 12>()); break;
@@ -294,13 +319,15 @@ __global__ void __launch_bounds__(kBsThreads) batch_bitslice_kernel(const __grid
         s_state[threadIdx.x] = WarpState{0, 0, 0, 0};
     __syncthreads();
     aesdev::wait_for_previous_launch();
+    if (CAP == 0 && blockIdx.x == 0 && threadIdx.x == 0)
+        *p.cleared = 0;
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t *mask = s_mask[threadIdx.x >> 5];
     const uint4 *cur = nullptr;  // schedule whose masks are in `mask`
     BatchReq rq;
     uint64_t k0;
     uint32_t n;
-    while (next_run<BsUnit>(p, p.requests(), &s_pos, &s_state[threadIdx.x >> 5], rq, k0, n)) {
+    while (next_run<BsUnitOf<CAP == 0>, CAP == 0>(p, p.requests(), &s_pos, &s_state[threadIdx.x >> 5], rq, k0, n)) {
         const uint64_t v0 = rq.iv_lo & 255u, nb = (rq.len + 15) >> 4;
         const uint64_t first = k0 << 5 > v0 ? (k0 << 5) - v0 : 0;
         const uint64_t end = ((k0 + n) << 5) - v0, last = end < nb ? end : nb;
@@ -321,13 +348,15 @@ __global__ void __launch_bounds__(kBsThreads) batch_bitslice_kernel(const __grid
     }
 }
 
-template <int MAXT, bool RK_REGS, int CAP>
+template <int MAXT, bool RK_REGS, int CAP, bool WHOLE = false>
 cudaError_t set_smem()
 {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    const cudaError_t e = cudaFuncSetAttribute(batch_ttable_kernel<MAXT, RK_REGS, CAP, false>, attr,
+    const cudaError_t e = cudaFuncSetAttribute(batch_ttable_kernel<MAXT, RK_REGS, CAP, false, WHOLE>, attr,
                                                (int)aestt::kTableBytes);
-    return e ? e : cudaFuncSetAttribute(batch_ttable_kernel<MAXT, RK_REGS, CAP, true>, attr, (int)aestt::kTableBytes);
+    return e ? e
+             : cudaFuncSetAttribute(batch_ttable_kernel<MAXT, RK_REGS, CAP, true, WHOLE>, attr,
+                                    (int)aestt::kTableBytes);
 }
 
 int g_bs_ctas_per_sm = 1;  // resident bitsliced batch CTAs per SM (set with the attributes)
@@ -340,7 +369,8 @@ cudaError_t batch_set_attributes()
 {
     cudaError_t e;
     if ((e = set_smem<kRegsMaxThreads, true, 0>()) || (e = set_smem<kRegsMaxThreads, true, kFewInParams>()) ||
-        (e = set_smem<kRegsMaxThreads, true, kMostInParams>()) || (e = set_smem<1024, false, 0>()) ||
+        (e = set_smem<kRegsMaxThreads, true, kMostInParams>()) || (e = set_smem<kRegsMaxThreads, true, 0, true>()) ||
+        (e = set_smem<1024, false, 0>()) || (e = set_smem<1024, false, 0, true>()) ||
         (e = set_smem<1024, false, kMostInParams>()))
         return e;
     int per_sm = 0;
@@ -388,10 +418,21 @@ static TileOrder make_order(uint64_t total, uint32_t seed)
     return o;
 }
 
+// From so many units on (chunks; 128 MiB) a launch with its table in device
+// memory claims from the whole line.  Plans in a row, by pieces and from the
+// whole line, on a free GPU and beside a server that holds 52 of the 152 SMs:
+// 96 requests of 1 to 2 MiB (140 MB) 169.2 and 171.1 us, 335 and 267; 256 of
+// 1 KiB to 8 MiB 341.4 and 341.6, 679 and 524; 4096 of them 4262 and 4237, 8471
+// and 6439; 300 of them in pinned host memory 2126 and 2092, 2069 and 1974.
+// Below it the claims show: 46 MB 62.6 and 68.9 on a free GPU (122.7 and 105.8
+// beside the server), 16 MB 24.1 and 29.3 (47.2 and 46.3).
+constexpr uint64_t kWholeFrom = 1u << 18;
+
 // What a launch needs to know of its requests.
 struct BatchSums {
     size_t n = 0;       // requests that hold any bytes
-    bool host = false;  // some payload lies in pinned host memory
+    bool table = false;  // for a launch with its table in device memory
+    bool host = false;   // some payload lies in pinned host memory
     uint64_t cost = 0, units = 0;
     uint64_t tiles = 0;  // of BatchShape::counted blocks; stays at kMostTiles + 1 once past it
     int64_t bytes = 0;
@@ -403,9 +444,9 @@ struct BatchSums {
         const bool bs = s.variant == AES_VARIANT_BITSLICE;
         if (s.counted)
             tiles = std::min(tiles + tiles_of(r.len, v0, s.counted), kMostTiles + 1);
-        const uint64_t u = bs ? (chunks + BsUnit::kChunks - 1) / BsUnit::kChunks : chunks;
+        const uint64_t u = bs ? (chunks + 31) / 32 : chunks;
         r.cost_begin = cost;
-        cost += u * (bs ? BsUnit::cost(r.nr) : TtUnit::cost(r.nr));
+        cost += u * (!bs ? TtUnit::cost(r.nr) : table ? BsUnitOf<true>::cost(r.nr) : BsUnitOf<false>::cost(r.nr));
         units += u;
         bytes += (int64_t)r.len;
         ++n;
@@ -504,11 +545,13 @@ static int fill_reqs(const aes_desc_t *descs, int n, int dev, const BatchShape &
 static int set_args(BatchArgs &p, const BatchSums &sum, const DeviceState &st, const BatchShape &s, uint32_t seed)
 {
     p.reqs = nullptr;
+    p.claimed = p.cleared = nullptr;
     p.n = (uint32_t)sum.n;
     p.total_cost = sum.cost;
-    p.tile_cost = s.variant == AES_VARIANT_BITSLICE
-                      ? (uint64_t)std::max(1, s.tile_blocks / 1024) * BsUnit::cost(10)
-                      : (uint64_t)(s.tile_blocks / 32) * TtUnit::cost(10);
+    const bool bs = s.variant == AES_VARIANT_BITSLICE;
+    p.tile_cost = !bs         ? (uint64_t)(s.tile_blocks / 32) * TtUnit::cost(10)
+                  : sum.table ? BsUnitOf<true>::cost(10)
+                              : (uint64_t)std::max(1, s.tile_blocks / 1024) * BsUnitOf<false>::cost(10);
     p.te0 = st.te0;
     p.order = make_order((sum.cost + p.tile_cost - 1) / p.tile_cost, seed);
     // as many CTAs as are resident at once (one T-table CTA per SM: its
@@ -518,20 +561,34 @@ static int set_args(BatchArgs &p, const BatchSums &sum, const DeviceState &st, c
     // row with 1 chunk, 5.13 with 8, 6.81 with 16, and beside the resident
     // server (4 SMs free) 174, 107 and 70 us; 8 such requests 4.2, 4.6, 5.5
     // and 107, 25, 17 us.
-    const bool bs = s.variant == AES_VARIANT_BITSLICE;
     const int resident = bs ? st.nsm * g_bs_ctas_per_sm : st.nsm;
     const int ctas = s.ctas > 0 ? std::min(s.ctas, resident) : resident;
     const uint64_t per = bs || s.ctas > 0 ? 1 : std::min(8, s.threads / 32);
     return (int)std::min((uint64_t)ctas, (sum.units + per - 1) / per);
 }
 
+// The table in device memory and, in one more entry behind it, the counters of
+// a kernel that claims from the whole line; both are zero before its first launch.
+static size_t table_entries(const BatchSums &sum) { return sum.n + 1; }
+static void set_table(BatchParams<0> &p, BatchReq *table, const BatchSums &sum, const BatchShape &s)
+{
+    p.reqs = table;
+    if (s.variant == AES_VARIANT_BITSLICE || sum.units >= kWholeFrom) {
+        p.claimed = reinterpret_cast<unsigned long long *>(table + sum.n);
+        p.cleared = p.claimed + 1;
+    }
+}
+
 template <int MAXT, bool RK_REGS, int CAP>
 static cudaError_t launch_ttable(const BatchParams<CAP> &p, int ctas, int threads, bool host, cudaStream_t stream)
 {
-    return host ? launch_overlapped(batch_ttable_kernel<MAXT, RK_REGS, CAP, true>, ctas, threads, aestt::kTableBytes,
-                                    stream, p)
-                : launch_overlapped(batch_ttable_kernel<MAXT, RK_REGS, CAP, false>, ctas, threads, aestt::kTableBytes,
-                                    stream, p);
+    auto kernel = host ? batch_ttable_kernel<MAXT, RK_REGS, CAP, true, false>
+                       : batch_ttable_kernel<MAXT, RK_REGS, CAP, false, false>;
+    if constexpr (CAP == 0)
+        if (p.claimed)
+            kernel = host ? batch_ttable_kernel<MAXT, RK_REGS, CAP, true, true>
+                          : batch_ttable_kernel<MAXT, RK_REGS, CAP, false, true>;
+    return launch_overlapped(kernel, ctas, threads, aestt::kTableBytes, stream, p);
 }
 
 template <int CAP>
@@ -687,6 +744,7 @@ struct aes_batch_plan_s {
             return e;
         launched = true;
         last_id = id;
+        std::swap(params.claimed, params.cleared);
         return cudaEventRecord(done, stream);
     }
 
@@ -747,21 +805,22 @@ int aes_ctr_batch_ex(const aes_desc_t *descs, int n, void *stream, const aes_bat
         return batch_by_params(descs, n, *st, s, seed, cs);
     std::vector<BatchReq> host;
     try {
-        host.resize((size_t)n);
+        host.resize((size_t)n + 1);
     } catch (const std::bad_alloc &) {
         return AES_ENOMEM;
     }
     BatchSums sum;
+    sum.table = true;
     if ((rc = fill_reqs(descs, n, st->device, s, host.data(), sum)) || !sum.n)
         return rc;
     BatchParams<0> p{};
     const int ctas = set_args(p, sum, *st, s, seed);
     BatchReq *reqs = nullptr;
-    const size_t bytes = sum.n * sizeof(BatchReq);
+    const size_t bytes = table_entries(sum) * sizeof(BatchReq);
     cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&reqs), bytes, st->pool, cs);
     if (e)
         return e == cudaErrorMemoryAllocation ? AES_ENOMEM : cuda_fail(e, "cudaMallocFromPoolAsync");
-    p.reqs = reqs;
+    set_table(p, reqs, sum, s);
     // Pageable source: the copy has finished reading the host vector when
     // cudaMemcpyAsync returns, so it may be destroyed afterwards.
     e = cudaMemcpyAsync(reqs, host.data(), bytes, cudaMemcpyHostToDevice, cs);
@@ -802,9 +861,10 @@ int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
         return AES_ENOMEM;
     plan->device = st->device;
     plan->shape = s;
+    plan->sum.table = true;
     std::vector<BatchReq> host;
     try {
-        host.resize((size_t)n);
+        host.resize((size_t)n + 1);
     } catch (const std::bad_alloc &) {
         delete plan;
         return AES_ENOMEM;
@@ -814,7 +874,7 @@ int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
         return rc;
     }
     if (plan->sum.n) {
-        const size_t bytes = plan->sum.n * sizeof(BatchReq);
+        const size_t bytes = table_entries(plan->sum) * sizeof(BatchReq);
         cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&plan->reqs), bytes);
         if (e) {
             delete plan;
@@ -830,7 +890,7 @@ int aes_batch_plan_create(aes_batch_plan_t *out, const aes_desc_t *descs, int n,
             return cuda_fail(e, "aes_batch_plan_create");
         }
         plan->ctas = set_args(plan->params, plan->sum, *st, s, opts ? opts->tile_order_seed : 0);
-        plan->params.reqs = plan->reqs;
+        set_table(plan->params, plan->reqs, plan->sum, s);
     }
     *out = plan;
     return AES_OK;

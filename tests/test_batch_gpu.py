@@ -366,3 +366,43 @@ def test_plan_launches_are_ordered_across_streams(cuda, aes):
     for key, b, iv, o, k in meta:
         np.testing.assert_array_equal(out[o: o + k], oracle.ctr(key, b, iv, payload[o: o + k]))
     plan.close()
+
+
+def test_claims_from_the_whole_line(cuda, aes, ncpu):
+    """Plans and one-shot tables of 2^18 chunks and more, whose warps claim
+    from the whole batch through one counter in device memory, launched
+    several times (two counters take turns): device and pinned payloads, keys
+    in registers and in shared memory, seeded tile orders, the bitsliced
+    kernel; short, empty and tailed requests among long ones, all key sizes."""
+    g = W.rng(5800)
+    n = 1100
+    lengths = [int(x) for x in np.exp(g.uniform(np.log(64), np.log(1 << 20), n))]
+    lengths[0] = lengths[-1] = lengths[500] = 0
+    lengths[7] = (9 << 20) + 5
+    lengths[900] = max((1 << 27) + 4096 - sum(lengths), 16)
+    bits = [(128, 192, 256)[int(x)] for x in g.integers(0, 3, n)]
+    kinds = [("random", "low32", "low64", "wrap128")[i % 4] for i in range(n)]
+    reqs, meta, payload, src, dst = make_requests(cuda, aes, g, lengths, bits, kinds)
+    cuda.cuda.synchronize()
+    hsrc, hdst = src.cpu().pin_memory(), dst.cpu().pin_memory()
+    h = [(c, iv, hsrc.data_ptr() + o, hdst.data_ptr() + o, k) for (c, iv, _, _, k), (_, _, _, o, _) in zip(reqs, meta)]
+    want = np.full(payload.size, 0xA5, np.uint8)
+    for key, b, iv, o, k in meta:
+        want[o: o + k] = oracle.ctr_mt(key, b, iv, payload[o: o + k], ncpu if k > 1 << 16 else 1)
+    for pinned in (False, True):
+        r, out = (h, hdst) if pinned else (reqs, dst)
+        for opts in ({}, {"threads": 1024}, {"tile_order_seed": 3}, {"tile_order_seed": 8, "tile_blocks": 256},
+                     {"variant": 2}, {"variant": 2, "tile_order_seed": 5}):
+            plan = aes.BatchPlan(r, **opts)
+            for launch in (plan.launch, plan.launch, lambda: aes.batch(r, **opts), plan.launch):
+                out.fill_(0xA5)
+                cuda.cuda.synchronize()
+                launch()
+                cuda.cuda.synchronize()
+                assert np.array_equal(out.cpu().numpy(), want), (pinned, opts)
+            plan.launch()  # in a row, on two streams
+            plan.launch(cuda.cuda.Stream())
+            plan.launch()
+            cuda.cuda.synchronize()
+            assert np.array_equal(out.cpu().numpy(), want), (pinned, opts)
+            plan.close()

@@ -16,8 +16,14 @@ P = 0x7F00_0000_0000  # a payload address (nothing reads it)
 
 class Launch(ctypes.Structure):
     _fields_ = [("device", ctypes.c_int), ("grid", ctypes.c_int), ("block", ctypes.c_int),
-                ("programmatic", ctypes.c_int), ("stream", ctypes.c_uint64), ("args", ctypes.c_char * 64),
+                ("programmatic", ctypes.c_int), ("stream", ctypes.c_uint64), ("args", ctypes.c_uint64 * 8),
                 ("name", ctypes.c_char * 128)]
+
+    def raw(self, n=64):
+        b = bytes(self.args)
+        if b"BatchParams" in self.name:
+            b = b[:12] + bytes(4) + b[16:]  # padding behind the request count
+        return b[:n]
 
 
 class Host:
@@ -113,7 +119,7 @@ def test_length_whose_end_wraps_is_no_work(host, low, below):
     for call in (lambda d: host.lib.aes_ctr_batch_ex(d, 2, None, None),
                  lambda d: host.lib.aes_ctr_batch_noalloc(d, 2, None)):
         rc, got = host.during(call, two)
-        assert rc == A.AES_OK and [(l.grid, l.args) for l in got] == [(l.grid, l.args) for l in want]
+        assert rc == A.AES_OK and [(l.grid, l.raw()) for l in got] == [(l.grid, l.raw()) for l in want]
 
 
 def _opts(variant=0, tile_blocks=0):
@@ -174,7 +180,7 @@ def test_plan_stays_on_its_device_and_in_order(host, variant):
                 assert lib.fake_device() == current
                 lib.fake_other_kernel(s)
                 before, got, after = host.launches()[i:]
-                assert (got.name, got.grid, got.args, got.device) == (first.name, first.grid, first.args, 0)
+                assert (got.name, got.grid, got.raw(40), got.device) == (first.name, first.grid, first.raw(40), 0)
                 assert lib.fake_behind(i + 1, i) and lib.fake_behind(i + 2, i + 1)
                 assert last is None or lib.fake_behind(i + 1, last)
                 last = i + 1
@@ -212,7 +218,7 @@ def test_noalloc_allocates_nothing(host, n, empty):
     assert host.lib.fake_news() == news
     got = host.launches()
     rc, want = host.during(host.lib.aes_ctr_batch_ex, d, n, None, None)
-    assert rc == A.AES_OK and [(l.name, l.grid, l.args) for l in got] == [(l.name, l.grid, l.args) for l in want]
+    assert rc == A.AES_OK and [(l.name, l.grid, l.raw()) for l in got] == [(l.name, l.grid, l.raw()) for l in want]
     work = sum(1 for r in reqs if r[4])
     assert len(got) == -(-work // 500)
     bad = host.descs(reqs[:-1] + [(ctxs[0], 0, P + 8, P, 16)])
@@ -260,3 +266,24 @@ def test_small_batches_leave_sms_to_others(host, n, nbytes):
     assert rc == A.AES_OK and [l.grid for l in got] == [min(152, g) for g in per_launch]
     rc, got = host.during(host.lib.aes_ctr_batch_ex, d, min(n, 64), None, ctypes.byref(A.BatchOpts(1, 512, 256, 40, 0, 1)))
     assert rc == A.AES_OK and got[0].grid == min(40, chunks // n * min(n, 64))
+
+
+def test_whole_line_counters_take_turns(host):
+    """A plan that claims from the whole line (T-tables from 2^18 chunks on,
+    the bitsliced kernel always) hands each launch the counter that the one
+    before cleared; smaller T-table plans have none."""
+    ctx = host.ctx()
+    for variant, n, whole in ((1, (1 << 27) - 512, False), (1, 1 << 27, True), (2, 5000, True), (1, 5000, False)):
+        d = host.descs([(ctx, 0, P, P, n)])
+        plan = ctypes.c_void_p()
+        assert host.lib.aes_batch_plan_create(ctypes.byref(plan), d, 1, _opts(variant)) == A.AES_OK
+        host.lib.fake_reset()
+        for _ in range(3):
+            assert host.lib.aes_batch_plan_launch(plan, None) == A.AES_OK
+        pairs = [tuple(l.args[5:7]) for l in host.launches()]  # claimed, cleared
+        if whole:
+            a, b = pairs[0]
+            assert a and b and a != b and pairs == [(a, b), (b, a), (a, b)]
+        else:
+            assert pairs == [(0, 0)] * 3
+        host.lib.aes_batch_plan_destroy(plan)

@@ -213,17 +213,16 @@ int PayloadChecks::resolve(const void *p, Range &r, const void **dptr, bool *hos
 {
     const uintptr_t a = (uintptr_t)p;
     if (a >= r.begin && a < r.end) {
-        r.misses = 0;
+        ++saved_;
         *dptr = p;
         return AES_OK;
     }
     bool is_host = false;
     const int rc = resolve_ptr(p, dev_, dptr, &is_host);
     *host |= is_host;
-    // payloads spread over many allocations: stop looking for their bounds
-    if (rc || is_host || *dptr != p || r.misses > 4)
+    if (rc || is_host || *dptr != p || saved_ < kLookup)
         return rc;
-    ++r.misses;
+    saved_ -= kLookup;
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess || at.type != cudaMemoryTypeDevice ||
         !allocation_bounds(p, &r.begin, &r.end))

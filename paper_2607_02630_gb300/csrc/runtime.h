@@ -50,8 +50,11 @@ int check_payload(const void *in, const void *out, size_t len, int dev, const vo
 // check_payload for the requests of one batch call.  Asking the driver about
 // a pointer costs 0.09 us, two of them per request; a batch's payloads mostly
 // lie in one or two allocations, so the call remembers the bounds of the last
-// allocation each of the inputs and the outputs were found in, and asks again
-// only for a pointer outside them.  Lives on the stack of one call, during
+// allocation that the inputs and the outputs were looked up in, and asks only
+// for pointers outside them.  A lookup of bounds costs as much as a dozen
+// queries: beyond the first two, one is made when so many have been saved, so
+// that payloads spread over many allocations cost what asking for each of them
+// does.  Lives on the stack of one call, during
 // which the caller keeps the payloads allocated.
 class PayloadChecks {
 public:
@@ -65,10 +68,11 @@ public:
 private:
     struct Range {
         uintptr_t begin = 0, end = 0;
-        int misses = 0;
     };
+    static constexpr int64_t kLookup = 13;  // a lookup of bounds, in queries
     int resolve(const void *p, Range &r, const void **dptr, bool *host);
     int dev_;
+    int64_t saved_ = 2 * kLookup;  // queries that a lookup may still be paid with
     Range in_, out_;
 };
 void iv_halves(const uint8_t *iv, uint64_t *hi, uint64_t *lo);

@@ -37,6 +37,8 @@ struct Event {
 };
 
 int g_device = 0, g_sms = 152;
+size_t g_segment = 1ull << 40;    // size of an allocation that payloads lie in
+long g_queries = 0, g_lookups = 0;  // pointers asked about, allocations looked up
 std::atomic<long> g_news{0};
 std::vector<Launch> g_log;
 std::vector<std::set<int>> g_before;  // of each launch: those it runs behind
@@ -116,8 +118,12 @@ void *fake_stream(int device)
     g_streams.insert(s);
     return s;
 }
+void fake_set_segment(size_t bytes) { g_segment = bytes; }
+long fake_queries() { return g_queries; }
+long fake_lookups() { return g_lookups; }
 void fake_reset()
 {
+    g_queries = g_lookups = 0;
     g_log.clear();
     g_before.clear();
     for (Stream &n : g_null)
@@ -167,15 +173,34 @@ cudaError_t cudaMemset(void *p, int v, size_t n) { return std::memset(p, v, n), 
 cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t) { return cudaMemset(p, v, n); }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p)
 {
+    ++g_queries;
     std::memset(a, 0, sizeof(*a));
     a->type = cudaMemoryTypeDevice;
     a->devicePointer = const_cast<void *>(p);
     return cudaSuccess;  // every address is memory of device 0
 }
-cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **, unsigned, unsigned long long,
-                                             cudaDriverEntryPointQueryResult *)
+// the driver calls behind an allocation's bounds: allocations of g_segment bytes
+static int retain(void *, void *) { return 1; }  // not of mapped ranges
+static int release(unsigned long long) { return 0; }
+static int attribute(void *v, int, unsigned long long) { return *(void **)v = nullptr, 0; }
+static int range(unsigned long long *base, size_t *size, unsigned long long p)
 {
-    return cudaErrorNotSupported;
+    ++g_lookups;
+    *base = p / g_segment * g_segment;
+    *size = g_segment;
+    return 0;
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char *name, void **fn, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult *r)
+{
+    const std::string n = name;
+    *fn = n == "cuMemGetAddressRange"          ? (void *)range
+          : n == "cuPointerGetAttribute"       ? (void *)attribute
+          : n == "cuMemRetainAllocationHandle" ? (void *)retain
+          : n == "cuMemRelease"                ? (void *)release
+                                               : nullptr;
+    *r = *fn ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+    return cudaSuccess;
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned)
 {

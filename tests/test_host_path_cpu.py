@@ -86,7 +86,10 @@ def host(built):
     lib.fake_launch.argtypes = [ci, vp]
     lib.fake_stream.restype = vp
     lib.fake_other_kernel.argtypes = [vp]
-    lib.fake_news.restype = ctypes.c_long
+    for f in (lib.fake_news, lib.fake_queries, lib.fake_lookups):
+        f.restype = ctypes.c_long
+    lib.fake_set_segment.argtypes = [sz]
+    lib.fake_set_segment(1 << 40)
     lib.fake_set_device(0)
     lib.fake_reset()
     return Host(lib)
@@ -287,3 +290,28 @@ def test_whole_line_counters_take_turns(host):
         else:
             assert pairs == [(0, 0)] * 3
         host.lib.aes_batch_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("n", [40, 1000])
+@pytest.mark.parametrize("segment", [1 << 40, 64 << 20, 20 << 20, 6 << 20, 4 << 20, 2 << 20])
+@pytest.mark.parametrize("stride", [1, 7])
+def test_payload_checks_pay_for_themselves(host, n, segment, stride):
+    """What a batch spends on its payload pointers, in pointer queries with a
+    lookup of an allocation's bounds counted as 12 (about 1 and 0.09 us): next
+    to nothing where the payloads share an allocation, and never much more
+    than the two queries a request that need no bounds, however the payloads
+    are spread over allocations."""
+    host.lib.fake_set_segment(segment)
+    ctx = host.ctx()
+    reqs = []
+    for i in range(n):
+        at = P + (i * stride % n) * (4 << 20)
+        reqs.append((ctx, 0, at, at + (2 << 20), 2000))
+    d = host.descs(reqs)
+    for call in (lambda: host.lib.aes_ctr_batch_ex(d, n, None, None), lambda: host.lib.aes_ctr_batch_noalloc(d, n, None)):
+        host.lib.fake_reset()
+        assert call() == A.AES_OK
+        cost = host.lib.fake_queries() + 12 * host.lib.fake_lookups()
+        assert cost <= 2 * n + 60
+        if segment >= n * (4 << 20):
+            assert cost <= 60

@@ -247,8 +247,12 @@ def _current_stream() -> int:
     if _raw_stream is None:
         import torch
         torch.cuda.init()  # as torch.cuda.current_stream does
-        device, raw = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
-        _raw_stream = lambda: raw(device())  # noqa: E731
+        device = getattr(torch._C, "_cuda_getDevice", None)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if device and raw:
+            _raw_stream = lambda: raw(device())  # noqa: E731
+        else:  # torch's own, not its interface: a version without them
+            _raw_stream = lambda: int(torch.cuda.current_stream().cuda_stream)  # noqa: E731
     return _raw_stream()
 
 

@@ -228,3 +228,20 @@ def test_descriptor_marshalling():
         with pytest.raises(ValueError):
             A._descs([(Ctx(1), bad, 0, 0, 0)])
     assert ctypes.sizeof(A._descs([])) >= ctypes.sizeof(A.Desc)
+
+
+@pytest.mark.parametrize("missing", ["", "_cuda_getDevice", "_cuda_getCurrentRawStream"])
+def test_current_stream_without_torch_internals(monkeypatch, missing):
+    """The current stream's handle comes from torch's internal calls where they
+    exist, else from torch.cuda.current_stream()."""
+    import sys
+    import types
+
+    internals = {"_cuda_getDevice": lambda: 3, "_cuda_getCurrentRawStream": lambda d: 100 + d}
+    internals.pop(missing, None)
+    fake = types.SimpleNamespace(
+        _C=types.SimpleNamespace(**internals),
+        cuda=types.SimpleNamespace(init=lambda: None, current_stream=lambda: types.SimpleNamespace(cuda_stream=77)))
+    monkeypatch.setitem(sys.modules, "torch", fake)
+    monkeypatch.setattr(A, "_raw_stream", None)
+    assert [A.stream_handle(None) for _ in range(2)] == [77 if missing else 103] * 2

@@ -153,7 +153,10 @@ typedef struct {
                            to 512 the warps keep round keys in registers,
                            above it in shared memory; the bitsliced kernel
                            takes 128 only */
-    int tile_blocks;    /* 16-byte blocks of the largest work tile: a multiple of 256 */
+    int tile_blocks;    /* 16-byte blocks of the largest work tile: a multiple of
+                           256 (T-table tiles of more than 3968 are rounded to
+                           runs of 7936; the bitsliced kernel's are passes of
+                           1024, one at a time in plans) */
     int ctas;           /* CTAs; 0 = one per SM (x occupancy) */
     uint32_t tile_order_seed; /* nonzero: tiles are claimed in a seeded
                                  pseudo-random permutation (testing aid; the

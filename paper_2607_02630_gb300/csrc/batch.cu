@@ -541,6 +541,18 @@ static int fill_reqs(const aes_desc_t *descs, int n, int dev, const BatchShape &
     return sum.tiles > kMostTiles ? AES_ETOOBIG : AES_OK;
 }
 
+// Chunks of the largest T-table tile for a shape's tile_blocks.  A warp does a
+// tile in runs of at most 248 chunks (7936 blocks), so from half a run on a
+// tile is whole runs: one of 4096 blocks, the tuner's largest, was half a run
+// (4096 requests of 1 KiB to 8 MiB 4054 us, 4029 as a run), one of 8192 a run
+// and a short one.
+static uint32_t tile_chunks(int tile_blocks)
+{
+    constexpr uint32_t run = aestile::kRunChunks;
+    const uint32_t chunks = (uint32_t)tile_blocks / 32u;
+    return chunks <= run / 2 ? chunks : (chunks + run / 2) / run * run;
+}
+
 // Everything of a launch but its requests; returns the grid size.
 static int set_args(BatchArgs &p, const BatchSums &sum, const DeviceState &st, const BatchShape &s, uint32_t seed)
 {
@@ -549,7 +561,7 @@ static int set_args(BatchArgs &p, const BatchSums &sum, const DeviceState &st, c
     p.n = (uint32_t)sum.n;
     p.total_cost = sum.cost;
     const bool bs = s.variant == AES_VARIANT_BITSLICE;
-    p.tile_cost = !bs         ? (uint64_t)(s.tile_blocks / 32) * TtUnit::cost(10)
+    p.tile_cost = !bs         ? (uint64_t)tile_chunks(s.tile_blocks) * TtUnit::cost(10)
                   : sum.table ? BsUnitOf<true>::cost(10)
                               : (uint64_t)std::max(1, s.tile_blocks / 1024) * BsUnitOf<false>::cost(10);
     p.te0 = st.te0;

@@ -315,3 +315,22 @@ def test_payload_checks_pay_for_themselves(host, n, segment, stride):
         assert cost <= 2 * n + 60
         if segment >= n * (4 << 20):
             assert cost <= 60
+
+
+def test_tuned_tiles_reach_the_built_in_run(host):
+    """The tuner's largest tile (4096 blocks) is cut as the built-in shape's:
+    T-table tiles of more than half a run are whole runs of 7936 blocks, which
+    leave no short run behind; smaller ones and the bitsliced kernel's stay."""
+    ctx = host.ctx()
+    d = host.descs([(ctx, 0, P, P, 64 << 20)])
+
+    def tile(variant, tile_blocks):
+        rc, got = host.during(host.lib.aes_ctr_batch_ex, d, 1, None, _opts(variant, tile_blocks))
+        assert rc == A.AES_OK
+        return got[0].args[3]
+
+    run = tile(0, 0)
+    assert [tile(1, t) for t in (4096, 7936, 8192)] == [run] * 3
+    assert tile(1, 16384) == 2 * run
+    assert [tile(1, t) * 31 for t in (256, 1024, 2048, 3840)] == [run, 4 * run, 8 * run, 15 * run]
+    assert tile(2, 4096) == 2 * tile(2, 2048) == 4 * tile(2, 1024)

@@ -216,8 +216,9 @@ int aes_batch_plan_destroy(aes_batch_plan_t plan);
 /* --------------------------------------------------------------- autotuner */
 
 /* Time the candidate launch shapes of aes_ctr (per size bucket and key
- * size) and of the batch kernel on the current device, on scratch buffers
- * the call allocates and frees, and keep the fastest for AES_VARIANT_AUTO.
+ * size, as calls in a row) and of the batch kernel on the current device, on
+ * scratch buffers the call allocates and frees, and keep the fastest for
+ * AES_VARIANT_AUTO.
  * Synchronous; takes roughly a second.  `path` (may be NULL) names a JSON
  * file the table is written to. */
 int aes_autotune(const char *path);

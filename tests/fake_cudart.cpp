@@ -2,7 +2,8 @@
 // linked with the library's own objects, it shows on the CPU which launches an
 // entry point makes, on which device and stream and with which grid.  Two
 // devices; device memory is host memory; streams and events keep which launches
-// run behind which.  Not modelled: capture, time, and what kernels compute.
+// run behind which.  Not modelled: capture, time beyond given costs, and what
+// kernels compute.
 #include <cuda_runtime_api.h>
 
 #include <atomic>
@@ -34,10 +35,12 @@ struct Stream {
 struct Event {
     int device;
     std::set<int> before;
+    size_t at = 0;  // launches made before it
 };
 
 int g_device = 0, g_sms = 152;
 size_t g_segment = 1ull << 40;    // size of an allocation that payloads lie in
+std::map<int, std::pair<float, float>> g_costs;  // by CTA size: us of a launch after an event, of one in a row
 long g_queries = 0, g_lookups = 0;  // pointers asked about, allocations looked up
 std::atomic<long> g_news{0};
 std::vector<Launch> g_log;
@@ -60,6 +63,8 @@ void enqueue(Stream *st, const Launch &l)
 {
     g_before.push_back(st->before);
     st->before.insert((int)g_log.size());
+    if (st->before.size() > 256)  // enough to check, and a long row stays quick
+        st->before.erase(st->before.begin());
     g_log.push_back(l);
 }
 
@@ -121,6 +126,8 @@ void *fake_stream(int device)
 void fake_set_segment(size_t bytes) { g_segment = bytes; }
 long fake_queries() { return g_queries; }
 long fake_lookups() { return g_lookups; }
+void fake_clear_costs() { g_costs.clear(); }
+void fake_cost(int threads, float first, float next) { g_costs[threads] = {first, next}; }
 void fake_reset()
 {
     g_queries = g_lookups = 0;
@@ -248,11 +255,20 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s)
     if (!st || st->device != ((Event *)e)->device)
         return cudaErrorInvalidResourceHandle;
     ((Event *)e)->before = st->before;
+    ((Event *)e)->at = g_log.size();
     return cudaSuccess;
 }
 cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.f, cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t a, cudaEvent_t b)
+{
+    *ms = 0;
+    for (size_t i = ((Event *)a)->at; i < ((Event *)b)->at; ++i) {
+        const auto c = g_costs.find(g_log[i].block);
+        *ms += 1e-3f * (c == g_costs.end() ? 1.f : i == ((Event *)a)->at ? c->second.first : c->second.second);
+    }
+    return cudaSuccess;
+}
 cudaError_t cudaFuncSetAttribute(const void *fn, cudaFuncAttribute, int v)
 {
     if (v > 49152)

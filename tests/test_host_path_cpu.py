@@ -89,6 +89,7 @@ def host(built):
     for f in (lib.fake_news, lib.fake_queries, lib.fake_lookups):
         f.restype = ctypes.c_long
     lib.fake_set_segment.argtypes = [sz]
+    lib.fake_cost.argtypes = [ci, ctypes.c_float, ctypes.c_float]
     lib.fake_set_segment(1 << 40)
     lib.fake_set_device(0)
     lib.fake_reset()
@@ -334,3 +335,33 @@ def test_tuned_tiles_reach_the_built_in_run(host):
     assert tile(1, 16384) == 2 * run
     assert [tile(1, t) * 31 for t in (256, 1024, 2048, 3840)] == [run, 4 * run, 8 * run, 15 * run]
     assert tile(2, 4096) == 2 * tile(2, 2048) == 4 * tile(2, 1024)
+
+
+def test_single_call_tuner_times_calls_in_a_row(host):
+    """aes_autotune times each candidate as calls in a row, whose set-up
+    overlaps, and keeps the built-in shape where no other is faster by more
+    than the launches of one shape differ."""
+    def tuned(n):
+        s = A.LaunchShape()
+        assert host.lib.aes_tuned_shape(n, 256, ctypes.byref(s)) == A.AES_OK
+        return s.variant, s.threads
+
+    def costs(**us):  # CTA size -> (us of a launch after an event, of one in a row)
+        host.lib.fake_clear_costs()
+        for k, (first, next_) in us.items():
+            host.lib.fake_cost(int(k[1:]), first, next_)
+
+    sizes = (4096, 1 << 20, 4 << 20, 64 << 20)
+    costs(t128=(90, 90), t256=(5, 6), t512=(10, 4), t768=(9, 6), t1024=(9, 6))
+    assert host.lib.aes_autotune(None) == A.AES_OK
+    assert [tuned(n) for n in sizes] == [(1, 512)] * 4
+    costs(t128=(90, 90), t256=(9.9, 4.97), t512=(10, 5), t768=(9.9, 4.96), t1024=(9.95, 4.99))
+    assert host.lib.aes_autotune(None) == A.AES_OK
+    assert [tuned(n) for n in sizes] == [(1, 512)] * 4
+    costs(t128=(90, 90), t256=(9, 5), t512=(10, 5), t768=(9, 3), t1024=(9, 3.5))
+    assert host.lib.aes_autotune(None) == A.AES_OK
+    assert [tuned(n) for n in sizes] == [(1, 768)] * 4
+    costs(t128=(90, 90), t256=(9, 5), t512=(10, 3), t768=(9, 4), t1024=(9, 4))
+    assert host.lib.aes_autotune(None) == A.AES_OK
+    assert [tuned(n) for n in sizes] == [(1, 512)] * 4
+    host.lib.fake_clear_costs()

@@ -146,10 +146,13 @@ def captured_traffic(step_bytes: int):
     return int(per_byte * step_bytes)
 
 
-def ttable_lookups(w) -> int:
+def ttable_lookups(w, hoisted: bool = False) -> int:
     """Shared-memory lookups the T-table method needs for workload w: 16*Nr
     per 16-byte block, except that counter-mode caching replaces the 32
-    lookups of rounds 1-2 by 5 per block plus 27 per 256-block counter group."""
+    lookups of rounds 1-2 by 5 per block plus 27 per 256-block counter group;
+    hoisted: by constants that whole runs of groups share (the single-buffer
+    and batch kernels), of which none is counted."""
+    per_block, per_group = (0, 0) if hoisted else (5, 27)
     total = 0
     for n, b, iv in zip(w.lengths, w.bits, w.ivs):
         nb = (int(n) + 15) // 16
@@ -158,7 +161,7 @@ def ttable_lookups(w) -> int:
         nr = int(b) // 32 + 6
         v0 = int(iv[15])
         groups = ((v0 + nb - 1) >> 8) + 1
-        total += nb * (16 * nr - 27) + 27 * groups
+        total += nb * (16 * (nr - 2) + per_block) + per_group * groups
     return total
 
 
@@ -363,8 +366,7 @@ def sweep(args, rank, local):
                         roof = nsm * mhz * 1e6 * 64.0 / ops * 16 / 1e9
                         bound = "alu (LOP3, 64/clk/SM)"
                     else:
-                        groups = ((255 + nblocks - 1) >> 8) + 1
-                        lookups = nblocks * (16 * nr - 27) + 27 * groups
+                        lookups = nblocks * 16 * (nr - 2)  # rounds 3..Nr
                         roof = n / (lookups / (32.0 * nsm * mhz * 1e6)) / 1e9
                         bound = "shared-memory wavefronts (32 lookups/clk/SM)"
                     rows.append({"bytes": n, "bits": bits, "variant": name, "us": round(t * 1e6, 3),
@@ -529,7 +531,7 @@ def served(args, rank, local):
     try:
         pk, _ = peaks()
         nsm = torch.cuda.get_device_properties(dev).multi_processor_count
-        lookups_per_block = 16 * 14 - 27 + 27 / 256.0
+        lookups_per_block = 16 * (14 - 2)  # rounds 3..Nr
         roof = 32.0 * nsm * float(pk.get("sm_max_mhz", 2070.0)) * 1e6 / lookups_per_block * 16 / 1e9
     except Exception:
         pass
@@ -973,11 +975,11 @@ def batch_roofline(torch, dev, w, step_bytes, per_launch, tuned, rates):
                 f"clk per SM")
         kernel = "batch_bitslice_kernel"
     else:
-        work = ttable_lookups(w)
+        work = ttable_lookups(w, hoisted=True)
         per_clk = rates["lds32_per_clk_sm"] if measured else 32.0
-        what = (f"{work / 1e9:.3f} G T-table lookups per step (16*Nr per block, rounds 1-2 counter-cached: 5 per "
-                f"block + 27 per 256-block counter group) at {per_clk:.2f} conflict-free 32-bit shared-memory "
-                f"loads per clk per SM")
+        what = (f"{work / 1e9:.3f} G T-table lookups per step (16*(Nr-2) per block; rounds 1-2 come from "
+                f"constants that runs of blocks share, not counted) at {per_clk:.2f} conflict-free 32-bit "
+                f"shared-memory loads per clk per SM")
         kernel = "batch_ttable_kernel"
     src = ("measured on this GPU by aes_measure_peaks (clock64 per SM)" if measured
            else f"nominal rate: aes_measure_peaks failed ({rates.get('error')})")
@@ -1039,10 +1041,10 @@ def run_extras(A, torch, dev, stream, sh, w, ctxs, reqs, src, dst, step_bytes, a
     out["per_call"] = {"value": round(pc, 3), "unit": UNIT, "launches_per_step": len(reqs),
                        "how": "4096 aes_ctr calls on one stream, tuned shapes"}
     out["batch_noalloc"] = {"value": round(na, 3), "unit": UNIT, "calls_per_step": -(-len(reqs) // 1024),
-                            "how": "aes_ctr_batch_noalloc in calls of 1024 requests (descriptor copy + launch "
-                                   "each call, no device allocation)"}
+                            "how": "aes_ctr_batch_noalloc in calls of 1024 requests (each three launches with "
+                                   "the requests in kernel parameters, nothing allocated or copied)"}
     out["batch_one_shot"] = {"value": round(one_shot, 3), "unit": UNIT,
-                             "how": "aes_ctr_batch (descriptor upload + launch each call)"}
+                             "how": "aes_ctr_batch (table allocated from a pool and uploaded, one launch each call)"}
 
     # latency of a 1 MiB offload: per-call path with cudaEventQuery polling
     g = W.rng(W.SEED_BASE + 1)

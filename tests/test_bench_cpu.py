@@ -134,3 +134,22 @@ def test_batch_roofline_divides_by_the_measured_rate_of_the_picked_variant(bench
     nominal = bench.batch_roofline(_FakeTorch, 0, w, step, [1e-3], {"variant": 1}, {"error": "no GPU"})
     assert "nominal rate" in nominal["peak_basis"]
     assert nominal["peak"] == pytest.approx(2 * tt["peak"], rel=1e-3)  # 32 per clk instead of the fake 16
+
+
+def test_roofline_counts_only_lookups_no_launch_can_do_without(bench, monkeypatch):
+    """The batch roofline's peak is rounds 3..Nr of every block (16 lookups
+    each) at the device's rate: rounds 1-2 come from constants that whole runs
+    share, and counting any of them would set the peak too low."""
+    import types
+
+    w = W.batch_varlen(n=24, min_len=1, max_len=20000, seed=11, with_payload=False)
+    need = sum((int(n) + 15) // 16 * 16 * (int(b) // 32 + 4) for n, b in zip(w.lengths, w.bits))
+    assert bench.ttable_lookups(w, hoisted=True) == need < bench.ttable_lookups(w)
+    monkeypatch.setattr(bench, "peaks", lambda: ({"sm_max_mhz": 2000.0, "hbm_gbs": 6000.0}, "measured"))
+    monkeypatch.setattr(bench, "captured_traffic", lambda b: None)
+    torch = types.SimpleNamespace(cuda=types.SimpleNamespace(
+        get_device_properties=lambda d: types.SimpleNamespace(multi_processor_count=150)))
+    step = int(w.lengths.sum())
+    r = bench.batch_roofline(torch, 0, w, step, [1e-3], {"variant": 1}, {"lds32_per_clk_sm": 32.0})
+    assert r["peak"] == pytest.approx(step / (need / (32.0 * 150 * 2e9)) / 1e9, rel=1e-3)
+    assert "5 per block" not in r["peak_basis"] and "16*(Nr-2)" in r["peak_basis"]

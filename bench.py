@@ -975,18 +975,26 @@ def batch_roofline(torch, dev, w, step_bytes, per_launch, tuned, rates):
                 f"clk per SM")
         kernel = "batch_bitslice_kernel"
     else:
-        work = ttable_lookups(w, hoisted=True)
+        work = ttable_lookups(w)
+        needed = ttable_lookups(w, hoisted=True)
         per_clk = rates["lds32_per_clk_sm"] if measured else 32.0
-        what = (f"{work / 1e9:.3f} G T-table lookups per step (16*(Nr-2) per block; rounds 1-2 come from "
-                f"constants that runs of blocks share, not counted) at {per_clk:.2f} conflict-free 32-bit "
-                f"shared-memory loads per clk per SM")
+        what = (f"{work / 1e9:.3f} G T-table lookups per step (16*Nr per block with rounds 1-2 cached per "
+                f"256-block counter group: 5 per block + 27 per group; the kernel shares these over whole runs, "
+                f"so its own floor is roofline.rounds_3_to_nr) at {per_clk:.2f} conflict-free 32-bit shared-memory "
+                f"loads per clk per SM")
         kernel = "batch_ttable_kernel"
     src = ("measured on this GPU by aes_measure_peaks (clock64 per SM)" if measured
            else f"nominal rate: aes_measure_peaks failed ({rates.get('error')})")
     floor_s = work / (per_clk * nsm * sm_max_mhz * 1e6)
     roof_gbs = step_bytes / floor_s / 1e9
+    strict = None
+    if not bitsliced:
+        # what no launch can do without: 16 lookups in each of rounds 3..Nr
+        strict_gbs = roof_gbs * work / needed
+        strict = {"lookups": needed, "peak": round(strict_gbs, 2), "frac": round(achieved / strict_gbs, 4)}
     return {"bound": "alu", "achieved": round(achieved, 2), "peak": round(roof_gbs, 2), "unit": "GB/s",
             "frac": round(achieved / roof_gbs, 4),
+            "rounds_3_to_nr": strict,
             "traffic": captured_traffic(step_bytes) if not bitsliced else None,
             "peak_basis": f"{what} ({src}) x {nsm} SMs x {sm_max_mhz:.0f} MHz ({pk_kind} max clock)",
             "rates": {k: (round(v, 3) if isinstance(v, float) else v) for k, v in rates.items()},

@@ -137,9 +137,10 @@ def test_batch_roofline_divides_by_the_measured_rate_of_the_picked_variant(bench
 
 
 def test_roofline_counts_only_lookups_no_launch_can_do_without(bench, monkeypatch):
-    """The batch roofline's peak is rounds 3..Nr of every block (16 lookups
-    each) at the device's rate: rounds 1-2 come from constants that whole runs
-    share, and counting any of them would set the peak too low."""
+    """Beside the peak by constants per counter group, the batch roofline
+    gives the one by rounds 3..Nr of every block (16 lookups each): the kernel
+    shares what rounds 1-2 need over whole runs, so counting any of it sets
+    the peak too low."""
     import types
 
     w = W.batch_varlen(n=24, min_len=1, max_len=20000, seed=11, with_payload=False)
@@ -151,5 +152,8 @@ def test_roofline_counts_only_lookups_no_launch_can_do_without(bench, monkeypatc
         get_device_properties=lambda d: types.SimpleNamespace(multi_processor_count=150)))
     step = int(w.lengths.sum())
     r = bench.batch_roofline(torch, 0, w, step, [1e-3], {"variant": 1}, {"lds32_per_clk_sm": 32.0})
-    assert r["peak"] == pytest.approx(step / (need / (32.0 * 150 * 2e9)) / 1e9, rel=1e-3)
-    assert "5 per block" not in r["peak_basis"] and "16*(Nr-2)" in r["peak_basis"]
+    strict = r["rounds_3_to_nr"]
+    assert strict["lookups"] == need and strict["peak"] > r["peak"]
+    assert strict["peak"] == pytest.approx(step / (need / (32.0 * 150 * 2e9)) / 1e9, rel=1e-3)
+    assert strict["frac"] == pytest.approx(step / 1e-3 / 1e9 / strict["peak"], rel=1e-2, abs=1e-4)
+    assert "roofline.rounds_3_to_nr" in r["peak_basis"]

@@ -343,7 +343,7 @@ def test_batch_checks_every_payload_pointer(cuda, aes, n):
     cuda.cuda.synchronize()
 
 
-def test_plan_launches_are_ordered_across_streams(cuda, aes):
+def test_plan_launches_are_ordered_across_streams(cuda, aes, ncpu):
     """Launches of one plan on different streams run one after the other: a
     plan that encrypts in place, launched an even number of times from two
     streams that wait for nothing, gives its input back."""
@@ -364,7 +364,7 @@ def test_plan_launches_are_ordered_across_streams(cuda, aes):
     cuda.cuda.synchronize()
     out = to_host(src)
     for key, b, iv, o, k in meta:
-        np.testing.assert_array_equal(out[o: o + k], oracle.ctr(key, b, iv, payload[o: o + k]))
+        np.testing.assert_array_equal(out[o: o + k], oracle.ctr_mt(key, b, iv, payload[o: o + k], ncpu))
     plan.close()
 
 
@@ -406,3 +406,53 @@ def test_claims_from_the_whole_line(cuda, aes, ncpu):
             cuda.cuda.synchronize()
             assert np.array_equal(out.cpu().numpy(), want), (pinned, opts)
             plan.close()
+
+
+@pytest.mark.parametrize("n", [6, 70, 600, 1100])
+@pytest.mark.parametrize("threads", [0, 1024])
+def test_pinned_payloads_in_every_kernel(cuda, aes, ncpu, n, threads, tmp_path):
+    """Pinned payloads (chunk pairs in address order) through every kernel
+    that takes them: requests in parameters (up to 64, up to 500, several
+    launches) and in a device table, keys in registers and in shared memory;
+    all key sizes, IV low bytes on both sides of a chunk edge, tails, odd
+    chunk counts (a half-empty last pair), a device payload among them."""
+    g = W.rng(5900 + n + threads)
+    sizes = [1, 16, 511, 512, 513, 1024 + 16, 1536, 1536 + 7, 4096 + 5, 40_000 + 3]
+    lengths = [int(sizes[i % len(sizes)]) for i in range(n)]
+    lengths[n // 2] = 300_000 + 9
+    bits = [(128, 192, 256)[int(x)] for x in g.integers(0, 3, n)]
+    reqs, meta, payload, src, dst = make_requests(cuda, aes, g, lengths, bits)
+    cuda.cuda.synchronize()
+    hsrc, hdst = src.cpu().pin_memory(), dst.cpu().pin_memory()
+    lows = [0x00, 0x1F, 0x20, 0xE1, 0xFF]
+    want = np.full(payload.size, 0xA5, np.uint8)
+    r = []
+    for i, ((c, iv, s, d, k), (key, b, _, o, _)) in enumerate(zip(reqs, meta)):
+        iv = iv[:15] + bytes([lows[i % 5]])
+        want[o: o + k] = oracle.ctr(key, b, np.frombuffer(iv, np.uint8), payload[o: o + k])
+        r.append((c, iv, s, d, k) if i == 1 else (c, iv, hsrc.data_ptr() + o, hdst.data_ptr() + o, k))
+    o, k = meta[1][3], meta[1][4]
+
+    def check(call):
+        hdst.fill_(0xA5)
+        dst.fill_(0xA5)
+        cuda.cuda.synchronize()
+        call()
+        cuda.cuda.synchronize()
+        out = hdst.numpy().copy()
+        out[o: o + k] = to_host(dst)[o: o + k]
+        np.testing.assert_array_equal(out, want)
+
+    check(lambda: aes.batch(r, threads=threads))
+    plan = aes.BatchPlan(r, threads=threads)
+    check(plan.launch)
+    plan.close()
+    if n <= 1024:
+        d = aes.batch_tuned_shape()
+        default = (d["variant"], d["threads"], d["tile_blocks"], d["blocks_per_thread"])
+        try:
+            if threads:
+                set_batch_shape(cuda, aes, tmp_path / "shape.json", (1, threads, 2048, 1))
+            check(lambda: aes.batch_noalloc_status(r))
+        finally:
+            set_batch_shape(cuda, aes, tmp_path / "shape.json", default)

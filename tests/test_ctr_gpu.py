@@ -298,3 +298,83 @@ def test_dependent_launches_in_a_row(cuda, aes, n):
             b.zero_()
     cuda.cuda.synchronize()
     np.testing.assert_array_equal(to_host(a), to_host(src))
+
+
+@pytest.mark.parametrize("n", [4096, 1 << 20, (5 << 20) + 3])
+def test_overlapped_launches_wait_for_events_of_other_streams(cuda, aes, ncpu, n):
+    """A launch whose set-up may overlap the one before it on its stream still
+    waits for an event that its stream waits for: two streams hand a payload
+    back and forth, each launch reading what the other stream wrote, with a
+    launch of the same stream directly before the wait."""
+    g = W.rng(3900 + n % 1000)
+    ctx = aes.Context(W.random_bytes(g, 16).tobytes(), 128)
+    ivs = [W.random_bytes(g, 16).tobytes() for _ in range(12)]
+    src = to_dev(cuda, W.random_bytes(g, n))
+    big = cuda.zeros(64 << 20, dtype=cuda.uint8, device="cuda")
+    bufs = [src.clone() for _ in range(13)]
+    side = cuda.zeros(4096, dtype=cuda.uint8, device="cuda")
+    streams = [cuda.cuda.Stream(), cuda.cuda.Stream()]
+    cuda.cuda.synchronize()
+    for i in range(12):
+        s, other = streams[i & 1], streams[1 - (i & 1)]
+        aes.ctr(ctx, ivs[0], side, side, 4096, stream=s)            # a launch the next could overlap with
+        with cuda.cuda.stream(other):
+            big.add_(1)                                             # keeps the other stream busy a while
+        aes.ctr(ctx, ivs[i], bufs[i], bufs[i + 1], n, stream=other)
+        done = cuda.cuda.Event()
+        done.record(other)
+        s.wait_event(done)
+        aes.ctr(ctx, ivs[i], bufs[i + 1], bufs[i + 1], n, stream=s)  # undoes it, if it has been written
+        aes.ctr(ctx, ivs[i], bufs[i + 1], bufs[i + 1], n, stream=s)  # and redoes it
+        done2 = cuda.cuda.Event()
+        done2.record(s)
+        streams[0].wait_event(done2)
+        streams[1].wait_event(done2)
+    cuda.cuda.synchronize()
+    want = to_host(src).copy()
+    key = np.frombuffer(ctx.round_keys()[:16], np.uint8)
+    for i in range(12):
+        want = oracle.ctr_mt(key, 128, np.frombuffer(ivs[i], np.uint8), want, ncpu)
+        np.testing.assert_array_equal(to_host(bufs[i + 1]), want, err_msg=f"step {i}")
+
+
+def test_overlapped_launches_from_two_threads(cuda, aes):
+    """Two threads, a stream and a payload each, and both on one plan: chains
+    of dependent calls give each thread its own bytes."""
+    import threading
+
+    g = W.rng(3950)
+    n = (1 << 20) + 5
+    ctxs = [aes.Context(W.random_bytes(g, b // 8).tobytes(), b) for b in (128, 256)]
+    iv = W.random_bytes(g, 16).tobytes()
+    srcs = [to_dev(cuda, W.random_bytes(g, n)) for _ in ctxs]
+    bufs = [s.clone() for s in srcs]
+    shared = srcs[0].clone()
+    plan = aes.BatchPlan([(ctxs[0], iv, shared.data_ptr(), shared.data_ptr(), n)])
+    cuda.cuda.synchronize()
+    errors = []
+
+    def work(k):
+        try:
+            s = cuda.cuda.Stream()
+            for _ in range(60):
+                aes.ctr(ctxs[k], iv, bufs[k], bufs[k], n, stream=s)
+                aes.batch([(ctxs[k], iv, bufs[k].data_ptr(), bufs[k].data_ptr(), n)], stream=s)
+                plan.launch(s)
+            aes.ctr_sync(ctxs[k], iv, bufs[k], bufs[k], n, stream=s)
+        except Exception as e:  # reported by the test's own thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    cuda.cuda.synchronize()
+    assert not errors
+    for k, bits in enumerate((128, 256)):
+        key = np.frombuffer(ctxs[k].round_keys()[: bits // 8], np.uint8)
+        np.testing.assert_array_equal(to_host(bufs[k]), oracle.ctr(key, bits, np.frombuffer(iv, np.uint8),
+                                                                   to_host(srcs[k])))
+    np.testing.assert_array_equal(to_host(shared), to_host(srcs[0]))  # an even number of in-place launches
+    plan.close()

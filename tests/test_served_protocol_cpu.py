@@ -170,3 +170,30 @@ def test_ring_placement_spreads_a_lease_over_partitions(tmp_path):
                     os.path.join(HERE, "ring_placement_test.cpp"), "-o", exe], check=True)
     r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0 and r.stdout.startswith("OK"), r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("mode", [0, 1], ids=["global_cursor", "per_request"])
+@pytest.mark.parametrize("case", [(4, 32, 3000, 0, 2000, 41), (12, 64, 3000, 0, 300, 42), (3, 1, 800, 0, 2000, 43)],
+                         ids=["wide", "idle", "one_slot"])
+def test_every_tile_level_is_processed_once(tmp_path_factory, mode, case):
+    """The same run with every tile level in turn in the requests' flags, as
+    offload_submit sets it by the requests in flight: fewer, larger tiles."""
+    src = open(os.path.join(HERE, "served_protocol_sim.cpp")).read()
+    for plain, leveled in (  # request i at level i & 3, its tiles counted for that level
+            ("qe.flags = r.emulated ? (uint16_t)kFlagEmulated : 0;",
+             "qe.flags = (uint16_t)((r.emulated ? kFlagEmulated : 0u) | ((uint32_t)i & 3u) << kFlagLevelShift);"),
+            ("tile_count(uint64_t len, uint64_t iv_lo) const", "tile_count(uint64_t len, uint64_t iv_lo, uint32_t level) const"),
+            ("(uint64_t)tb * 512 < nb", "(uint64_t)tb * (512u >> level) < nb"),
+            ("tile_count(r.len, r.iv_lo)", "tile_count(r.len, r.iv_lo, (uint32_t)i & 3u)")):
+        assert src.count(plain) == 1, plain
+        src = src.replace(plain, leveled)
+    work = tmp_path_factory.mktemp("levels")
+    (work / "sim.cpp").write_text(src)
+    nvcc = B._nvcc()
+    cuda_inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-pthread", "-Wno-unknown-pragmas", "-fsanitize=undefined",
+                    "-fno-sanitize-recover=undefined", "-I", B.INCLUDE, "-I", B.CSRC, "-I", cuda_inc, "-I", HERE,
+                    str(work / "sim.cpp"), "-o", str(work / "sim")], check=True)
+    r = subprocess.run([str(work / "sim"), str(mode)] + [str(x) for x in case], capture_output=True, text=True,
+                       timeout=240)
+    assert r.returncode == 0 and r.stdout.startswith("OK"), r.stdout + r.stderr

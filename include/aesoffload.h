@@ -145,7 +145,7 @@ typedef struct {
     size_t len;
 } aes_desc_t;
 
-/* Options of the persistent batch kernel (all-zero = tuned defaults). */
+/* Options of the batch kernel (all-zero = tuned defaults). */
 typedef struct {
     int variant;        /* AES_VARIANT_* (AUTO: the tuned variant, T-table
                            until aes_batch_autotune picks otherwise) */

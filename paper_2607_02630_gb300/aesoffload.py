@@ -372,7 +372,7 @@ def batch_noalloc_status(requests, stream=None) -> int:
 
 
 def batch(requests, stream=None, **opts) -> None:
-    """One persistent launch over requests = [(ctx, iv, src, dst, nbytes), ...]."""
+    """aes_ctr_batch_ex over requests = [(ctx, iv, src, dst, nbytes), ...]."""
     _check(batch_status(requests, stream, **opts), "aes_ctr_batch")
 
 

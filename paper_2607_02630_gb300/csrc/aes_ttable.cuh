@@ -101,15 +101,15 @@ struct RkConst {
     }
 };
 
-// Round keys staged in shared memory (per-request keys of the batch and
-// served kernels); one broadcast 16-byte load per round.
+// Round keys staged in shared memory (per-request keys in batch CTAs of more
+// than 512 threads); one broadcast 16-byte load per round.
 struct RkShared {
     const uint4 *w;
     __device__ __forceinline__ uint4 get(int r) const { return w[r]; }
 };
 
 // Round keys held in registers -- the batch kernel's warps, one request at a
-// time.  The schedule is read once per tile (NR + 1 uniform 16-byte loads);
+// time.  The schedule is read once per run (NR + 1 uniform 16-byte loads);
 // indices are compile-time after unrolling, so every round's key is four
 // register operands and costs no shared-memory wavefront.  The price is
 // 4 * (NR + 1) registers a thread, which the 512-thread batch CTA can pay.

@@ -127,7 +127,9 @@ struct BatchParams<0> : BatchArgs {
 // Requests that fit the kernel's parameters (32764 bytes at most): a batch of
 // up to so many needs no descriptor table in device memory, hence no
 // allocation, no copy and no wait for one.  The small size keeps the launch
-// of a small batch from copying 32 KB.
+// of a small batch from copying 32 KB: calls of 1000-byte requests in a row,
+// with it and with the large size, 1 request 3.8 and 4.3 us, 64 7.8 and 7.9
+// (enqueued in 4.7-4.9 and 5.1-5.5); 65 requests, in the large size, 8.7.
 constexpr int kFewInParams = 64;
 constexpr int kMostInParams = 500;
 static_assert(sizeof(BatchParams<kMostInParams>) <= 32764, "kernel parameters");
@@ -243,14 +245,17 @@ __device__ __forceinline__ bool next_run(const BatchArgs &p, const BatchReq *req
 // The T-table batch kernel, bound by shared-memory wavefronts (95 % of the
 // pipe busy on a 256 MiB AES-128 request).  Measured as plans against the
 // kernel with a tile map, a device counter and two blocks per lane: 4096
-// requests of 1 KiB to 8 MiB (3.66 GB) 4396 -> 4043 us, 512 of them 638 ->
-// 565, 256 of 4 KiB to 1 MiB 111 -> 58, 64 of 1 to 16 KiB 37 -> 5.4 (one warp
+// requests of 1 KiB to 8 MiB (3.66 GB) 4396 -> 4029 us, 512 of them 638 ->
+// 562, 256 of 4 KiB to 1 MiB 111 -> 58, 64 of 1 to 16 KiB 37 -> 5.1 (one warp
 // used to take up to 8 groups of a short request in turn).  Other CTA sizes
 // on the 4096: 1024 threads (keys in shared memory) 4491 us, 256 threads
 // 5148; 384 threads with up to 168 registers were 2 % faster on AES-256
 // alone and 3 % slower on AES-128.  MAXT: largest CTA it is launched with;
 // RK_REGS: round keys in registers (else in the warp's slice of shared
-// memory); HOST: some payload lies in pinned host memory.
+// memory); HOST: some payload lies in pinned host memory, and every request
+// of the launch takes that walk (256 device requests of 4 KiB to 1 MiB 62.7
+// us, one of them in pinned memory 65.6, or 63.0 with the device's walk for
+// all; one in 16 62.7 and 59.6); WHOLE: claims from the whole line.
 template <int MAXT, bool RK_REGS, int CAP, bool HOST, bool WHOLE>
 __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_constant__ BatchParams<CAP> p)
 {

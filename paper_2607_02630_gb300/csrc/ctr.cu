@@ -50,7 +50,7 @@ constexpr size_t kCtrSmem = aestt::kTableBytesOf<TABLES> + kGroupsPerPass * size
 // 13.4 -> 10.7 us, 256 MiB 263 -> 240 us (1.12 TB/s; 137 wavefronts per
 // chunk at the measured rate and 2070 MHz are 228 us).  Back to back on a
 // stream, with the set-up overlapped (launch_overlapped): 1 MiB 3.5 us, 8 MiB
-// 10.2 us.
+// 10.2 us (9.4 with two tables).
 //
 // With two tables (64 KiB) and 512 threads, two CTAs fit an SM, so the next
 // launch's CTAs set up beside the running ones instead of after them.
@@ -143,9 +143,14 @@ cudaError_t set_tt_attr()
 // Two tables from 2 to 16 MiB, where a launch's set-up counts and the extra
 // logic operations hide behind the lookups; four below (one chunk per warp:
 // the longer chain of a round counts) and above.  Launches in a row, four and
-// two tables: 1 MiB AES-128 3.24 and 3.26 us, AES-256 3.70 and 4.18; 4 MiB
-// 6.30 and 5.65, 8.03 and 7.39; 8 MiB 9.9 and 9.4, 13.2 and 12.75; 32 MiB
-// 32.4 and 32.5; 256 MiB 241.9 and 245.3, 348 and 352.
+// two tables, AES-128 and AES-256:
+//   1 MiB     3.26 3.29 us   3.72 4.16 us      8 MiB    9.9  9.4    13.2  12.75
+//   1.25 MiB  3.67 3.88      4.34 3.74         16 MiB   17.4 17.1   24.0  23.7
+//   1.5 MiB   3.87 3.14      4.57 3.84         20 MiB   20.94 20.82  29.3 29.1
+//   2 MiB     4.18 3.47      5.01 4.32         32 MiB   32.0 32.1   45.3  45.3
+//   4 MiB     6.30 5.65      8.03 7.39         256 MiB  241.9 245.3  348  352
+// The upper line is where they meet; the lower one is on the safe side (1.25
+// MiB goes either way, 1.5 MiB would gain).
 bool two_tables(uint64_t len, int threads) { return len >= (2u << 20) && len <= (16u << 20) && threads == 512; }
 
 template <int NR>

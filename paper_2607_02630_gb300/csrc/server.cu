@@ -311,8 +311,12 @@ void release_slot(offload_server_s *s, uint32_t d)
 // the tiles, not the lookups, bound the server.  From 16 requests on half as
 // many tiles each still fill the resident CTAs' ~2200 worker warps twice
 // over, from 32 a quarter, from 64 an eighth (requests of 1 MiB).  256
-// requests of the served mix in a burst: 949 -> 770 us; one in flight as
-// before (17.8 and 17.7 us).
+// requests of the served mix in a burst from Python: 949 -> 770 us; one in
+// flight as before (17.8 and 17.7 us).  Bursts from one native submitter with
+// the levels below, with level 0, 1, 2 and 3 for all of their requests: 15 of
+// 1 MiB 96 us, 96, 90, 104, 136; 31 145, 157, 137, 151, 192; 63 244, 278, 227,
+// 219, 267; 256 725, 995, 760, 672, 791; 256 of the mix 852, 1030, 886, 840,
+// 865.  A burst's first requests are cut for few in flight, whatever follows.
 static uint32_t tile_level(uint32_t in_flight)
 {
     return in_flight >= 64 ? 3u : in_flight >= 32 ? 2u : in_flight >= 16 ? 1u : 0u;

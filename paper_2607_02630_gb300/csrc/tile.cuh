@@ -94,8 +94,9 @@ __device__ __forceinline__ void xor_run(const uint4 *__restrict__ in, uint4 *__r
 // The same run for payloads in pinned host memory, where the link and the
 // host's memory bound the kernel: chunks in address order, two at a time,
 // loaded together and stored together, so that each warp moves 1 KiB bursts
-// (1024 requests of 1 KiB to 8 MiB in pinned memory, 0.9 GB each way: 139 GB/s
-// each way, 134 with xor_run, 168 being the link's measured most).  The lane's
+// (1024 requests of 1 KiB to 8 MiB in pinned memory, 0.9 GB each way: 144 GB/s
+// each way, 168 being the link's measured most; claimed by fixed pieces 141,
+// and 134 with xor_run).  The lane's
 // part of round 2 is derived for each chunk; the lookups do not bound here.
 template <int NR, class RK>
 __device__ __forceinline__ void xor_run_host(const uint4 *__restrict__ in, uint4 *__restrict__ out, uint64_t len,

@@ -109,19 +109,28 @@ struct BatchArgs {
     uint64_t total_cost;
     uint64_t tile_cost;  // largest tile
     const uint32_t *te0;
-    // Kernels that claim from the whole line (CAP == 0): this launch's counter,
-    // zero when it starts, and the next one's, which it clears.
-    unsigned long long *claimed, *cleared;
     TileOrder order;
 };
 template <int CAP>
 struct BatchParams : BatchArgs {
     BatchReq in_params[CAP];
     __device__ __forceinline__ const BatchReq *requests() const { return in_params; }
+    __device__ __forceinline__ unsigned long long *whole_line() const { return nullptr; }
+    __device__ __forceinline__ void clear_next() const {}
 };
+static_assert(sizeof(BatchArgs) == 64, "requests in parameters start on a 64-byte line");
 template <>
 struct BatchParams<0> : BatchArgs {
+    // Kernels that claim from the whole line: this launch's counter, zero when
+    // it starts, and the next one's, which it clears.
+    unsigned long long *claimed, *cleared;
     __device__ __forceinline__ const BatchReq *requests() const { return reqs; }
+    __device__ __forceinline__ unsigned long long *whole_line() const { return claimed; }
+    __device__ __forceinline__ void clear_next() const
+    {
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            *cleared = 0;
+    }
 };
 
 // Requests that fit the kernel's parameters (32764 bytes at most): a batch of
@@ -172,10 +181,11 @@ struct WarpState {
 
 // The warp's next run: n > 0 chunks from chunk k0 on of request rq (every
 // lane gets the same), or false when the CTA's piece (WHOLE: the line) is done.
-// s_pos: the counter of the CTA's piece; st: this warp's state; both zeroed
-// before the CTA's last barrier.
+// pos: the piece's counter in shared memory, the line's in device memory; st:
+// this warp's state, which like the piece's counter is zeroed before the CTA's
+// last barrier.
 template <class UNIT, bool WHOLE>
-__device__ __forceinline__ bool next_run(const BatchArgs &p, const BatchReq *reqs, unsigned long long *s_pos,
+__device__ __forceinline__ bool next_run(const BatchArgs &p, const BatchReq *reqs, unsigned long long *pos,
                                          WarpState *st, BatchReq &rq, uint64_t &k0, uint32_t &n)
 {
     const uint32_t lane = threadIdx.x & 31u;
@@ -192,7 +202,6 @@ __device__ __forceinline__ bool next_run(const BatchArgs &p, const BatchReq *req
             const uint64_t size = WHOLE ? units : q + (blockIdx.x < r ? 1 : 0);
             unsigned long long at = 0, take = 1;
             if (lane == 0) {
-                unsigned long long *pos = WHOLE ? p.claimed : s_pos;
                 if (!p.order.tiles && !UNIT::kEven) {
                     const unsigned long long cur = *(volatile unsigned long long *)pos;
                     const uint32_t warps = (blockDim.x >> 5) * (WHOLE ? gridDim.x : 1u);
@@ -272,8 +281,8 @@ __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_cons
     aestt::fill_tables(smem, p.te0);
     __syncthreads();
     aesdev::wait_for_previous_launch();
-    if (WHOLE && blockIdx.x == 0 && threadIdx.x == 0)
-        *p.cleared = 0;
+    if constexpr (WHOLE)
+        p.clear_next();
     const aestt::Lanes ln(smem);
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     uint4 *w_group = s_group[warp];
@@ -298,7 +307,7 @@ __global__ void __launch_bounds__(MAXT, 1) batch_ttable_kernel(const __grid_cons
     BatchReq rq;
     uint64_t k0;
     uint32_t n;
-    while (next_run<TtUnit, WHOLE>(p, p.requests(), &s_pos, &s_state[warp], rq, k0, n)) {
+    while (next_run<TtUnit, WHOLE>(p, p.requests(), WHOLE ? p.whole_line() : &s_pos, &s_state[warp], rq, k0, n)) {
         switch (rq.nr) {
         case 10: xor_with(rq, k0, n, std::integral_constant<int, 10>()); break;
         case 12: xor_with(rq, k0, n, std::integral_constant<int, 12>()); break;
@@ -324,15 +333,15 @@ __global__ void __launch_bounds__(kBsThreads) batch_bitslice_kernel(const __grid
         s_state[threadIdx.x] = WarpState{0, 0, 0, 0};
     __syncthreads();
     aesdev::wait_for_previous_launch();
-    if (CAP == 0 && blockIdx.x == 0 && threadIdx.x == 0)
-        *p.cleared = 0;
+    p.clear_next();
     const uint32_t lane = threadIdx.x & 31u;
     uint32_t *mask = s_mask[threadIdx.x >> 5];
     const uint4 *cur = nullptr;  // schedule whose masks are in `mask`
     BatchReq rq;
     uint64_t k0;
     uint32_t n;
-    while (next_run<BsUnitOf<CAP == 0>, CAP == 0>(p, p.requests(), &s_pos, &s_state[threadIdx.x >> 5], rq, k0, n)) {
+    while (next_run<BsUnitOf<CAP == 0>, CAP == 0>(p, p.requests(), CAP == 0 ? p.whole_line() : &s_pos,
+                                               &s_state[threadIdx.x >> 5], rq, k0, n)) {
         const uint64_t v0 = rq.iv_lo & 255u, nb = (rq.len + 15) >> 4;
         const uint64_t first = k0 << 5 > v0 ? (k0 << 5) - v0 : 0;
         const uint64_t end = ((k0 + n) << 5) - v0, last = end < nb ? end : nb;
@@ -562,7 +571,6 @@ static uint32_t tile_chunks(int tile_blocks)
 static int set_args(BatchArgs &p, const BatchSums &sum, const DeviceState &st, const BatchShape &s, uint32_t seed)
 {
     p.reqs = nullptr;
-    p.claimed = p.cleared = nullptr;
     p.n = (uint32_t)sum.n;
     p.total_cost = sum.cost;
     const bool bs = s.variant == AES_VARIANT_BITSLICE;

@@ -24,7 +24,7 @@ struct Launch {
     int grid, block;
     int programmatic;  // 1: may start before the stream's previous kernel has ended
     uint64_t stream;
-    char args[64];     // the first bytes of the first parameter
+    char args[80];     // the first bytes of the first parameter
     char name[128];
 };
 

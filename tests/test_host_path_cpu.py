@@ -16,10 +16,10 @@ P = 0x7F00_0000_0000  # a payload address (nothing reads it)
 
 class Launch(ctypes.Structure):
     _fields_ = [("device", ctypes.c_int), ("grid", ctypes.c_int), ("block", ctypes.c_int),
-                ("programmatic", ctypes.c_int), ("stream", ctypes.c_uint64), ("args", ctypes.c_uint64 * 8),
+                ("programmatic", ctypes.c_int), ("stream", ctypes.c_uint64), ("args", ctypes.c_uint64 * 10),
                 ("name", ctypes.c_char * 128)]
 
-    def raw(self, n=64):
+    def raw(self, n=80):
         b = bytes(self.args)
         if b"BatchParams" in self.name:
             b = b[:12] + bytes(4) + b[16:]  # padding behind the request count
@@ -284,7 +284,7 @@ def test_whole_line_counters_take_turns(host):
         host.lib.fake_reset()
         for _ in range(3):
             assert host.lib.aes_batch_plan_launch(plan, None) == A.AES_OK
-        pairs = [tuple(l.args[5:7]) for l in host.launches()]  # claimed, cleared
+        pairs = [tuple(l.args[8:10]) for l in host.launches()]  # claimed, cleared
         if whole:
             a, b = pairs[0]
             assert a and b and a != b and pairs == [(a, b), (b, a), (a, b)]
